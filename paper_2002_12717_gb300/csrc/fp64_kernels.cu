@@ -748,6 +748,7 @@ void launch_zgemm(dim3 grid, cudaStream_t st, const ZGemm &g, int reduce, int pe
 
 void zgemm(Launcher &L, const ZGemm &g) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
+  if (fp64_tc_zgemm(L, g)) return;
   dim3 grid((g.N + GBN - 1) / GBN, (g.M + GBM - 1) / GBM, std::min(g.batch, 65535));
   L.before("fp64_zgemm");
   launch_zgemm(grid, L.stream, g, 0, 1, nullptr, 1, g.K);
@@ -756,6 +757,7 @@ void zgemm(Launcher &L, const ZGemm &g) {
 
 void zgemm_reduce(Launcher &L, const ZGemm &g, cplx *partial, int splits) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
+  if (fp64_tc_zgemm_reduce(L, g)) return;
   // cut K as well when the batch alone gives fewer units than splits
   const int kblocks = (g.K + GBK - 1) / GBK;
   const int kparts = std::max(1, std::min(kblocks, (splits + g.batch - 1) / g.batch));

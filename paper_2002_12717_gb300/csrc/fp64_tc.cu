@@ -1,0 +1,864 @@
+// FP64 matrix products of the FP64 form on the tensor cores.
+//
+// GB300 issues about two FP64 multiply-adds per SM and clock (1.2 TFLOP/s for the chip), so a
+// contraction of the FP64 form is bound by the FP64 pipe 50 to 100 times above the time its
+// bytes take.  Here each real operand is cut into seven signed 8-bit digits, the digit
+// products run as BF16 MMAs on tcgen05 and are summed as integers (the error-free
+// splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 95 (2012)):
+//
+//   x = 2^(e - 1077) sum_s d_s 256^(6 - s),  |d_s| <= 128,
+//
+// with one exponent e per row of A (column of B) and segment of the contraction (at most 256 terms), the one
+// of its largest entry there, so that 56 bits below that entry's leading bit are kept: every entry
+// within a factor 4 of the largest is held exactly.  Digits are small integers, exact in BF16.  The products
+// d_s d'_t of one order o = s + t have one common weight 256^-o and a TMEM accumulator of their own; orders
+// 0..7 are formed (34 MMAs per 16-element K step).  The dropped ones weigh 2^-64 of the largest product: with
+// seven orders (28 MMAs) they weighed 2^-56, and rows whose largest entry is ten times the typical one
+// (w and n of a general basis) lost 3e-15 of the result, more than FP64 multiply-adds do.  An FP32
+// accumulator is exact while its sum of integers stays below 2^24: o + 1 products of at most 2^14 over 256
+// terms, so the orders 0..3 never round, and a rounding of the higher ones weighs below 2^-56.  At the end of
+// a segment the accumulators go into 64-bit integers (hi: orders 0..3, lo: orders 4..7), whose sum is
+// rounded once to FP64; the segments of a long contraction are added in FP64.  (One exponent for a whole row
+// of 32768 terms lost a factor ten against FP64 multiply-adds in the gradients of sparse cotangents.)  Against FP64
+// multiply-adds, which round after every term, the result is closer to the exact sum: right-hand sides
+// at nb = 16, 20, 24 are 2.2e-16, 2.4e-16, 3.7e-16 off (2-norm, extended precision) instead of 3.3e-16, 4.7e-16,
+// 6.4e-16.
+//
+// All conversions run on the integer pipe: FP64 instructions in the prologue or epilogue would
+// cost as much as the MMAs (two per SM and clock).  A row or column that holds an Inf or a NaN has
+// no digits; its outputs are recomputed with FP64 multiply-adds in the epilogue, which gives
+// the values the CUDA-core kernel gives.
+#include "g1g2_internal.h"
+#include "tc_ptx.cuh"
+
+#include <algorithm>
+#include <new>
+
+namespace g1g2 {
+
+namespace {
+
+using namespace tc;
+
+constexpr int kDig = 7;                    // digits per real operand
+constexpr int kOrd = 8;                    // orders of digit products
+constexpr int kTM = 128;                   // rows of A per tile (TMEM lanes)
+constexpr int kTNMax = 128;                // real columns per tile, at most
+constexpr int kKB = 16;                    // K elements per block: one MMA step, 32-byte rows
+constexpr int kSeg = 16;                   // K blocks of a segment (256 terms)
+constexpr uint32_t kADig = kTM * 32;       // one digit plane of an A block: 4 KB
+constexpr uint32_t kABlk = kDig * kADig;   // 28 KB
+constexpr uint32_t kStageBytes = 2 * kABlk;   // A and B (at most 128 columns) blocks
+constexpr int kStages = 3;
+constexpr int kEpiWarps = 16;
+constexpr int kThreads = 64 + 32 * kEpiWarps;   // loader warp, MMA warp, epilogue warps
+constexpr int kStgPitch = 5;               // complex per staged row (4 used)
+constexpr uint32_t kStgWarp = 32 * kStgPitch * 16;
+constexpr size_t kSmem = 1024 + kStages * kStageBytes + kEpiWarps * kStgWarp + 256;
+
+constexpr int kNonFinite = 2047;           // row exponent of a row with an Inf or a NaN
+
+// ---------------------------------------------------------------------------
+// Digits
+// ---------------------------------------------------------------------------
+// One strided complex operand: row r = (b, x) with x < X, element k at p[b sb + x sx + (k / kin) kout + (k % kin) sk].
+struct Operand {
+  const cplx *p;
+  long long sb, sx, sk, kout;
+  int X, kin;
+  int rows, K;
+  int conj;
+};
+__device__ __forceinline__ long long row_offset(const Operand &o, int r) {
+  const int b = r / o.X;
+  return (long long)b * o.sb + (long long)(r - b * o.X) * o.sx;
+}
+__device__ __forceinline__ long long k_offset(const Operand &o, int k) {
+  const int b = k / o.kin;
+  return (long long)b * o.kout + (long long)(k - b * o.kin) * o.sk;
+}
+
+// The digits of x at row exponent emax as one word: byte 6 - s is d_s + 128 for s = 1..6, the
+// bits from 48 up are d_0 (a balanced base-256 expansion is the plain one of X + 128 (256^0 + .. + 256^5)).
+__device__ __forceinline__ unsigned long long digits(double x, int emax) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo;
+  const int s = emax - max(e, 1) - 2;      // X = m 2^-s, to nearest
+  if (s <= 0) m <<= -s;
+  else m = (s > 60) ? 0ull : (m + (1ull << (s - 1))) >> s;
+  const long long X = ((int)hi < 0) ? -(long long)m : (long long)m;
+  return (unsigned long long)(X + 0x0000808080808080ll);
+}
+
+// d_s of two neighbouring elements as a BF16 pair: 2^23 + byte is an FP32 number, the subtraction
+// exact, and an integer of at most 8 bits has nothing in the low half of its FP32 word.
+template <int S>
+__device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned long long b) {
+  float fa, fb;
+  if (S == 0) {
+    fa = (float)((int)(a >> 32) >> 16);
+    fb = (float)((int)(b >> 32) >> 16);
+  } else {
+    constexpr int byte = 6 - S;
+    const uint32_t wa = byte < 4 ? (uint32_t)a : (uint32_t)(a >> 32), wb = byte < 4 ? (uint32_t)b : (uint32_t)(b >> 32);
+    fa = __uint_as_float(__byte_perm(wa, 0x4B000000u, 0x7440 | (byte & 3))) - 8388736.0f;
+    fb = __uint_as_float(__byte_perm(wb, 0x4B000000u, 0x7440 | (byte & 3))) - 8388736.0f;
+  }
+  return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
+}
+
+// Digit planes in global memory, ready for the MMA: block (tile of TR rows, K block) holds kDig planes
+// of TR rows x 32 bytes in the 32-byte-swizzled K-major layout, so that the GEMM brings the leading planes
+// of a block in with one contiguous bulk copy and no tensor map.
+__device__ __forceinline__ void store_digits(uint8_t *out, int TR, int KB, int row, int q, const unsigned long long (&w)[8],
+                                             uint32_t flip) {
+  const int tile = row / TR, rr = row - tile * TR, kb = q >> 1, c2 = q & 1;
+  const uint32_t plane = (uint32_t)TR * 32;
+  uint8_t *o = out + ((size_t)tile * KB + kb) * (kDig * plane) + rr * 32 + ((c2 ^ ((rr >> 2) & 1)) << 4);
+#define G1G2_PUT(S)                                                                                          \
+  *reinterpret_cast<uint4 *>(o + S * plane) =                                                                \
+      make_uint4(digit_pair<S>(w[0], w[1]) ^ flip, digit_pair<S>(w[2], w[3]) ^ flip,                         \
+                 digit_pair<S>(w[4], w[5]) ^ flip, digit_pair<S>(w[6], w[7]) ^ flip)
+  G1G2_PUT(0); G1G2_PUT(1); G1G2_PUT(2); G1G2_PUT(3); G1G2_PUT(4); G1G2_PUT(5); G1G2_PUT(6);
+#undef G1G2_PUT
+}
+
+// How a complex operand becomes real rows:
+//   kRows    row r: [re | im] along K' (the A side of a complex product)
+//   kReal    rows 2 r, 2 r + 1: [re | -im], [im | re] (its B side: columns re, im of the product)
+//   kPlanes  rows 2 r, 2 r + 1: re, im over K (both sides of a long contraction; the four
+//            real products are combined at the end)
+enum Form : int { kRows = 0, kReal = 1, kPlanes = 2 };
+
+constexpr int kCutVals = 4096;   // complex values of an operand per CTA: one segment of kCutVals / K rows
+__host__ __device__ constexpr int seg_k(int form) { return form == kPlanes ? 256 : 128; }   // operand K values per segment
+__host__ __device__ constexpr int cut_rows(int form) { return kCutVals / seg_k(form); }
+
+// Cuts rows x K of an operand into digits, and finds the exponents.  A CTA stages one segment of 32 rows (16 for
+// kPlanes) in shared memory, read along whichever index is contiguous in memory, takes the largest exponent of each
+// row there, and every thread then cuts eight consecutive K values of one row at a time into seven
+// 16-byte stores; a warp writes 16 rows x 32 bytes, 512 contiguous bytes, per digit.  Bound by its 16
+// bytes read and 28 written per complex element (56 for kReal).
+template <int FORM>
+__global__ void __launch_bounds__(256) cut_digits_kernel(const Operand A, int r_begin, int k_begin, int Klen, int Kp,
+                                                         int TR, int KB, int *__restrict__ rexp,
+                                                         uint8_t *__restrict__ out) {
+  constexpr int SK = seg_k(FORM), SR = cut_rows(FORM);
+  extern __shared__ double sh[];
+  __shared__ long long roff[SR], koff[SK];
+  __shared__ int emax[SR];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int r0 = blockIdx.x * SR;                         // within the panel
+  const int nr = min(SR, A.rows - r0);                    // A.rows: rows of the panel
+  const int seg = blockIdx.y, k0 = seg * SK;
+  const int kt = min(SK, Kp - k0);                        // padded K values of this segment (multiple of 8)
+  const int pitch = kt + 1;
+  double *re = sh, *im = sh + SR * pitch;
+  if (tid < SR) roff[tid] = row_offset(A, r_begin + r0 + min(tid, nr - 1));
+  if (tid < SK) koff[tid] = (k0 + tid < Klen) ? k_offset(A, k_begin + k0 + tid) : -1;
+  __syncthreads();
+  const int flip_im = A.conj ? (int)0x80000000u : 0;
+  auto stage = [&](int r, int k) {
+    cplx v = {0.0, 0.0};
+    if (koff[k] >= 0) v = A.p[roff[r] + koff[k]];
+    re[r * pitch + k] = v.x;
+    im[r * pitch + k] = __hiloint2double(__double2hiint(v.y) ^ flip_im, __double2loint(v.y));
+  };
+  if (A.sk == 1) {
+#pragma unroll
+    for (int i = 0; i < SR / 8; ++i)
+      for (int k = lane; k < kt; k += 32) stage(warp + 8 * i, k);
+  } else {
+    constexpr int kPerWarp = 32 / SR;                     // K values that a warp reads at once
+#pragma unroll 4
+    for (int k = warp * kPerWarp + lane / SR; k < kt; k += 8 * kPerWarp) stage(lane % SR, k);
+  }
+  __syncthreads();
+  {
+    constexpr int T = 256 / SR;                           // threads per row
+    const int r = tid / T, j = tid % T;
+    int e = 0;
+    for (int k = j; k < kt; k += T) {
+      e = max(e, __double2hiint(re[r * pitch + k]) & 0x7ff00000);
+      e = max(e, __double2hiint(im[r * pitch + k]) & 0x7ff00000);
+    }
+#pragma unroll
+    for (int o = T / 2; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    e = max(e >> 20, 1);
+    if (j == 0) {
+      emax[r] = e;
+      if (r < nr) rexp[(size_t)seg * A.rows + r0 + r] = e;
+    }
+  }
+  __syncthreads();
+  const int c2 = lane & 1, rs = lane >> 1;
+  const int nch = kt >> 3;                                // chunks of 8 per plane; pairs of them over both planes
+  for (int g = warp; g < nch * (SR / 16); g += 8) {
+    const int r = (g % (SR / 16)) * 16 + rs, qq = (g / (SR / 16)) * 2 + c2;
+    const int u = qq >= nch ? 1 : 0, kc = qq - u * nch;
+    if (r >= nr) continue;
+    const double *src = (u ? im : re) + r * pitch + kc * 8;
+    const int e = emax[r];
+    unsigned long long w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = digits(e == kNonFinite ? 0.0 : src[i], e);
+    const int q0 = seg * 2 * kSeg, row = r0 + r;          // 16-byte chunks before this segment
+    if (FORM == kRows) {
+      store_digits(out, TR, KB, row, q0 + u * nch + kc, w, 0u);
+    } else if (FORM == kReal) {
+      store_digits(out, TR, KB, 2 * row, q0 + u * nch + kc, w, u ? 0x80008000u : 0u);
+      store_digits(out, TR, KB, 2 * row + 1, q0 + (1 - u) * nch + kc, w, 0u);
+    } else {
+      store_digits(out, TR, KB, 2 * row + u, q0 + kc, w, 0u);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// GEMM
+// ---------------------------------------------------------------------------
+struct TcGemm {
+  const uint8_t *A, *B;       // digit blocks
+  int KB, segs;               // K blocks of a row tile, in segments of kSeg
+  int nt;                     // real columns per tile (multiple of 16)
+  int mtiles, ntiles;         // unit = (split mtiles + m_tile) ntiles + n_tile
+  int splits, segs_per_split; // long contractions: segments cut over the units
+  int *err;
+  long long *sums;            // per CTA: [hi, lo][column][row] of a segment
+  double *part;               // FP64 sums over segments [unit (long contractions) or CTA][column][row]
+  int accumulate;             // long contractions: part holds earlier panels
+  Operand X, Y;               // rows r_begin + m of X, columns y_begin + y of Y, K from k_begin
+  const int *ex, *ey;         // exponents [segment][row of the panel]
+  int exs, eys;               // rows of the panel
+  int r_begin, y_begin, k_begin;
+  int rows, cols;             // complex rows and columns of this panel
+  cplx *C;
+  long long scb, scx, scy;
+  int unit_alpha;             // alpha = i^unit_alpha
+  int beta;                   // 0 or 1
+};
+
+// K-major operand tile with 32-byte rows and 32-byte swizzling (8-row atoms of 256 bytes)
+__device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);          // start address
+  d |= (uint64_t)1 << 16;                            // leading byte offset (unused for swizzled K-major)
+  d |= (uint64_t)(256u >> 4) << 32;                  // stride byte offset: next 8-row group
+  d |= (uint64_t)1 << 46;                            // descriptor version
+  d |= (uint64_t)6 << 61;                            // 32-byte swizzle
+  return d;
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
+// the loaded registers carry no value before the wait: tie them to a point after it
+__device__ __forceinline__ void after_wait(uint32_t (&r)[8]) {
+  asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
+}
+__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+
+// 2^e mant with the sign, where the exponent needs care (subnormal or overflowing results)
+__device__ __noinline__ double scaled(uint32_t mhi, uint32_t mlo, int e, uint32_t sign) {
+  const double v = ldexp((double)(((unsigned long long)mhi << 32) | mlo), e);
+  return sign ? -v : v;
+}
+
+// (hi 2^32 + lo) 2^e as FP64, rounded to nearest, in about fifty 32-bit integer instructions (an FP64 instruction
+// occupies its pipe for 64 cycles per warp: a conversion with two of them was 1.5 times slower) without a branch (but for
+// results outside the normal range): the 96-bit magnitude is shifted left to its leading one by whole words and
+// a funnel shift.  |hi| < 2^62, |lo| < 2^62.
+__device__ __forceinline__ double fixed_to_double(long long hi, long long lo, int e) {
+  hi += lo >> 32;
+  uint32_t w0 = (uint32_t)lo;
+  const uint32_t s = (uint32_t)(int)(hi >> 63);
+  w0 = (w0 ^ s) - s;
+  hi = (hi ^ (long long)(int)s) + ((s & 1u) & (w0 == 0 ? 1u : 0u));
+  uint32_t w2 = (uint32_t)(hi >> 32), w1 = (uint32_t)hi;
+  int p = 1022 + 95 + e;                         // biased exponent - 1 of the result, minus the shift
+  if (w2 == 0) { w2 = w1; w1 = w0; w0 = 0; p -= 32; }
+  if (w2 == 0) { w2 = w1; w1 = 0; p -= 32; }
+  const int lz = __clz((int)w2);
+  const uint32_t t1 = __funnelshift_l(w1, w2, lz), t0 = __funnelshift_l(w0, w1, lz);
+  p -= lz;
+  uint32_t mhi = t1 >> 11, mlo = __funnelshift_r(t0, t1, 11);
+  const uint32_t up = (t0 >> 10) & 1u;
+  mlo += up;
+  mhi += (mlo < up) ? 1u : 0u;
+  if (w2 == 0) return 0.0;
+  if ((uint32_t)p > 2044u) return scaled(mhi, mlo, p + 1 - 1023 - 52, s);
+  return __hiloint2double((int)((mhi + ((uint32_t)p << 20)) | (s & 0x80000000u)), (int)mlo);
+}
+
+// alpha z for alpha = i^u: signs by the integer pipe
+__device__ __forceinline__ cplx mul_unit(cplx z, int u) {
+  const uint32_t sx = (u == 1 || u == 2) ? 0x80000000u : 0u, sy = (u >= 2) ? 0x80000000u : 0u;   // of the results
+  const double x = (u & 1) ? z.y : z.x, y = (u & 1) ? z.x : z.y;
+  return {__hiloint2double(__double2hiint(x) ^ sx, __double2loint(x)),
+          __hiloint2double(__double2hiint(y) ^ sy, __double2loint(y))};
+}
+
+// The FP64 multiply-add sum over one segment of an output element whose row or column holds an Inf or a NaN there.
+__device__ __noinline__ cplx plain_sum(const Operand &X, const Operand &Y, int r, int y, int k0, int k1) {
+  const cplx *a = X.p + row_offset(X, r), *b = Y.p + row_offset(Y, y);
+  cplx s = {0.0, 0.0};
+  for (int k = k0; k < k1; ++k) {
+    cplx u = a[k_offset(X, k)], v = b[k_offset(Y, k)];
+    if (X.conj) u.y = -u.y;
+    if (Y.conj) v.y = -v.y;
+    s = {fma(u.x, v.x, fma(-u.y, v.y, s.x)), fma(u.x, v.y, fma(u.y, v.x, s.y))};
+  }
+  return s;
+}
+// The same for one of the four real products of a long contraction: part pa of A times part pb of B.
+__device__ __noinline__ double plain_part(const Operand &X, const Operand &Y, int r, int pa, int y, int pb, int k0, int k1) {
+  const cplx *a = X.p + row_offset(X, r), *b = Y.p + row_offset(Y, y);
+  double s = 0.0;
+  for (int k = k0; k < k1; ++k) {
+    const cplx u = a[k_offset(X, k)], v = b[k_offset(Y, k)];
+    const double x = pa ? (X.conj ? -u.y : u.y) : u.x, z = pb ? (Y.conj ? -v.y : v.y) : v.x;
+    s = fma(x, z, s);
+  }
+  return s;
+}
+
+// 256 (256 (256 q0 + q1) + q2) + q3 of eight columns, q_o the integer values of four FP32 accumulators.  An
+// integer up to 2^22 shows in the low bits of its sum with 1.5 2^23; larger ones (sums of digit
+// products near their bound) are converted one by one, at a quarter of the rate.
+__device__ __forceinline__ void join_orders(const uint32_t (&v)[4][8], long long (&s)[8]) {
+  float mx = 0.f;
+#pragma unroll
+  for (int o = 0; o < 4; ++o)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) mx = fmaxf(mx, fabsf(__uint_as_float(v[o][j])));
+  if (__any_sync(0xffffffffu, !(mx <= 4194304.f))) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      s[j] = 0;
+#pragma unroll
+      for (int o = 0; o < 4; ++o) s[j] = s[j] * 256 + __float2int_rn(__uint_as_float(v[o][j]));
+    }
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    uint32_t q[4];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) q[o] = __float_as_uint(__uint_as_float(v[o][j]) + 12582912.f);   // 0x4B400000 + q_o
+    const int a = (int)((q[0] << 8) + q[1] - 0x8B400000u), b = (int)((q[2] << 8) + q[3] - 0x8B400000u);
+    s[j] = (long long)a * 65536ll + b;
+  }
+}
+
+// Persistent over units of one 128-row tile x nt real columns x a range of segments.  Roles: warp 0 loads
+// digit blocks (bulk copies, three stages of one 16-element K step), warp 1 issues the MMAs, warps 2-17 drain
+// the accumulators at the end of a segment (a warp reads its lane quarter, every fourth group of eight columns) into
+// integer sums in global memory, which stay in L2, and read them back, convert and store (or add up) while the
+// next MMAs run.  (With the sums in registers the loops over columns had to be unrolled into 70 to 140 KB of
+// code, and instruction fetches made the epilogue three times the MMA time.)
+//
+// An MMA costs the larger of its N / 2 cycles and its operands' shared-memory reads, about (4096 + 32 N) / 88
+// (70 cycles at N = 64, 93 at 128), so wide tiles halve the cost per column.  TMEM holds 512 columns:
+//   G = 8: tiles of up to 64 columns, all eight orders at once (34 MMAs per K step);
+//   G = 4: tiles of up to 128 columns in two phases over a segment, orders 4..7 (24 MMAs), which the conversion of
+//          the last segment overlaps, then orders 0..3 (ten MMAs, four digit planes loaded).
+template <int G, bool kSplit>
+__global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm p) {
+  constexpr int kPhases = kOrd / G;
+  constexpr int kTN = 512 / G;                       // TMEM columns per accumulator
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t *stg_all = smem + kStages * kStageBytes;
+  uint64_t *bars = reinterpret_cast<uint64_t *>(stg_all + kEpiWarps * kStgWarp);
+  uint64_t *full = bars, *empty = bars + kStages, *tfull = bars + 2 * kStages, *tempty = tfull + 1, *fin = tempty + 1;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fin + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t bdig = (uint32_t)p.nt * 32, bblk = kDig * bdig;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(tfull, 1);
+    mbar_init(tempty, 32 * kEpiWarps);
+    mbar_init(fin, 1);
+    mbar_fence_init();
+  }
+  if (warp == 1) tmem_alloc(tmem_slot, 512);
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int units = p.mtiles * p.ntiles * p.splits;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+        const int nt = u % p.ntiles, mt = (u / p.ntiles) % p.mtiles, sp = u / (p.ntiles * p.mtiles);
+        const int s0 = sp * p.segs_per_split, s1 = min(p.segs, s0 + p.segs_per_split);
+        for (int sf = s0 * kPhases; sf < s1 * kPhases && ok; ++sf) {
+          const int f = sf % kPhases, kb0 = (sf / kPhases) * kSeg, kb1 = min(p.KB, kb0 + kSeg);
+          const uint32_t nd = (kPhases == 2 && f == 1) ? 4u : (uint32_t)kDig;
+          for (int kb = kb0; kb < kb1; ++kb) {
+            if (!mbar_wait(&empty[s], ph ^ 1u, p.err)) { ok = false; break; }
+            uint8_t *st = smem + (size_t)s * kStageBytes;
+            mbar_arrive_expect_tx(&full[s], nd * (kADig + bdig));
+            bulk_load(st, p.A + ((size_t)mt * p.KB + kb) * kABlk, nd * kADig, &full[s]);
+            bulk_load(st + kABlk, p.B + ((size_t)nt * p.KB + kb) * bblk, nd * bdig, &full[s]);
+            if (++s == kStages) { s = 0; ph ^= 1u; }
+          }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const uint32_t idesc = idesc_bf16(kTM, p.nt);
+      int s = 0;
+      uint32_t ph = 0, acc_ph = 0;
+      bool ok = true;
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+        const int sp = u / (p.ntiles * p.mtiles);
+        const int s0 = sp * p.segs_per_split, s1 = min(p.segs, s0 + p.segs_per_split);
+        for (int seg = s0; seg < s1 && ok; ++seg) {
+          const int kb0 = seg * kSeg, kb1 = min(p.KB, kb0 + kSeg);
+#pragma unroll
+          for (int f = 0; f < kPhases; ++f) {
+            if (!ok || !mbar_wait(tempty, acc_ph ^ 1u, p.err)) { ok = false; break; }
+            tc_fence_after();
+            for (int kb = kb0; kb < kb1; ++kb) {
+              if (!mbar_wait(&full[s], ph, p.err)) { ok = false; break; }
+              tc_fence_after();
+              const uint32_t sa = smem_u32(smem + (size_t)s * kStageBytes), sb = sa + kABlk;
+              uint64_t a[kDig], b[kDig];
+#pragma unroll
+              for (int q = 0; q < kDig; ++q) {
+                a[q] = smem_desc_sw32(sa + q * kADig);
+                b[q] = smem_desc_sw32(sb + q * bdig);
+              }
+#pragma unroll
+              for (int g = 0; g < G; ++g) {
+                const int o = (kPhases - 1 - f) * G + g, q0 = o < kDig ? 0 : o - kDig + 1;
+#pragma unroll
+                for (int q = q0; q <= o && q < kDig; ++q)
+                  mma_bf16(tmem + (uint32_t)(g * kTN), a[q], b[o - q], idesc, (q == q0 && kb == kb0) ? 0u : 1u);
+              }
+              mma_commit(&empty[s]);
+              if (++s == kStages) { s = 0; ph ^= 1u; }
+            }
+            if (!ok) break;
+            mma_commit(tfull);
+            acc_ph ^= 1u;
+          }
+        }
+      }
+      mma_commit(fin);
+      mbar_wait(fin, 0, p.err);
+    }
+  } else {
+    const int quarter = warp & 3, cg = (warp - 2) >> 2;
+    const int r = 32 * quarter + lane;
+    const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
+    const int ngroups = p.nt >> 3;
+    cplx *stg = reinterpret_cast<cplx *>(stg_all + (warp - 2) * kStgWarp);
+    uint32_t acc_ph = 0;
+    bool ok = true;
+    long long *sums = p.sums + (size_t)blockIdx.x * 2 * kTNMax * kTM + r;
+    for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+      const int ntile = u % p.ntiles, mt = (u / p.ntiles) % p.mtiles, sp = u / (p.ntiles * p.mtiles);
+      const int s0 = sp * p.segs_per_split, s1 = min(p.segs, s0 + p.segs_per_split);
+      double *part = p.part + (size_t)(kSplit ? u : blockIdx.x) * kTNMax * kTM + r;
+      // this lane's row, its exponents and its place in C (a long contraction has rows 2 i + re / im)
+      const int m = mt * kTM + r, mc = kSplit ? m >> 1 : m;
+      const bool valid = mc < p.rows;
+      const int y_tile = (ntile * p.nt) >> 1;           // first complex column of the tile
+      long long off = 0;
+      if (!kSplit && valid) {
+        const int row = p.r_begin + m, b = row / p.X.X;
+        off = (long long)b * p.scb + (long long)(row - b * p.X.X) * p.scx;
+      }
+      for (int seg = s0; seg < s1 && ok; ++seg) {
+        // exponents, loaded before the MMAs are waited for: lane 4 i + j holds that of column j of this warp's
+        // i-th group
+        const int yl = y_tile + 4 * (cg + (lane & ~3)) + (lane & 3);
+        const int ea = valid ? p.ex[(size_t)seg * p.exs + mc] : 1;
+        const int eyl = (lane < 16 && yl < p.cols) ? p.ey[(size_t)seg * p.eys + yl] : 1;
+        const bool any_bad = __any_sync(0xffffffffu, ea == kNonFinite || eyl == kNonFinite);
+#pragma unroll 1
+        for (int f = 0; f < kPhases; ++f) {
+          if (!__all_sync(0xffffffffu, mbar_wait(tfull, acc_ph, p.err))) { ok = false; break; }
+          tc_fence_after();
+#pragma unroll 1
+          for (int g = cg; g < ngroups; g += 4) {
+#pragma unroll
+            for (int w = 0; w < G / 4; ++w) {
+              long long *q = sums + (size_t)(8 * g) * kTM + ((G == 8 ? w : 1 - f) ? kTNMax * kTM : 0);
+              long long s[8];
+              uint32_t v[4][8];
+#pragma unroll
+              for (int o = 0; o < 4; ++o)
+                tmem_ld8(tmem + lane_base + (uint32_t)((4 * w + o) * kTN + 8 * g), v[o]);
+              asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+              for (int o = 0; o < 4; ++o) after_wait(v[o]);
+              join_orders(v, s);
+#pragma unroll
+              for (int j = 0; j < 8; ++j) __stcg(q + j * kTM, s[j]);
+            }
+          }
+          tc_fence_before();
+          mbar_arrive(tempty);
+          acc_ph ^= 1u;
+        }
+        if (!ok) break;
+        const bool first = seg == s0 && !(kSplit && p.accumulate), last = seg == s1 - 1;
+        const int seg_len = seg_k(kSplit ? kPlanes : kRows);
+        const int k0 = p.k_begin + seg * seg_len, k1 = min(p.X.K, k0 + seg_len);
+#pragma unroll 1
+        for (int g = cg; g < ngroups; g += 4) {
+          const int y0 = y_tile + 4 * g;                 // first complex column of the group
+          const int ny = min(4, p.cols - y0);
+          if (ny <= 0) break;
+          const long long *q = sums + (size_t)(8 * g) * kTM;
+          double *pq = part + (size_t)(8 * g) * kTM;
+          long long hi[8], lo[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            hi[j] = __ldcg(q + j * kTM);
+            lo[j] = __ldcg(q + j * kTM + kTNMax * kTM);
+          }
+          double v[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int e = ea + __shfl_sync(0xffffffffu, eyl, g - cg + (j >> 1)) - 2114;
+            v[j] = fixed_to_double(hi[j], lo[j], e);
+          }
+          if (any_bad) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int eb = __shfl_sync(0xffffffffu, eyl, g - cg + j);   // every lane: not behind a condition
+              if ((ea == kNonFinite || eb == kNonFinite) && valid && j < ny) {
+                if (kSplit) {
+                  v[2 * j] = plain_part(p.X, p.Y, mc, m & 1, y0 + j, 0, k0, k1);
+                  v[2 * j + 1] = plain_part(p.X, p.Y, mc, m & 1, y0 + j, 1, k0, k1);
+                } else {
+                  const cplx z = plain_sum(p.X, p.Y, p.r_begin + m, p.y_begin + y0 + j, k0, k1);
+                  v[2 * j] = z.x;
+                  v[2 * j + 1] = z.y;
+                }
+              }
+            }
+            __syncwarp();
+          }
+          if (!first) {   // a branch, not a select: an idle FP64 addition costs as much as a needed one
+            double o[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) o[j] = __ldcg(pq + j * kTM);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] += o[j];
+          }
+          if (kSplit || !last) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) __stcg(pq + j * kTM, v[j]);
+            continue;
+          }
+          cplx z[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) z[j] = mul_unit({v[2 * j], v[2 * j + 1]}, p.unit_alpha);
+          if (p.scy != 1) {
+            // rows contiguous in C (or neither): a lane stores its own row, loads of the old values first
+            cplx *c = p.C + off + (long long)(p.y_begin + y0) * p.scy;
+            if (p.beta) {
+              cplx c0[4];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) c0[j] = (valid && j < ny) ? c[(long long)j * p.scy] : cplx{0.0, 0.0};
+#pragma unroll
+              for (int j = 0; j < 4; ++j) z[j] = {z[j].x + c0[j].x, z[j].y + c0[j].y};
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (valid && j < ny) c[(long long)j * p.scy] = z[j];
+          } else {
+            // columns contiguous in C: through the warp's staging tile, then 64 contiguous bytes of eight
+            // rows per store
+            const int j = lane & 3;
+            cplx *c = p.C + p.y_begin + y0 + j;
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) stg[lane * kStgPitch + i] = z[i];
+            __syncwarp();
+            long long ro[4];
+            bool in[4];
+            cplx t[4];
+#pragma unroll
+            for (int it = 0; it < 4; ++it) {
+              const int rr = 8 * it + (lane >> 2);
+              ro[it] = __shfl_sync(0xffffffffu, off, rr);
+              in[it] = mt * kTM + 32 * quarter + rr < p.rows && j < ny;
+              t[it] = stg[rr * kStgPitch + j];
+            }
+            if (p.beta) {
+              cplx c0[4];
+#pragma unroll
+              for (int it = 0; it < 4; ++it) c0[it] = in[it] ? c[ro[it]] : cplx{0.0, 0.0};
+#pragma unroll
+              for (int it = 0; it < 4; ++it) t[it] = {t[it].x + c0[it].x, t[it].y + c0[it].y};
+            }
+#pragma unroll
+            for (int it = 0; it < 4; ++it)
+              if (in[it]) c[ro[it]] = t[it];
+          }
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+}
+
+// Sums the units of a long contraction in a fixed order and combines the four real products:
+// C[i][j] = alpha ((re re - im im) + i (re im + im re)) + beta C.  One warp per output element.
+__global__ void __launch_bounds__(256) fp64_tc_reduce_kernel(const TcGemm p) {
+  const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (idx >= p.rows * p.cols) return;
+  const int i = idx / p.cols, j = idx - i * p.cols;
+  const int mt = 2 * i / kTM, nt = 2 * j / p.nt, rr = 2 * i - mt * kTM, cc = 2 * j - nt * p.nt;
+  double x = 0.0, y = 0.0;
+  for (int sp = lane; sp < p.splits; sp += 32) {
+    const double *q = p.part + ((size_t)(sp * p.mtiles + mt) * p.ntiles + nt) * kTNMax * kTM + (size_t)cc * kTM + rr;
+    x += q[0] - q[kTM + 1];
+    y += q[kTM] + q[1];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    x += __shfl_xor_sync(0xffffffffu, x, o);
+    y += __shfl_xor_sync(0xffffffffu, y, o);
+  }
+  if (lane != 0) return;
+  cplx z = mul_unit({x, y}, p.unit_alpha);
+  cplx *c = p.C + (long long)i * p.scx + (long long)j * p.scy;
+  if (p.beta) z = {z.x + c->x, z.y + c->y};
+  *c = z;
+}
+
+int unit_of(cplx a) {
+  if (a.x == 1.0 && a.y == 0.0) return 0;
+  if (a.x == 0.0 && a.y == 1.0) return 1;
+  if (a.x == -1.0 && a.y == 0.0) return 2;
+  if (a.x == 0.0 && a.y == -1.0) return 3;
+  return -1;
+}
+
+int round_up(int x, int m) { return (x + m - 1) / m * m; }
+
+// Real columns per tile: as few tiles of at most 128 as the columns need, evenly filled.  Up to 64 columns
+// run with all orders in TMEM at once (G = 8).
+int tile_columns(int real_cols) {
+  const int tiles = (real_cols + kTNMax - 1) / kTNMax;
+  return round_up((real_cols + tiles - 1) / tiles, 16);
+}
+
+template <bool kSplit>
+void launch_gemm(Launcher &L, const TcGemm &t, int ctas, const char *tag) {
+  L.before(tag);
+  if (t.nt <= 64) fp64_tc_gemm_kernel<8, kSplit><<<ctas, kThreads, kSmem, L.stream>>>(t);
+  else fp64_tc_gemm_kernel<4, kSplit><<<ctas, kThreads, kSmem, L.stream>>>(t);
+  L.after_launch();
+}
+
+template <int FORM>
+void cut(Launcher &L, const Operand &o, int r_begin, int rows, int k_begin, int Klen, int Kp, int TR, int KB, int *rexp,
+         uint8_t *out) {
+  Operand A = o;
+  A.rows = rows;
+  const int kt = std::min(seg_k(FORM), Kp);
+  const size_t sh = (size_t)2 * cut_rows(FORM) * (kt + 1) * sizeof(double);
+  dim3 grid((rows + cut_rows(FORM) - 1) / cut_rows(FORM), (Kp + seg_k(FORM) - 1) / seg_k(FORM));
+  L.before("fp64_tc_digits");
+  cut_digits_kernel<FORM><<<grid, 256, sh, L.stream>>>(A, r_begin, k_begin, Klen, Kp, TR, KB, rexp, out);
+  L.after_launch();
+}
+
+}  // namespace
+
+constexpr int kMinK = 8, kMinCols = 8;
+constexpr double kMinWork = 1e6;
+
+int fp64_tc_min_nb() { return 16; }
+
+struct Fp64Tc {
+  uint8_t *A = nullptr, *B = nullptr;   // digit blocks of the two operands
+  size_t a_bytes = 0, b_bytes = 0;
+  int *ex = nullptr, *ey = nullptr;     // exponents
+  long long exps = 0;                   // of each
+  long long *sums = nullptr;            // hi and lo sums of a tile per CTA
+  double *part = nullptr;               // FP64 sums of a tile per CTA
+  int *err = nullptr;
+  int sms = 0;
+};
+
+void fp64_tc_destroy(Fp64Tc *f) {
+  if (!f) return;
+  for (void *p : {(void *)f->A, (void *)f->B, (void *)f->ex, (void *)f->ey, (void *)f->sums, (void *)f->part, (void *)f->err})
+    if (p) cudaFree(p);
+  delete f;
+}
+
+Fp64Tc *fp64_tc_create(int nb, bool pair_products) {
+  const long long N = nb, N2 = N * N, N3 = N2 * N;
+  Fp64Tc *f = new (std::nothrow) Fp64Tc;
+  if (!f) return nullptr;
+  // digit blocks: all of a big operand up to kPanelBytes, panels of it above
+  constexpr size_t kPanelBytes = (size_t)1 << 30;
+  auto blocks = [](long long rows, long long Kp) { return (size_t)((rows + 127) / 128 * 128) * (size_t)Kp * 2 * kDig; };
+  const size_t big = blocks(N3, 2 * ((N + 7) / 8 * 8)), pair = pair_products ? blocks(2 * N2, 2 * ((N2 + 7) / 8 * 8)) : 0;
+  const size_t lng = blocks(2 * N, (N3 + 255) / 256 * 256);
+  f->a_bytes = std::min(kPanelBytes, std::max({big, pair, lng}));
+  f->b_bytes = std::min(kPanelBytes, std::max({blocks(2 * N, 2 * ((N + 7) / 8 * 8)), pair, lng}));
+  f->exps = std::max({N3, N2 * ((N2 + 127) / 128), N * ((N3 + 255) / 256)});
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&f->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    goto bad;
+  if (cudaMalloc(&f->A, f->a_bytes) != cudaSuccess || cudaMalloc(&f->B, f->b_bytes) != cudaSuccess ||
+      cudaMalloc(&f->ex, sizeof(int) * (size_t)f->exps) != cudaSuccess ||
+      cudaMalloc(&f->ey, sizeof(int) * (size_t)f->exps) != cudaSuccess ||
+      cudaMalloc(&f->sums, (size_t)f->sms * 2 * kTNMax * kTM * sizeof(long long)) != cudaSuccess ||
+      cudaMalloc(&f->part, (size_t)f->sms * kTNMax * kTM * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&f->err, sizeof(int)) != cudaSuccess || cudaMemset(f->err, 0, sizeof(int)) != cudaSuccess)
+    goto bad;
+  for (const void *k : {(const void *)fp64_tc_gemm_kernel<8, false>, (const void *)fp64_tc_gemm_kernel<8, true>,
+                        (const void *)fp64_tc_gemm_kernel<4, false>, (const void *)fp64_tc_gemm_kernel<4, true>})
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem) != cudaSuccess) goto bad;
+  {
+    const int sh = 2 * (kCutVals + 32) * (int)sizeof(double);
+    for (const void *k : {(const void *)cut_digits_kernel<kRows>, (const void *)cut_digits_kernel<kReal>,
+                          (const void *)cut_digits_kernel<kPlanes>})
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sh) != cudaSuccess) goto bad;
+  }
+  return f;
+bad:
+  cudaGetLastError();
+  fp64_tc_destroy(f);
+  return nullptr;
+}
+
+int fp64_tc_error(Fp64Tc *f, cudaStream_t stream) {
+  int e = 0;
+  if (cudaMemcpyAsync(&e, f->err, sizeof(int), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+      cudaStreamSynchronize(stream) != cudaSuccess) {
+    set_error_detail("reading the FP64 tensor-core error word failed");
+    return G1G2_ECUDA;
+  }
+  if (e == 0) return G1G2_OK;
+  cudaMemsetAsync(f->err, 0, sizeof(int), stream);
+  set_error_detail("a barrier wait of an FP64 tensor-core kernel gave up");
+  return G1G2_ETIMEOUT;
+}
+
+// C_b = alpha A_b B_b + beta C_b.  The operand with the batch (or the more rows) gives the tile rows, the other the
+// columns.
+bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
+  Fp64Tc *f = L.ftc;
+  if (!f) return false;
+  const int alpha = unit_of(g.alpha);
+  if (alpha < 0 || (g.beta != 0.0 && g.beta != 1.0)) return false;
+  if (g.batch > 1 && g.sa_b != 0 && g.sb_b != 0) return false;
+  const bool a_rows = g.batch > 1 ? g.sa_b != 0 : g.M >= g.N;
+  Operand X{}, Y{};
+  Operand a{g.A, g.sa_b, g.sa_m, g.sa_k, 0, g.M, g.K, g.M, g.K, g.conjA ? 1 : 0};
+  Operand b{g.B, g.sb_b, g.sb_n, g.sb_k, 0, g.N, g.K, g.N, g.K, g.conjB ? 1 : 0};
+  X = a_rows ? a : b;
+  Y = a_rows ? b : a;
+  const long long rows = (long long)X.X * g.batch;
+  const int cols = Y.X;
+  if (g.K < kMinK || cols < kMinCols || (double)rows * cols * g.K < kMinWork) return false;
+  const int Kp = round_up(g.K, 8), KB = 2 * Kp / kKB, segs = (KB + kSeg - 1) / kSeg;
+  if (std::max<long long>(rows, cols) * segs > f->exps) return false;
+  X.rows = (int)rows;
+  const int nt = tile_columns(2 * cols);
+  // panels of whole tiles
+  const size_t a_tile = (size_t)KB * kABlk, b_tile = (size_t)KB * kDig * nt * 32;
+  const int all_m = (int)((rows + kTM - 1) / kTM), all_n = (2 * cols + nt - 1) / nt;
+  const int pm = (int)std::min<size_t>(all_m, f->a_bytes / a_tile), pn = (int)std::min<size_t>(all_n, f->b_bytes / b_tile);
+  if (pm < 1 || pn < 1) return false;
+  for (int n0 = 0; n0 < all_n; n0 += pn) {
+    const int y0 = n0 * nt / 2, ny = std::min(cols - y0, std::min(pn, all_n - n0) * nt / 2);
+    cut<kReal>(L, Y, y0, ny, 0, g.K, Kp, nt, KB, f->ey, f->B);
+    for (int m0 = 0; m0 < all_m; m0 += pm) {
+      const int r0 = m0 * kTM, nr = (int)std::min<long long>(rows - r0, (long long)std::min(pm, all_m - m0) * kTM);
+      if (n0 == 0 || pm < all_m) cut<kRows>(L, X, r0, nr, 0, g.K, Kp, kTM, KB, f->ex, f->A);
+      TcGemm t{};
+      t.A = f->A; t.B = f->B; t.KB = KB; t.segs = segs; t.nt = nt;
+      t.mtiles = (nr + kTM - 1) / kTM; t.ntiles = (2 * ny + nt - 1) / nt;
+      t.splits = 1; t.segs_per_split = segs; t.err = f->err; t.sums = f->sums; t.part = f->part;
+      t.X = X; t.Y = Y; t.ex = f->ex; t.ey = f->ey; t.exs = nr; t.eys = ny;
+      t.r_begin = r0; t.y_begin = y0; t.rows = nr; t.cols = ny;
+      t.C = g.C; t.scb = g.sc_b; t.scx = a_rows ? g.sc_m : g.sc_n; t.scy = a_rows ? g.sc_n : g.sc_m;
+      t.unit_alpha = alpha; t.beta = g.beta != 0.0;
+      launch_gemm<false>(L, t, std::min(f->sms, t.mtiles * t.ntiles), segs > 1 ? "fp64_tc_gemm_pair" : "fp64_tc_gemm");
+    }
+  }
+  return true;
+}
+
+// C = alpha sum_b A_b B_b + beta C: one contraction over c = (b, k), both operands as re and im rows.
+bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g) {
+  Fp64Tc *f = L.ftc;
+  if (!f) return false;
+  const int alpha = unit_of(g.alpha);
+  if (alpha < 0 || (g.beta != 0.0 && g.beta != 1.0)) return false;
+  const long long Kl = (long long)g.K * g.batch;
+  if (Kl > (1ll << 30) || std::min(g.M, g.N) < kMinCols || (double)g.M * g.N * Kl < kMinWork) return false;
+  const int K = (int)Kl;
+  Operand X{g.A, 0, g.sa_m, g.sa_k, g.sa_b, g.M, g.K, g.M, K, g.conjA ? 1 : 0};
+  Operand Y{g.B, 0, g.sb_n, g.sb_k, g.sb_b, g.N, g.K, g.N, K, g.conjB ? 1 : 0};
+  const int nt = tile_columns(2 * g.N);
+  const int mtiles = (2 * g.M + kTM - 1) / kTM, ntiles = (2 * g.N + nt - 1) / nt;
+  const int splits_max = f->sms / (mtiles * ntiles);   // one unit per CTA
+  if (splits_max < 1) return false;
+  const size_t a_seg = (size_t)mtiles * kSeg * kABlk, b_seg = (size_t)ntiles * kSeg * kDig * nt * 32;   // bytes per segment
+  const int all_segs = (K + kSeg * kKB - 1) / (kSeg * kKB);
+  int ps = (int)std::min<size_t>(all_segs, std::min(f->a_bytes / a_seg, f->b_bytes / b_seg));
+  ps = (int)std::min<long long>(ps, f->exps / std::max(g.M, g.N));
+  if (ps < 1) return false;
+  TcGemm t{};
+  for (int sg0 = 0; sg0 < all_segs; sg0 += ps) {
+    const int ns = std::min(ps, all_segs - sg0), k0 = sg0 * kSeg * kKB, Klen = std::min(K - k0, ns * kSeg * kKB);
+    const int Kp = round_up(Klen, kKB), KB = Kp / kKB;
+    cut<kPlanes>(L, X, 0, g.M, k0, Klen, Kp, kTM, KB, f->ex, f->A);
+    cut<kPlanes>(L, Y, 0, g.N, k0, Klen, Kp, nt, KB, f->ey, f->B);
+    t.A = f->A; t.B = f->B; t.KB = KB; t.segs = ns; t.nt = nt; t.mtiles = mtiles; t.ntiles = ntiles;
+    // the first panel is the longest: its split count holds for the later ones
+    if (sg0 == 0) {
+      t.segs_per_split = (ns + splits_max - 1) / splits_max;
+      t.splits = (ns + t.segs_per_split - 1) / t.segs_per_split;
+    } else {
+      t.segs_per_split = (ns + t.splits - 1) / t.splits;
+    }
+    t.err = f->err; t.X = X; t.Y = Y; t.ex = f->ex; t.ey = f->ey; t.exs = g.M; t.eys = g.N; t.rows = g.M; t.cols = g.N;
+    t.k_begin = k0;
+    t.C = g.C; t.scx = g.sc_m; t.scy = g.sc_n; t.unit_alpha = alpha; t.beta = g.beta != 0.0;
+    t.sums = f->sums; t.part = f->part; t.accumulate = sg0 > 0;
+    launch_gemm<true>(L, t, t.splits * mtiles * ntiles, "fp64_tc_gemm_long");
+  }
+  L.before("fp64_tc_reduce");
+  fp64_tc_reduce_kernel<<<(g.M * g.N + 7) / 8, 256, 0, L.stream>>>(t);
+  L.after_launch();
+  return true;
+}
+
+}  // namespace g1g2

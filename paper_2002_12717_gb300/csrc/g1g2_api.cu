@@ -67,6 +67,7 @@ struct g1g2_ctx {
   double *W_dev = nullptr;          // accumulated drive work
   std::vector<void *> allocs;
   TcPath *tc = nullptr;             // split-precision tensor-core path (precision != FP64)
+  Fp64Tc *ftc = nullptr;            // tensor-core FP64 products (FP64 form)
   Profiler prof;
   // discrete adjoint (FP64 form), allocated on first use
   cplx *zero_h = nullptr;                       // nb*nb zeros: h for the w-part of the RHS
@@ -96,6 +97,7 @@ struct g1g2_ctx {
     L.stream = stream;
     L.counter = &launches;
     L.prof = &prof;
+    L.ftc = ftc;
     return L;
   }
 };
@@ -122,6 +124,13 @@ int cuda_check(cudaError_t e, const char *what) {
 int launch_status(Launcher &L, const char *what) {
   if (L.err != cudaSuccess) return fail(G1G2_ECUDA, std::string(what) + ": " + cudaGetErrorString(L.err));
   return G1G2_OK;
+}
+
+// G1G2_ETIMEOUT when a tensor-core kernel of this context gave up on a barrier
+int wait_error(g1g2_ctx *c) {
+  int rc = c->tc ? tc_error(c->tc, c->stream) : G1G2_OK;
+  if (!rc && c->ftc) rc = fp64_tc_error(c->ftc, c->stream);
+  return rc;
 }
 
 using zc = std::complex<double>;
@@ -532,7 +541,7 @@ int observables_impl(g1g2_ctx *c, g1g2_obs *out, double *density, double *nonfin
       return rc;
   }
   if ((rc = cuda_check(cudaStreamSynchronize(c->stream), "obs sync"))) return rc;
-  if (c->tc && (rc = tc_error(c->tc, c->stream))) return rc;
+  if ((rc = wait_error(c))) return rc;
   const bool restricted = c->basis == G1G2_SPIN_RESTRICTED;
   const double s = restricted ? 2.0 : 1.0;
   out->t = c->t;
@@ -1049,6 +1058,7 @@ void g1g2_destroy(g1g2_ctx *c) {
   if (!c) return;
   if (c->stream) cudaStreamSynchronize(c->stream);
   if (c->tc) tc_destroy(c->tc);
+  fp64_tc_destroy(c->ftc);
   for (void *p : c->adj_allocs) cudaFree(p);
   for (void *p : c->allocs) cudaFree(p);
   delete c;
@@ -1217,6 +1227,8 @@ int g1g2_init(g1g2_ctx **out, int nb, const double *h, const double *w, const do
       return bail(rc);
     c->splits = 4 * 152;
     if ((rc = dalloc(c, &c->partial, (size_t)c->splits * N2))) return bail(rc);
+    if (nb >= fp64_tc_min_nb())
+      c->ftc = fp64_tc_create(nb, !restricted_gw && se != G1G2_SOA);
     if ((se == G1G2_GW && !restricted_gw) || se == G1G2_TPH || se == G1G2_DSL) {
       if ((rc = dalloc(c, &c->Hb, N4)) || (rc = dalloc(c, &c->Gp, N4)) || (rc = dalloc(c, &c->Hp, N4)) ||
           (rc = dalloc(c, &c->Pp, N4)))
@@ -1501,7 +1513,7 @@ int g1g2_propagate(g1g2_ctx *c, double dt, int nsteps, int obs_every, g1g2_obs *
     if (recording && (s + 1) % obs_every == 0 && (rc = record())) return rc;
   }
   if ((rc = cuda_check(cudaStreamSynchronize(c->stream), "propagate sync"))) return rc;
-  return c->tc ? tc_error(c->tc, c->stream) : G1G2_OK;
+  return wait_error(c);
 }
 
 // Original HF-GKBA with the SOA selfenergy, the memory-integral form the G1-G2
@@ -1581,6 +1593,7 @@ int g1g2_propagate_hfgkba(g1g2_ctx *c, double dt, int nsteps, double *G1_history
                        "history")))
     return rc;
   if ((rc = cuda_check(cudaStreamSynchronize(c->stream), "memory-integral sync"))) return rc;
+  if ((rc = wait_error(c))) return rc;
   c->t += nsteps * dt;
   return G1G2_OK;
 }
@@ -1957,6 +1970,7 @@ int g1g2_adjoint(g1g2_ctx *c, double dt, int nsteps, int ckpt_every, int objecti
   std::vector<cplx> hg(N2);
   if (grad_h) cudaMemcpyAsync(hg.data(), c->adj_hsum, N2 * sizeof(cplx), cudaMemcpyDeviceToHost, c->stream);
   if ((rc = cuda_check(cudaStreamSynchronize(c->stream), "adjoint sync"))) return done(rc);
+  if ((rc = wait_error(c))) return done(rc);
   *J_out = J;
   // E(T) - E(0) also depends on w directly: its interaction energies are linear in w
   if (grad_wscale) *grad_wscale = hacc[0] + (objective == 2 ? EintT - Eint0 : 0.0);

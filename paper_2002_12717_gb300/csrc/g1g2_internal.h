@@ -36,7 +36,10 @@ struct Profiler {
   ~Profiler() { for (cudaEvent_t e : pool) cudaEventDestroy(e); }
 };
 
+struct Fp64Tc;   // digit workspaces of the tensor-core FP64 products (fp64_tc.cu)
+
 struct Launcher {
+  Fp64Tc *ftc = nullptr;
   cudaStream_t stream = nullptr;
   long long *counter = nullptr;
   Profiler *prof = nullptr;
@@ -73,6 +76,19 @@ struct ZGemm {
 };
 void zgemm(Launcher &L, const ZGemm &g);
 void zgemm_reduce(Launcher &L, const ZGemm &g, cplx *partial, int splits);
+
+// The same products on the tensor cores from digits of the FP64 operands (fp64_tc.cu), FP64-accurate.  Both
+// return false, with nothing launched, for a product that the CUDA-core kernels take (no workspace
+// in L, too small, a general alpha, both operands batched): zgemm and zgemm_reduce ask them first.
+bool fp64_tc_zgemm(Launcher &L, const ZGemm &g);
+bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g);
+// Workspaces for one context of basis size nb (nullptr when they do not fit: the CUDA-core kernels then take
+// every product); pair_products: nb^2 x nb^2 x nb^2 products are among them.
+Fp64Tc *fp64_tc_create(int nb, bool pair_products);
+int fp64_tc_min_nb();   // smallest basis size with a product that takes this path
+void fp64_tc_destroy(Fp64Tc *f);
+// G1G2_ETIMEOUT when one of the kernels gave up on a barrier (synchronises the stream).
+int fp64_tc_error(Fp64Tc *f, cudaStream_t stream);
 
 // out(a0,a1,a2,a3) = beta*out + alpha*op(in(a_p0, a_p1, a_p2, a_p3)), op = conj if conj.
 void permute4(Launcher &L, int nb, const cplx *in, cplx *out, const int p[4], cplx alpha, double beta,
