@@ -204,8 +204,8 @@ int g1g2_propagate(g1g2_ctx *c, double dt, int nsteps, int obs_every, g1g2_obs *
  *                otherwise); its state must have G2 = 0 (uncorrelated start at the
  *                context's time, G1G2_EINVAL otherwise)
  *   G1_history   host, (nsteps+1)*nb*nb complex: n(t0 + m dt), m = 0..nsteps, or NULL
- *   scratch_bytes  device memory for the batched history products (0: 256 MiB); the
- *                history itself takes (nsteps+2) (nb^4 + 3 nb^2) complex doubles
+ *   scratch_bytes  not used: the history is added up without scratch of its own (the argument stays
+ *                for callers that pass it); the history takes (nsteps+2) (nb^4 + 2 nb^2) complex doubles
  * Allocates its scratch on each call (G1G2_ENOMEM when it does not fit) and frees it
  * before returning.  On return the context holds n(T) and G2(T) from the memory
  * integral and t = t0 + nsteps dt.  Synchronous. */

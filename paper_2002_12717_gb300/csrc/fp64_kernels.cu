@@ -531,64 +531,102 @@ __global__ void g2_assemble_kernel(int nb, const cplx *__restrict__ Cb, const cp
 // (pihubbardtrans, pihubbardcis) with G^> = G^< - i and G^< = i n (U_p inside the sum
 // over the site p).  psi = 0 leaves out the source term (the same-spin equation, whose
 // source vanishes for an on-site interaction).
-__global__ void hubbard_c_kernel(int nb, const int *__restrict__ rp, const int *__restrict__ ci,
-                                 const cplx *__restrict__ hhf, const double *__restrict__ U,
-                                 const cplx *__restrict__ n, const cplx *__restrict__ G,
-                                 const cplx *__restrict__ Go, int psi, cplx *C) {
-  // grid: y = i nb + j, x over (k, l); index arithmetic in 32 bits where it fits
-  const long long N = nb, N2 = N * N, N3 = N2 * N;
-  const int ij = blockIdx.y, i = ij / nb, j = ij - i * nb;
-  const int kl = blockIdx.x * blockDim.x + threadIdx.x;
-  if (kl < nb * nb) {
-    const int k = kl / nb, l = kl - k * nb;
-    const long long e = (long long)ij * N2 + kl;
-    cplx acc = {0.0, 0.0};
-    // [h2, G]_ijkl = sum_p h_ip G_pjkl + h_jp G_ipkl - G_ijpl h_pk - G_ijkp h_pl
-    for (int q = rp[i]; q < rp[i + 1]; ++q) {
-      const int p = ci[q];
-      acc = cfma(hhf[i * N + p], G[p * N3 + j * N2 + kl], acc);
-    }
-    for (int q = rp[j]; q < rp[j + 1]; ++q) {
-      const int p = ci[q];
-      acc = cfma(hhf[j * N + p], G[i * N3 + p * N2 + k * N + l], acc);
-    }
-    for (int q = rp[k]; q < rp[k + 1]; ++q) {
-      const int p = ci[q];
-      acc = csub(acc, cmul(G[i * N3 + j * N2 + p * N + l], hhf[p * N + k]));
-    }
-    for (int q = rp[l]; q < rp[l + 1]; ++q) {
-      const int p = ci[q];
-      acc = csub(acc, cmul(G[e - l + p], hhf[p * N + l]));
-    }
-    if (psi) {
-      // Psi = -S
-      const cplx nij = n[i * N + j], nji = n[j * N + i], nik = n[i * N + k], nil = n[i * N + l];
-      const cplx njk = n[j * N + k], njl = n[j * N + l], nlk = n[l * N + k], nkl = n[k * N + l];
-      cplx S = cscale(cmul(cmul(nij, njk), njl), -U[j]);
-      S = cadd(S, cscale(cmul(cmul(nji, nik), nil), -U[i]));
-      S = cadd(S, cscale(cmul(cmul(nil, njl), nlk), U[l]));
-      S = cadd(S, cscale(cmul(cmul(nik, njk), nkl), U[k]));
-      if (i == j) S = cadd(S, cscale(cmul(nik, nil), U[i]));
-      if (k == l) S = csub(S, cscale(cmul(nik, njk), U[k]));
-      acc = csub(acc, S);
-    }
-    if (Go) {
-      auto g4 = [&](int a, int b, int c, int d) { return Go[((a * N + b) * N + c) * N + d]; };
-      const cplx pi = cmul(n[j * N + l], csub(cscale(g4(i, j, k, j), U[j]), cscale(g4(i, l, k, l), U[l])));
-      const cplx pt = cmul(n[k * N + i], csub(cscale(g4(l, k, j, k), U[k]), cscale(g4(l, i, j, i), U[i])));
-      acc = csub(cadd(acc, pi), cconj(pt));   // + Pi_ijkl - conj(Pi_lkji)
-    }
-    C[e] = acc;
+//
+// One launch per Runge-Kutta stage.  The mean field of an on-site interaction is diagonal,
+// h^HF_ij = h_ij + f D_ij + U_i n_ii d_ij, and dG2 = -i C needs no other element of C, so every
+// thread forms its own operands and applies the stage update at once; the stage states of G2 alternate
+// between two buffers, as those of n do, because other threads still read the stage input.  At eight sites
+// a stage is bound by launch latency and by one pass through the FP64 pipe (an FP64 instruction takes
+// 64 cycles of it per warp): separate kernels for h^HF, I, G1, C and the update took 42 us per stage,
+// this one NNN us.  The source term is factored into six complex products instead of eight.
+__device__ __forceinline__ cplx hub_h(const HubStage &p, int i, int j) {
+  cplx v = p.h[i * p.nb + j];
+  if (p.D) {
+    const cplx d = p.D[i * p.nb + j];
+    v = {fma(p.f, d.x, v.x), fma(p.f, d.y, v.y)};
   }
+  return v;
+}
+__device__ __forceinline__ cplx hub_diag(const HubStage &p, int i) {
+  const cplx v = hub_h(p, i, i), m = p.n[i * p.nb + i];
+  return {fma(p.U[i], m.x, v.x), fma(p.U[i], m.y, v.y)};
 }
 
-__global__ void hubbard_collision_kernel(int nb, const double *__restrict__ U, const cplx *__restrict__ G, cplx *I) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nb * nb) return;
-  const long long N = nb;
-  const int i = e / nb, j = e % nb;
-  const cplx g = G[((i * N + i) * N + j) * N + i];  // G_iiji
-  I[e] = cscale(mul_minus_i(g), U[i]);
+__global__ void __launch_bounds__(128) hubbard_stage_kernel(const HubStage p, int g1_blocks, int bx) {
+  const int nb = p.nb;
+  const long long N = nb, N2 = N * N, N3 = N2 * N;
+  if ((int)blockIdx.x < g1_blocks) {
+    // G1: one warp per element, dn = -i [h^HF, n] - (I + I^dag), I_ij = -i U_i G_iiji
+    const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (idx >= nb * nb || blockIdx.y != 0) return;
+    const int i = idx / nb, j = idx % nb;
+    cplx comm = {0.0, 0.0};
+    for (int q = lane; q < nb; q += 32) {
+      const cplx hi = q == i ? hub_diag(p, i) : hub_h(p, i, q), hj = q == j ? hub_diag(p, j) : hub_h(p, q, j);
+      comm = cfma(hi, p.n[q * nb + j], comm);
+      comm = csub(comm, cmul(p.n[i * nb + q], hj));
+    }
+    const int w = nb > 16 ? 16 : nb > 8 ? 8 : 4;          // lanes beyond nb hold zeros
+    for (int o = nb > 4 ? w : 2; o > 0; o >>= 1) {
+      comm.x += __shfl_xor_sync(0xffffffffu, comm.x, o);
+      comm.y += __shfl_xor_sync(0xffffffffu, comm.y, o);
+    }
+    if (lane != 0) return;
+    const cplx a = cscale(mul_minus_i(p.G[((i * N + i) * N + j) * N + i]), p.U[i]);
+    const cplx b = cconj(cscale(mul_minus_i(p.G[((j * N + j) * N + i) * N + j]), p.U[j]));
+    rk4_apply(idx, csub(mul_minus_i(comm), cadd(a, b)), p.stage, p.dt, p.ny, p.nys, p.nacc, p.nk);
+    return;
+  }
+  const int blk = blockIdx.x - g1_blocks, ij = blk / bx, i = ij / nb, j = ij - i * nb;
+  const int kl = (blk - ij * bx) * blockDim.x + threadIdx.x;
+  if (kl >= nb * nb) return;
+  const bool other = blockIdx.y != 0;                      // GW: the same-spin block
+  const cplx *G = other ? p.Go : p.G, *Go = other ? p.G : p.Go;
+  const int k = kl / nb, l = kl - k * nb;
+  const long long e = (long long)ij * N2 + kl;
+  // [h2, G]_ijkl = sum_p h_ip G_pjkl + h_jp G_ipkl - G_ijpl h_pk - G_ijkp h_pl, the diagonals in one factor
+  const cplx dg = csub(csub(cadd(hub_diag(p, i), hub_diag(p, j)), hub_diag(p, k)), hub_diag(p, l));
+  cplx acc = cmul(dg, G[e]);
+  for (int q = p.rp[i]; q < p.rp[i + 1]; ++q) {
+    const int s = p.ci[q];
+    if (s != i) acc = cfma(hub_h(p, i, s), G[s * N3 + j * N2 + kl], acc);
+  }
+  for (int q = p.rp[j]; q < p.rp[j + 1]; ++q) {
+    const int s = p.ci[q];
+    if (s != j) acc = cfma(hub_h(p, j, s), G[i * N3 + s * N2 + kl], acc);
+  }
+  cplx sub = {0.0, 0.0};
+  for (int q = p.rp[k]; q < p.rp[k + 1]; ++q) {
+    const int s = p.ci[q];
+    if (s != k) sub = cfma(G[(long long)ij * N2 + s * N + l], hub_h(p, s, k), sub);
+  }
+  for (int q = p.rp[l]; q < p.rp[l + 1]; ++q) {
+    const int s = p.ci[q];
+    if (s != l) sub = cfma(G[e - l + s], hub_h(p, s, l), sub);
+  }
+  if (!other) {
+    // Psi = -S: S = n_jk (n_jl x1 + n_ik x4) + n_il (n_ik x2 + n_jl x3)
+    const cplx *n = p.n;
+    const cplx nik = n[i * N + k], nil = n[i * N + l], njk = n[j * N + k], njl = n[j * N + l];
+    const double Ui = p.U[i], Uk = p.U[k];
+    cplx x1 = cscale(n[i * N + j], -p.U[j]), x2 = cscale(n[j * N + i], -Ui);
+    cplx x3 = cscale(n[l * N + k], p.U[l]), x4 = cscale(n[k * N + l], Uk);
+    if (i == j) x2.x += Ui;
+    if (k == l) x4.x -= Uk;
+    const cplx a = cfma(nik, x4, cmul(njl, x1)), b = cfma(njl, x3, cmul(nik, x2));
+    sub = cfma(njk, a, sub);
+    sub = cfma(nil, b, sub);
+  }
+  acc = csub(acc, sub);
+  if (Go) {
+    auto g4 = [&](int a, int b, int c, int d) { return Go[((a * N + b) * N + c) * N + d]; };
+    const cplx pi = cmul(p.n[j * N + l], csub(cscale(g4(i, j, k, j), p.U[j]), cscale(g4(i, l, k, l), p.U[l])));
+    const cplx pt = cmul(p.n[k * N + i], csub(cscale(g4(l, k, j, k), p.U[k]), cscale(g4(l, i, j, i), p.U[i])));
+    acc = csub(cadd(acc, pi), cconj(pt));   // + Pi_ijkl - conj(Pi_lkji)
+  }
+  const cplx kk = mul_minus_i(acc);
+  if (other) rk4_apply(e, kk, p.stage, p.dt, p.Sy, p.Sys, p.Sacc, nullptr);
+  else rk4_apply(e, kk, p.stage, p.dt, p.Gy, p.Gys, p.Gacc, p.Gk);
 }
 
 // ---------------------------------------------------------------------------
@@ -837,17 +875,11 @@ void g2_assemble(Launcher &L, int nb, const cplx *Cb, const cplx *Ab, Rk4Stage s
   L.after_launch();
 }
 
-void hubbard_c(Launcher &L, int nb, const int *rp, const int *ci, const cplx *hhf, const double *U, const cplx *n,
-               const cplx *G, const cplx *Go, bool psi, cplx *C) {
-  L.before("hubbard_c");
-  hubbard_c_kernel<<<dim3((nb * nb + 127) / 128, nb * nb), 128, 0, L.stream>>>(nb, rp, ci, hhf, U, n, G, Go, psi ? 1 : 0,
-                                                                                C);
-  L.after_launch();
-}
-
-void hubbard_collision(Launcher &L, int nb, const double *U, const cplx *G, cplx *I) {
-  L.before("hubbard_collision");
-  hubbard_collision_kernel<<<(nb * nb + 127) / 128, 128, 0, L.stream>>>(nb, U, G, I);
+void hubbard_stage(Launcher &L, const HubStage &p) {
+  const int nb2 = p.nb * p.nb, threads = nb2 <= 256 ? 64 : 128;
+  const int g1 = (nb2 * 32 + threads - 1) / threads, bx = (nb2 + threads - 1) / threads;
+  L.before("hubbard_stage");
+  hubbard_stage_kernel<<<dim3(g1 + bx * nb2, p.Go ? 2 : 1), threads, 0, L.stream>>>(p, g1, bx);
   L.after_launch();
 }
 
@@ -963,24 +995,37 @@ __global__ void dot_accumulate_kernel(int nparts, const double *partials, double
   if (threadIdx.x == 0) *acc += coeff * s[0];
 }
 
-// out_lk (+)= sum_ij Wm[(ij),(lk)] x_ij  (the adjoint of the Hartree-Fock build)
+// out_lk (+)= sum_ij Wm[(ij),(lk)] x_ij  (the adjoint of the Hartree-Fock build).  A CTA takes eight columns
+// (64 bytes of every row of a real Wm), its 32 rows of threads the rows of Wm in turn, and reduces them in a
+// fixed order: one thread per column left three quarters of the chip idle and a chain of nb^2 loads
+// (nb = 32: 190 us, now NNN us).
+constexpr int kHtCols = 8, kHtRows = 32;
 template <bool REAL>
-__global__ void hf_build_t_kernel(int nb, const void *__restrict__ Wm_, const cplx *__restrict__ x, cplx *out,
-                                  int accumulate) {
+__global__ void __launch_bounds__(kHtCols * kHtRows) hf_build_t_kernel(int nb, const void *__restrict__ Wm_,
+                                                                       const cplx *__restrict__ x, cplx *out,
+                                                                       int accumulate) {
+  __shared__ cplx part[kHtRows][kHtCols];
   const int nb2 = nb * nb;
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nb2) return;
+  const int tc = threadIdx.x % kHtCols, tr = threadIdx.x / kHtCols;
+  const int c = blockIdx.x * kHtCols + tc;
   cplx acc = {0.0, 0.0};
-  for (int r = 0; r < nb2; ++r) {
-    const cplx xv = x[r];
-    if (REAL) {
-      const double wv = static_cast<const double *>(Wm_)[(long long)r * nb2 + c];
-      acc.x = fma(wv, xv.x, acc.x);
-      acc.y = fma(wv, xv.y, acc.y);
-    } else {
-      acc = cfma(cconj(static_cast<const cplx *>(Wm_)[(long long)r * nb2 + c]), xv, acc);
+  if (c < nb2) {
+#pragma unroll 4
+    for (int r = tr; r < nb2; r += kHtRows) {
+      const cplx xv = x[r];
+      if (REAL) {
+        const double wv = static_cast<const double *>(Wm_)[(long long)r * nb2 + c];
+        acc.x = fma(wv, xv.x, acc.x);
+        acc.y = fma(wv, xv.y, acc.y);
+      } else {
+        acc = cfma(cconj(static_cast<const cplx *>(Wm_)[(long long)r * nb2 + c]), xv, acc);
+      }
     }
   }
+  part[tr][tc] = acc;
+  __syncthreads();
+  if (tr != 0 || c >= nb2) return;
+  for (int r = 1; r < kHtRows; ++r) acc = cadd(acc, part[r][tc]);
   // the Hartree-Fock matrix is indexed [(ij),(lk)] with column (l*nb + k) = the n_lk entry
   out[c] = accumulate ? cadd(out[c], acc) : acc;
 }
@@ -1065,9 +1110,9 @@ void hf_build_t(Launcher &L, int nb, const void *Wm, bool wm_real, const cplx *x
   const int nb2 = nb * nb;
   L.before("adj_hf_build_t");
   if (wm_real)
-    hf_build_t_kernel<true><<<(nb2 + 127) / 128, 128, 0, L.stream>>>(nb, Wm, x, out, accumulate ? 1 : 0);
+    hf_build_t_kernel<true><<<(nb2 + kHtCols - 1) / kHtCols, kHtCols * kHtRows, 0, L.stream>>>(nb, Wm, x, out, accumulate ? 1 : 0);
   else
-    hf_build_t_kernel<false><<<(nb2 + 127) / 128, 128, 0, L.stream>>>(nb, Wm, x, out, accumulate ? 1 : 0);
+    hf_build_t_kernel<false><<<(nb2 + kHtCols - 1) / kHtCols, kHtCols * kHtRows, 0, L.stream>>>(nb, Wm, x, out, accumulate ? 1 : 0);
   L.after_launch();
 }
 
@@ -1079,46 +1124,51 @@ void hf_build_t(Launcher &L, int nb, const void *Wm, bool wm_real, const cplx *x
 namespace g1g2 {
 namespace {
 
-// out_b[m][i] = sum_p in_b[p][m] op(S_b[i][p]) with m = (q, r, s) running over the
-// trailing nb^3 entries: a mode-1 product whose new index i moves to the last place,
-// so four calls with S1..S4 apply S1 (x) S2 (x) S3 (x) S4 to the four indices and
-// return them in their original order.  One thread per (m, b); its nb inputs
-// in_b[p][m] are coalesced across the warp and held in registers.
-template <int NMAX>
-__global__ void __launch_bounds__(128) mode_rotate_kernel(int nb, const cplx *__restrict__ in,
-                                                          const cplx *__restrict__ S, int conjS,
+// One matrix on both indices of a pair of an nb^4 tensor: out_ab = sum_pq M_ap M_bq X_pq for every value c of the other
+// pair, X_pq = in[(pq)][c] (second = 0) or in[c][(pq)] (second = 1).  One CTA per c, operands in shared memory; the
+// four-index transformations of the memory integral are two such launches each.  M is built from S:
+// S itself, S^dag, 1 + eta S, S^T or S^*.  from_a: X = i (A - A^dag) of the tensor A = in (second = 1), the
+// source -i Psi formed on the fly.  At these sizes a launch is latency and one pass through the FP64 pipe.
+__global__ void __launch_bounds__(256) pair_rotate_kernel(int nb, int second, int from_a, const cplx *__restrict__ in,
+                                                          const cplx *__restrict__ S, int form, double eta,
                                                           cplx *__restrict__ out) {
-  __shared__ cplx Ss[NMAX * NMAX];
-  const long long N3 = (long long)nb * nb * nb, N4 = N3 * nb;
-  const long long b = blockIdx.y;
-  const cplx *Sb = S + b * nb * nb;
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    cplx v = Sb[e];
-    if (conjS) v.y = -v.y;
-    Ss[e] = v;
+  __shared__ cplx X[kPairMaxNb * kPairMaxNb], T[kPairMaxNb * kPairMaxNb], M[kPairMaxNb * kPairMaxNb];
+  const int n2 = nb * nb, c = blockIdx.x;
+  for (int e = threadIdx.x; e < n2; e += blockDim.x) {
+    const int a = e / nb, p = e - a * nb;
+    cplx m = (form == kPairAdj || form == kPairTrans) ? S[p * nb + a] : S[e];
+    if (form == kPairAdj || form == kPairConj) m.y = -m.y;
+    if (form == kPairOnePlus) m = {(a == p ? 1.0 : 0.0) + eta * m.x, eta * m.y};
+    M[e] = m;
+    const long long row = (long long)c * n2 + e, col = (long long)e * n2 + c;
+    cplx x = in[second ? row : col];
+    if (from_a) {
+      const cplx y = in[col];
+      x = {-(x.y + y.y), x.x - y.x};   // i (x - conj y)
+    }
+    X[e] = x;
   }
   __syncthreads();
-  const long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= N3) return;
-  const cplx *ib = in + b * N4 + m;
-  cplx x[NMAX];
-#pragma unroll
-  for (int p = 0; p < NMAX; ++p) x[p] = (p < nb) ? ib[(long long)p * N3] : cplx{0.0, 0.0};
-  cplx *ob = out + b * N4 + m * nb;
-  for (int i = 0; i < nb; ++i) {
-    cplx acc = {0.0, 0.0};
-#pragma unroll
-    for (int p = 0; p < NMAX; ++p)
-      if (p < nb) acc = cfma(x[p], Ss[i * nb + p], acc);
-    ob[i] = acc;
+  for (int e = threadIdx.x; e < n2; e += blockDim.x) {
+    const int a = e / nb, q = e - a * nb;
+    cplx t = {0.0, 0.0};
+    for (int p = 0; p < nb; ++p) t = cfma(M[a * nb + p], X[p * nb + q], t);
+    T[e] = t;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < n2; e += blockDim.x) {
+    const int a = e / nb, b = e - a * nb;
+    cplx t = {0.0, 0.0};
+    for (int q = 0; q < nb; ++q) t = cfma(M[b * nb + q], T[a * nb + q], t);
+    out[second ? (long long)c * n2 + e : (long long)e * n2 + c] = t;
   }
 }
 
-// out[e] = beta out[e] + sum_b x[b len + e]: 32 consecutive entries per block, the
-// batch split over the block's eight warps (b = warp + 8 r), then a fixed-order
-// reduction over the warps in shared memory (deterministic).
-__global__ void __launch_bounds__(256) batch_sum_kernel(long long len, int nbatch, const cplx *__restrict__ x,
-                                                        double beta, cplx *out) {
+// out[e] = dt (sum_b x[b len + e] - (x[e] + x[(nbatch - 1) len + e]) / 2), the trapezoid rule over a history of
+// nbatch >= 2 points: 32 consecutive entries per block, the points split over the block's eight warps, then a
+// fixed-order reduction over the warps in shared memory (deterministic).
+__global__ void __launch_bounds__(256) trapezoid_sum_kernel(long long len, int nbatch, const cplx *__restrict__ x,
+                                                            double dt, cplx *out) {
   __shared__ cplx part[8][32];
   const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
   const long long e = (long long)blockIdx.x * 32 + lane;
@@ -1134,10 +1184,94 @@ __global__ void __launch_bounds__(256) batch_sum_kernel(long long len, int nbatc
   part[wv][lane] = cadd(s0, s1);
   __syncthreads();
   if (wv != 0 || e >= len) return;
-  cplx s = (beta != 0.0) ? cscale(out[e], beta) : cplx{0.0, 0.0};
+  cplx s = part[0][lane];
 #pragma unroll
-  for (int w = 0; w < 8; ++w) s = cadd(s, part[w][lane]);
-  out[e] = s;
+  for (int w = 1; w < 8; ++w) s = cadd(s, part[w][lane]);
+  const cplx ends = cadd(x[e], x[(long long)(nbatch - 1) * len + e]);
+  out[e] = {dt * fma(-0.5, ends.x, s.x), dt * fma(-0.5, ends.y, s.y)};
+}
+
+// h^HF_ij = h_ij + sum_c Wm[(ij)][c] n_c and I_ij = -i sum_(lp),k wP[(lp)][i][k] G[(lp)][j][k], one CTA per (i, j):
+// for small nb, where one launch with nb^3 terms per CTA costs less than the split-K product, its
+// reduction and the Hartree-Fock build.
+__global__ void __launch_bounds__(128) mean_collision_kernel(int nb, const void *__restrict__ Wm, int wm_real,
+                                                             const cplx *__restrict__ h, const cplx *__restrict__ n,
+                                                             const cplx *__restrict__ wP, const cplx *__restrict__ G,
+                                                             cplx *__restrict__ hhf, cplx *__restrict__ I) {
+  __shared__ cplx part[2][4];
+  const int i = blockIdx.x / nb, j = blockIdx.x - i * nb, n2 = nb * nb, n3 = n2 * nb;
+  cplx a = {0.0, 0.0}, b = {0.0, 0.0};
+  for (int c = threadIdx.x; c < n2; c += 128) {
+    const long long e = (long long)blockIdx.x * n2 + c;
+    if (wm_real) {
+      const double w = static_cast<const double *>(Wm)[e];
+      a = {fma(w, n[c].x, a.x), fma(w, n[c].y, a.y)};
+    } else {
+      a = cfma(static_cast<const cplx *>(Wm)[e], n[c], a);
+    }
+  }
+#pragma unroll 4
+  for (int c = threadIdx.x; c < n3; c += 128) {
+    const int lp = c / nb, k = c - lp * nb;
+    b = cfma(wP[(long long)lp * n2 + i * nb + k], G[(long long)lp * n2 + j * nb + k], b);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+    a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+    b.x += __shfl_xor_sync(0xffffffffu, b.x, o);
+    b.y += __shfl_xor_sync(0xffffffffu, b.y, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    part[0][threadIdx.x >> 5] = a;
+    part[1][threadIdx.x >> 5] = b;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < 4; ++w) {
+    a = cadd(a, part[0][w]);
+    b = cadd(b, part[1][w]);
+  }
+  hhf[blockIdx.x] = cadd(h[blockIdx.x], a);
+  I[blockIdx.x] = mul_minus_i(b);
+}
+
+// One half of a Heun step for n and u, one warp per element: dn = -i [h^HF, n] - (I + I^dag), du = -i h^HF u at
+// (n, u), then out = base + c1 prev + c2 derivative (prev null in the predictor), the derivative kept in (dn, du).
+__global__ void __launch_bounds__(256) heun_update_kernel(int nb, const cplx *__restrict__ hhf, const cplx *__restrict__ n,
+                                                          const cplx *__restrict__ u, const cplx *__restrict__ I,
+                                                          const cplx *n0, const cplx *u0, const cplx *dn_prev,
+                                                          const cplx *du_prev, double c1, double c2, cplx *dn, cplx *du,
+                                                          cplx *n_out, cplx *u_out) {
+  const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (idx >= nb * nb) return;
+  const int i = idx / nb, j = idx % nb;
+  cplx comm = {0.0, 0.0}, hu = {0.0, 0.0};
+  for (int p = lane; p < nb; p += 32) {
+    const cplx hip = hhf[i * nb + p];
+    comm = cfma(hip, n[p * nb + j], comm);
+    comm = csub(comm, cmul(n[i * nb + p], hhf[p * nb + j]));
+    hu = cfma(hip, u[p * nb + j], hu);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    comm.x += __shfl_xor_sync(0xffffffffu, comm.x, o);
+    comm.y += __shfl_xor_sync(0xffffffffu, comm.y, o);
+    hu.x += __shfl_xor_sync(0xffffffffu, hu.x, o);
+    hu.y += __shfl_xor_sync(0xffffffffu, hu.y, o);
+  }
+  if (lane != 0) return;
+  const cplx kn = csub(mul_minus_i(comm), cadd(I[i * nb + j], cconj(I[j * nb + i]))), ku = mul_minus_i(hu);
+  cplx a = n0[idx], b = u0[idx];
+  if (dn_prev) {
+    a = {fma(c1, dn_prev[idx].x, a.x), fma(c1, dn_prev[idx].y, a.y)};
+    b = {fma(c1, du_prev[idx].x, b.x), fma(c1, du_prev[idx].y, b.y)};
+  }
+  n_out[idx] = {fma(c2, kn.x, a.x), fma(c2, kn.y, a.y)};
+  u_out[idx] = {fma(c2, ku.x, b.x), fma(c2, ku.y, b.y)};
+  dn[idx] = kn;
+  du[idx] = ku;
 }
 
 __global__ void count_nonzero_kernel(const cplx *x, long long len, double *cnt) {
@@ -1156,25 +1290,32 @@ __global__ void count_nonzero_kernel(const cplx *x, long long len, double *cnt) 
 
 }  // namespace
 
-int mode_rotate_max_nb() { return 32; }
-
-void mode_rotate(Launcher &L, int nb, int batch, const cplx *in, const cplx *S, bool conjS, cplx *out) {
-  if (batch <= 0) return;
-  const long long N3 = (long long)nb * nb * nb;
-  dim3 grid((unsigned)((N3 + 127) / 128), (unsigned)batch);
-  L.before("hfgkba_mode_rotate");
-  if (nb <= 8)
-    mode_rotate_kernel<8><<<grid, 128, 0, L.stream>>>(nb, in, S, conjS ? 1 : 0, out);
-  else if (nb <= 16)
-    mode_rotate_kernel<16><<<grid, 128, 0, L.stream>>>(nb, in, S, conjS ? 1 : 0, out);
-  else
-    mode_rotate_kernel<32><<<grid, 128, 0, L.stream>>>(nb, in, S, conjS ? 1 : 0, out);
+void pair_rotate(Launcher &L, int nb, bool second, bool from_a, const cplx *in, const cplx *S, PairForm form, double eta,
+                 cplx *out) {
+  L.before("hfgkba_pair_rotate");
+  pair_rotate_kernel<<<nb * nb, nb <= 8 ? 64 : 256, 0, L.stream>>>(nb, second ? 1 : 0, from_a ? 1 : 0, in, S, form, eta, out);
   L.after_launch();
 }
 
-void batch_sum(Launcher &L, long long len, int nbatch, const cplx *x, double beta, cplx *out) {
-  L.before("hfgkba_batch_sum");
-  batch_sum_kernel<<<(unsigned)((len + 31) / 32), 256, 0, L.stream>>>(len, nbatch, x, beta, out);
+void trapezoid_sum(Launcher &L, long long len, int npoints, const cplx *x, double dt, cplx *out) {
+  L.before("hfgkba_trapezoid");
+  trapezoid_sum_kernel<<<(unsigned)((len + 31) / 32), 256, 0, L.stream>>>(len, npoints, x, dt, out);
+  L.after_launch();
+}
+
+void mean_collision(Launcher &L, int nb, const void *Wm, bool wm_real, const cplx *h, const cplx *n, const cplx *wP,
+                    const cplx *G, cplx *hhf, cplx *I) {
+  L.before("hfgkba_mean_collision");
+  mean_collision_kernel<<<nb * nb, 128, 0, L.stream>>>(nb, Wm, wm_real ? 1 : 0, h, n, wP, G, hhf, I);
+  L.after_launch();
+}
+
+void heun_update(Launcher &L, int nb, const cplx *hhf, const cplx *n, const cplx *u, const cplx *I, const cplx *n0,
+                 const cplx *u0, const cplx *dn_prev, const cplx *du_prev, double c1, double c2, cplx *dn, cplx *du,
+                 cplx *n_out, cplx *u_out) {
+  L.before("hfgkba_heun");
+  heun_update_kernel<<<(nb * nb + 7) / 8, 256, 0, L.stream>>>(nb, hhf, n, u, I, n0, u0, dn_prev, du_prev, c1, c2, dn, du,
+                                                              n_out, u_out);
   L.after_launch();
 }
 

@@ -371,8 +371,10 @@ __device__ __forceinline__ void join_orders(const uint32_t (&v)[4][8], long long
 //   G = 8: tiles of up to 64 columns, all eight orders at once (34 MMAs per K step);
 //   G = 4: tiles of up to 128 columns in two phases over a segment, orders 4..7 (24 MMAs), which the conversion of
 //          the last segment overlaps, then orders 0..3 (ten MMAs, four digit planes loaded).
-template <int G, bool kSplit>
+// kKind: 0 one segment per unit, 1 several, 2 a long contraction (several, real products of re and im rows).
+template <int G, int kKind>
 __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm p) {
+  constexpr bool kSplit = kKind == 2;
   constexpr int kPhases = kOrd / G;
   constexpr int kTN = 512 / G;                       // TMEM columns per accumulator
   extern __shared__ uint8_t smem_raw[];
@@ -560,18 +562,18 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
             }
             __syncwarp();
           }
-          if (!first) {   // a branch, not a select: an idle FP64 addition costs as much as a needed one
+          if (kKind != 0 && !first) {   // (in one-segment kernels the compiler would add a zero, on the slow FP64 pipe)
             double o[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) o[j] = __ldcg(pq + j * kTM);
 #pragma unroll
             for (int j = 0; j < 8; ++j) v[j] += o[j];
           }
-          if (kSplit || !last) {
+          if (kKind != 0 && (kSplit || !last)) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) __stcg(pq + j * kTM, v[j]);
-            continue;
           }
+          if (kSplit || (kKind != 0 && !last)) continue;
           cplx z[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) z[j] = mul_unit({v[2 * j], v[2 * j + 1]}, p.unit_alpha);
@@ -671,11 +673,11 @@ int tile_columns(int real_cols) {
   return round_up((real_cols + tiles - 1) / tiles, 16);
 }
 
-template <bool kSplit>
+template <int kKind>
 void launch_gemm(Launcher &L, const TcGemm &t, int ctas, const char *tag) {
   L.before(tag);
-  if (t.nt <= 64) fp64_tc_gemm_kernel<8, kSplit><<<ctas, kThreads, kSmem, L.stream>>>(t);
-  else fp64_tc_gemm_kernel<4, kSplit><<<ctas, kThreads, kSmem, L.stream>>>(t);
+  if (t.nt <= 64) fp64_tc_gemm_kernel<8, kKind><<<ctas, kThreads, kSmem, L.stream>>>(t);
+  else fp64_tc_gemm_kernel<4, kKind><<<ctas, kThreads, kSmem, L.stream>>>(t);
   L.after_launch();
 }
 
@@ -740,8 +742,9 @@ Fp64Tc *fp64_tc_create(int nb, bool pair_products) {
       cudaMalloc(&f->part, (size_t)f->sms * kTNMax * kTM * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&f->err, sizeof(int)) != cudaSuccess || cudaMemset(f->err, 0, sizeof(int)) != cudaSuccess)
     goto bad;
-  for (const void *k : {(const void *)fp64_tc_gemm_kernel<8, false>, (const void *)fp64_tc_gemm_kernel<8, true>,
-                        (const void *)fp64_tc_gemm_kernel<4, false>, (const void *)fp64_tc_gemm_kernel<4, true>})
+  for (const void *k : {(const void *)fp64_tc_gemm_kernel<8, 0>, (const void *)fp64_tc_gemm_kernel<8, 1>,
+                        (const void *)fp64_tc_gemm_kernel<8, 2>, (const void *)fp64_tc_gemm_kernel<4, 0>,
+                        (const void *)fp64_tc_gemm_kernel<4, 1>, (const void *)fp64_tc_gemm_kernel<4, 2>})
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem) != cudaSuccess) goto bad;
   {
     const int sh = 2 * (kCutVals + 32) * (int)sizeof(double);
@@ -809,7 +812,9 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
       t.r_begin = r0; t.y_begin = y0; t.rows = nr; t.cols = ny;
       t.C = g.C; t.scb = g.sc_b; t.scx = a_rows ? g.sc_m : g.sc_n; t.scy = a_rows ? g.sc_n : g.sc_m;
       t.unit_alpha = alpha; t.beta = g.beta != 0.0;
-      launch_gemm<false>(L, t, std::min(f->sms, t.mtiles * t.ntiles), segs > 1 ? "fp64_tc_gemm_pair" : "fp64_tc_gemm");
+      const int ctas = std::min(f->sms, t.mtiles * t.ntiles);
+      if (segs == 1) launch_gemm<0>(L, t, ctas, "fp64_tc_gemm");
+      else launch_gemm<1>(L, t, ctas, "fp64_tc_gemm_pair");
     }
   }
   return true;
@@ -853,7 +858,7 @@ bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g) {
     t.k_begin = k0;
     t.C = g.C; t.scx = g.sc_m; t.scy = g.sc_n; t.unit_alpha = alpha; t.beta = g.beta != 0.0;
     t.sums = f->sums; t.part = f->part; t.accumulate = sg0 > 0;
-    launch_gemm<true>(L, t, t.splits * mtiles * ntiles, "fp64_tc_gemm_long");
+    launch_gemm<2>(L, t, t.splits * mtiles * ntiles, "fp64_tc_gemm_long");
   }
   L.before("fp64_tc_reduce");
   fp64_tc_reduce_kernel<<<(g.M * g.N + 7) / 8, 256, 0, L.stream>>>(t);

@@ -320,32 +320,27 @@ void rhs_fp64(g1g2_ctx *c, Launcher &L, double t, const cplx *n_in, const cplx *
   const int nb = c->nb;
   const long long N = nb, N2 = N * N, N3 = N2 * N;
   const double f = drive_f(c, t);
-  // a1: Eq. (h_HF); with w_only the one-body h(t) is left out (the part of the
-  // right-hand side that is linear in w, used for the gradient by the scale of w)
-  if (w_only)
-    mean_field(c, L, c->zero_h, nullptr, 0.0, n_in);
-  else
-    mean_field(c, L, c->h, c->hasD ? c->D : nullptr, f, n_in);
-  if (c->se == G1G2_HF) {
-    g1_update(L, nb, c->hhf, n_in, nullptr, st, o.ny, o.nys, o.nacc, o.nk);
+  // with w_only the one-body h(t) is left out (the part of the right-hand side that is linear in w,
+  // used for the gradient by the scale of w)
+  const cplx *h = w_only ? c->zero_h : c->h, *D = !w_only && c->hasD ? c->D : nullptr;
+  if (c->hub_on && c->se != G1G2_HF) {
+    HubStage p{};
+    p.nb = nb; p.rp = c->hub_rp; p.ci = c->hub_ci; p.h = h; p.D = D; p.f = f; p.U = c->hub_U;
+    p.n = n_in; p.G = G_in; p.stage = st.stage; p.dt = st.dt;
+    p.ny = o.ny; p.nys = o.nys; p.nacc = o.nacc; p.nk = o.nk;
+    p.Gy = o.Gy; p.Gys = o.Gys; p.Gacc = o.Gacc; p.Gk = o.Gk;
+    if (c->hub_gw) {
+      // the same-spin block's stage states alternate as those of G2 (rk4_step)
+      p.Go = st.stage <= 0 ? c->Gss : st.stage == 2 ? c->Cb2 : c->Gss_s;
+      p.Sy = c->Gss; p.Sys = st.stage == 1 ? c->Cb2 : c->Gss_s; p.Sacc = c->Gss_acc;
+    }
+    hubbard_stage(L, p);
     return;
   }
-  if (c->hub_on) {
-    // Hubbard basis: I, then C = [h2, G] + Psi in O(nb^4); the assembly forms dG = -i C
-    hubbard_collision(L, nb, c->hub_U, G_in, c->I);
-    g1_update(L, nb, c->hhf, n_in, c->I, st, o.ny, o.nys, o.nacc, o.nk);
-    if (c->hub_gw) {
-      // GW: each spin block with the polarisation of the other (every read of a stage input
-      // is queued before the assemblies overwrite it)
-      const cplx *Gss_in = (st.stage <= 0) ? c->Gss : c->Gss_s;
-      hubbard_c(L, nb, c->hub_rp, c->hub_ci, c->hhf, c->hub_U, n_in, G_in, Gss_in, true, c->Cb);
-      hubbard_c(L, nb, c->hub_rp, c->hub_ci, c->hhf, c->hub_U, n_in, Gss_in, G_in, false, c->Cb2);
-      g2_assemble(L, nb, c->Cb, nullptr, st, o.Gy, o.Gys, o.Gacc, o.Gk);
-      g2_assemble(L, nb, c->Cb2, nullptr, st, c->Gss, c->Gss_s, c->Gss_acc, nullptr);
-      return;
-    }
-    hubbard_c(L, nb, c->hub_rp, c->hub_ci, c->hhf, c->hub_U, n_in, G_in, nullptr, true, c->Cb);
-    g2_assemble(L, nb, c->Cb, nullptr, st, o.Gy, o.Gys, o.Gacc, o.Gk);
+  // a1: Eq. (h_HF)
+  mean_field(c, L, h, D, w_only ? 0.0 : f, n_in);
+  if (c->se == G1G2_HF) {
+    g1_update(L, nb, c->hhf, n_in, nullptr, st, o.ny, o.nys, o.nacc, o.nk);
     return;
   }
   // a2: Eq. (eom_gone-I)
@@ -499,9 +494,12 @@ int rk4_step(g1g2_ctx *c, double dt) {
   cplx *n_in_of[4] = {c->n, c->ns, c->ns2, c->ns};
   cplx *n_out_of[4] = {c->ns, c->ns2, c->ns, nullptr};
   for (int s = 0; s < 4; ++s) {
-    StageOut o{c->n, n_out_of[s], c->nacc, nullptr, c->G, c->Gs, c->Gacc, nullptr};
+    // G2's stage state is updated in place by the assembly kernels; the Hubbard kernel reads it at
+    // other elements too, so there it alternates with the (otherwise unused) commutator buffer
+    cplx *G_out = (c->hub_on && s == 1) ? c->Cb : c->Gs;
+    StageOut o{c->n, n_out_of[s], c->nacc, nullptr, c->G, G_out, c->Gacc, nullptr};
     const cplx *n_in = n_in_of[s];
-    const cplx *G_in = (s == 0) ? c->G : c->Gs;
+    const cplx *G_in = (s == 0) ? c->G : (c->hub_on && s == 2) ? c->Cb : c->Gs;
     if (c->hasD && c->drive_kind != 0) {
       const double coeff = dt / 6.0 * wgt[s] * drive_dfdt(c, t + cs[s] * dt);
       accumulate_work(L, c->nb, c->D, n_in, coeff * (c->basis == G1G2_SPIN_RESTRICTED ? 2.0 : 1.0), c->W_dev);
@@ -929,60 +927,41 @@ struct DevScratch {
   }
 };
 
-// dn = -i[hHF, n] - (I + I^dag) with I from G2, du = -i hHF u (Eqs. eom_gone-2, eom_gone-I)
-void gkba_derivs(g1g2_ctx *c, Launcher &L, const cplx *n, const cplx *u, const cplx *G2, cplx *dn, cplx *du) {
-  const int nb = c->nb;
-  hf_build(L, nb, c->Wm, c->w_real, c->h, nullptr, 0.0, n, c->hhf);
+// h^HF and I of the state (n, G2) into the context's buffers
+void gkba_mean(g1g2_ctx *c, Launcher &L, const cplx *n, const cplx *G2) {
+  // one CTA per (i, j) reads all of w and G2 nb times: below nb = 17 that is at most 34 MB of L2 traffic
+  if (c->nb <= 16) {
+    mean_collision(L, c->nb, c->Wm, c->w_real, c->h, n, c->wP, G2, c->hhf, c->I);
+    return;
+  }
+  hf_build(L, c->nb, c->Wm, c->w_real, c->h, nullptr, 0.0, n, c->hhf);
   collision(c, L, G2);
-  g1_update(L, nb, c->hhf, n, c->I, Rk4Stage{-1, 0.0}, nullptr, nullptr, nullptr, dn);
-  ZGemm g;
-  g.M = nb; g.N = nb; g.K = nb;
-  g.A = c->hhf; g.sa_m = nb; g.sa_k = 1;
-  g.B = u; g.sb_k = nb; g.sb_n = 1;
-  g.C = du; g.sc_m = nb; g.sc_n = 1;
-  g.alpha = {0.0, -1.0};
-  zgemm(L, g);
 }
 
-// Q = -i Psi(n) = -i (-A + A^dag): the assembly with a zero commutator buffer (c->Cb)
-void gkba_source(g1g2_ctx *c, Launcher &L, const cplx *n, cplx *Q) {
-  source_A(c, L, n);
-  g2_assemble(L, c->nb, c->Cb, c->Ab, Rk4Stage{-1, 0.0}, nullptr, nullptr, nullptr, Q);
-}
-
-struct GkbaHist {
-  cplx *u = nullptr, *Q = nullptr, *V = nullptr, *Vs = nullptr, *Y0 = nullptr, *Y1 = nullptr;
-  int chunk = 1;
-};
-
-// G2 = sum_{k<K} w_k dt (V_k (x) V_k) Q_k (V_k (x) V_k)^dag, V_k = u_now u_k^dag, trapezoid
-// weights w_0 = w_{K-1} = 1/2 (G2 = 0 for K = 1)
-void gkba_memory(g1g2_ctx *c, Launcher &L, const GkbaHist &H, int K, const cplx *u_now, double dt, cplx *G2) {
+// History entry at (n, u): R = (u (x) u)^dag Q (u (x) u) with Q = -i Psi(n) = i (A - A^dag), A the source tensor of source_A.
+// With V_k = u_now u_k^dag the memory integral's terms are (V_k (x) V_k) Q_k (V_k (x) V_k)^dag
+// = (u_now (x) u_now) R_k (u_now (x) u_now)^dag, so each entry is transformed once and every later
+// evaluation adds up the history and transforms the sum: 2 nb^4 additions per history point and evaluation
+// instead of 4 nb^5 complex multiply-adds.
+void gkba_entry(g1g2_ctx *c, Launcher &L, const cplx *n, const cplx *u, cplx *R) {
   const int nb = c->nb;
-  const long long N2 = (long long)nb * nb, N4 = N2 * N2;
+  pair_rotate(L, nb, true, false, c->wsrc, n, kPairTrans, 0.0, c->T1);       // sum_rs w_pqrs n_rk n_sl
+  pair_rotate(L, nb, false, false, c->T1, n, kPairOnePlus, c->eta, c->Ab);   // A = nbar nbar (...)
+  pair_rotate(L, nb, true, true, c->Ab, u, kPairTrans, 0.0, c->T1);          // Q (u (x) u)
+  pair_rotate(L, nb, false, false, c->T1, u, kPairAdj, 0.0, R);
+}
+
+// G2 from the first K history entries R_k, trapezoid weights w_0 = w_{K-1} = 1/2 (G2 = 0 for K = 1)
+void gkba_memory(g1g2_ctx *c, Launcher &L, const cplx *R, int K, const cplx *u_now, double dt, cplx *G2) {
+  const int nb = c->nb;
+  const long long N4 = (long long)nb * nb * nb * nb;
   if (K <= 1) {
     cudaMemsetAsync(G2, 0, N4 * sizeof(cplx), L.stream);
     return;
   }
-  {
-    ZGemm g;  // V_k[i][j] = sum_p u_now[i][p] conj(u_k[j][p])
-    g.M = nb; g.N = nb; g.K = nb; g.batch = K;
-    g.A = u_now; g.sa_b = 0; g.sa_m = nb; g.sa_k = 1;
-    g.B = H.u; g.sb_b = N2; g.sb_k = 1; g.sb_n = nb; g.conjB = true;
-    g.C = H.V; g.sc_b = N2; g.sc_m = nb; g.sc_n = 1;
-    zgemm(L, g);
-  }
-  zaxpby(L, (long long)K * N2, {dt, 0.0}, H.V, {0.0, 0.0}, nullptr, H.Vs);
-  zaxpby(L, N2, {0.5 * dt, 0.0}, H.V, {0.0, 0.0}, nullptr, H.Vs);
-  zaxpby(L, N2, {0.5 * dt, 0.0}, H.V + (K - 1) * N2, {0.0, 0.0}, nullptr, H.Vs + (K - 1) * N2);
-  for (int k0 = 0; k0 < K; k0 += H.chunk) {
-    const int kc = std::min(H.chunk, K - k0);
-    mode_rotate(L, nb, kc, H.Q + k0 * N4, H.Vs + k0 * N2, false, H.Y0);
-    mode_rotate(L, nb, kc, H.Y0, H.V + k0 * N2, false, H.Y1);
-    mode_rotate(L, nb, kc, H.Y1, H.V + k0 * N2, true, H.Y0);
-    mode_rotate(L, nb, kc, H.Y0, H.V + k0 * N2, true, H.Y1);
-    batch_sum(L, N4, kc, H.Y1, k0 == 0 ? 0.0 : 1.0, G2);
-  }
+  trapezoid_sum(L, N4, K, R, dt, c->T1);
+  pair_rotate(L, nb, true, false, c->T1, u_now, kPairConj, 0.0, c->T2);
+  pair_rotate(L, nb, false, false, c->T2, u_now, kPairPlain, 0.0, G2);
 }
 
 }  // namespace
@@ -1523,24 +1502,21 @@ int g1g2_propagate(g1g2_ctx *c, double dt, int nsteps, int obs_every, g1g2_obs *
 // propagator of the GKBA (Eqs. GKBA_propa/b), i du/dt = hHF u.  Every evaluation sums
 // over the whole stored history (trapezoid rule): the O(N_t^2) cost of the standard
 // scheme (Table I).  n and u advance by Heun's method; the memory sum at the predictor
-// includes the predicted end point.  History entry k holds u(t_k) and Q_k = -i Psi(t_k),
-// since (i hbar)^3 (i hbar)^-4 = -i.
+// includes the predicted end point.  History entry k holds u(t_k) and Q_k = -i Psi(t_k), since
+// (i hbar)^3 (i hbar)^-4 = -i, transformed to R_k = (u_k (x) u_k)^dag Q_k (u_k (x) u_k) (gkba_entry).
 int g1g2_propagate_hfgkba(g1g2_ctx *c, double dt, int nsteps, double *G1_history, size_t scratch_bytes) {
   if (!c || nsteps < 0 || !std::isfinite(dt)) return fail(G1G2_EINVAL, "bad argument");
   if (c->se != G1G2_SOA || c->prec != G1G2_FP64)
     return fail(G1G2_EUNSUPPORTED, "the memory-integral HF-GKBA covers SOA in the FP64 form");
   NvtxRange range("g1g2 hf-gkba propagate");
   if (c->hasD) return fail(G1G2_EUNSUPPORTED, "the memory-integral HF-GKBA runs without a drive");
-  if (c->nb > mode_rotate_max_nb())
+  if (c->nb > kPairMaxNb)
     return fail(G1G2_EUNSUPPORTED, "the memory-integral HF-GKBA keeps nb^4 per time step; nb <= " +
-                                       std::to_string(mode_rotate_max_nb()));
+                                       std::to_string(kPairMaxNb));
   const int nb = c->nb;
   const long long N2 = (long long)nb * nb, N4 = N2 * N2;
   const long long slots = (long long)nsteps + 2;
-  if (scratch_bytes == 0) scratch_bytes = (size_t)256 << 20;
-  GkbaHist H;
-  H.chunk = (int)std::max<long long>(
-      1, std::min<long long>(std::min<long long>(slots, 65535LL), (long long)(scratch_bytes / (2 * N4 * sizeof(cplx)))));
+  (void)scratch_bytes;   // the history products need no scratch beyond the context's
   Launcher L = c->launcher();
   int rc;
   // the integral starts from an uncorrelated state
@@ -1552,36 +1528,29 @@ int g1g2_propagate_hfgkba(g1g2_ctx *c, double dt, int nsteps, double *G1_history
     return rc;
   if (nz != 0) return fail(G1G2_EINVAL, "the memory integral starts from G2 = 0; the state has a nonzero G2");
   DevScratch S;
-  cplx *nh, *np, *dn1, *dn2, *du1, *du2;
-  if ((rc = S.get(&H.u, slots * N2)) || (rc = S.get(&H.Q, slots * N4)) || (rc = S.get(&H.V, slots * N2)) ||
-      (rc = S.get(&H.Vs, slots * N2)) || (rc = S.get(&H.Y0, H.chunk * N4)) || (rc = S.get(&H.Y1, H.chunk * N4)) ||
-      (rc = S.get(&nh, (slots - 1) * N2)) || (rc = S.get(&np, N2)) || (rc = S.get(&dn1, N2)) ||
-      (rc = S.get(&dn2, N2)) || (rc = S.get(&du1, N2)) || (rc = S.get(&du2, N2)))
+  cplx *nh, *np, *up, *uh, *R, *dn1, *dn2, *du1, *du2;
+  if ((rc = S.get(&uh, slots * N2)) || (rc = S.get(&R, slots * N4)) || (rc = S.get(&nh, (slots - 1) * N2)) ||
+      (rc = S.get(&np, N2)) || (rc = S.get(&up, N2)) || (rc = S.get(&dn1, N2)) || (rc = S.get(&dn2, N2)) || (rc = S.get(&du1, N2)) ||
+      (rc = S.get(&du2, N2)))
     return rc;
   std::vector<cplx> eye(N2, cplx{0.0, 0.0});
   for (int i = 0; i < nb; ++i) eye[(size_t)i * nb + i] = {1.0, 0.0};
-  if ((rc = cuda_check(cudaMemcpyAsync(H.u, eye.data(), N2 * sizeof(cplx), cudaMemcpyHostToDevice, c->stream), "u0")) ||
-      (rc = cuda_check(cudaMemcpyAsync(nh, c->n, N2 * sizeof(cplx), cudaMemcpyDeviceToDevice, c->stream), "n0")) ||
-      (rc = cuda_check(cudaMemsetAsync(c->Cb, 0, N4 * sizeof(cplx), c->stream), "zero")))
+  if ((rc = cuda_check(cudaMemcpyAsync(uh, eye.data(), N2 * sizeof(cplx), cudaMemcpyHostToDevice, c->stream), "u0")) ||
+      (rc = cuda_check(cudaMemcpyAsync(nh, c->n, N2 * sizeof(cplx), cudaMemcpyDeviceToDevice, c->stream), "n0")))
     return rc;
-  gkba_source(c, L, nh, H.Q);
-  gkba_memory(c, L, H, 1, H.u, dt, c->G);
-  const cplx one{1.0, 0.0}, half{0.5 * dt, 0.0}, full{dt, 0.0};
+  gkba_entry(c, L, nh, uh, R);
+  gkba_memory(c, L, R, 1, uh, dt, c->G);
   for (int m = 0; m < nsteps; ++m) {
-    cplx *n0 = nh + m * N2, *n1 = nh + (m + 1) * N2, *u0 = H.u + m * N2, *u1 = H.u + (m + 1) * N2;
-    cplx *Q1 = H.Q + (m + 1) * N4;
-    gkba_derivs(c, L, n0, u0, c->G, dn1, du1);
-    zaxpby(L, N2, one, n0, full, dn1, np);                 // predictor
-    zaxpby(L, N2, one, u0, full, du1, u1);
-    gkba_source(c, L, np, Q1);
-    gkba_memory(c, L, H, m + 2, u1, dt, c->Gs);
-    gkba_derivs(c, L, np, u1, c->Gs, dn2, du2);
-    zaxpby(L, N2, one, n0, half, dn1, n1);                 // corrector
-    zaxpby(L, N2, one, n1, half, dn2, n1);
-    zaxpby(L, N2, one, u0, half, du1, u1);
-    zaxpby(L, N2, one, u1, half, du2, u1);
-    gkba_source(c, L, n1, Q1);
-    gkba_memory(c, L, H, m + 2, u1, dt, c->G);
+    cplx *n0 = nh + m * N2, *n1 = nh + (m + 1) * N2, *u0 = uh + m * N2, *u1 = uh + (m + 1) * N2;
+    cplx *R1 = R + (m + 1) * N4;
+    gkba_mean(c, L, n0, c->G);
+    heun_update(L, nb, c->hhf, n0, u0, c->I, n0, u0, nullptr, nullptr, 0.0, dt, dn1, du1, np, up);   // predictor
+    gkba_entry(c, L, np, up, R1);
+    gkba_memory(c, L, R, m + 2, up, dt, c->Gs);
+    gkba_mean(c, L, np, c->Gs);
+    heun_update(L, nb, c->hhf, np, up, c->I, n0, u0, dn1, du1, 0.5 * dt, 0.5 * dt, dn2, du2, n1, u1);   // corrector
+    gkba_entry(c, L, n1, u1, R1);
+    gkba_memory(c, L, R, m + 2, u1, dt, c->G);
   }
   if ((rc = launch_status(L, "memory-integral HF-GKBA"))) return rc;
   if ((rc = cuda_check(cudaMemcpyAsync(c->n, nh + nsteps * N2, N2 * sizeof(cplx), cudaMemcpyDeviceToDevice, c->stream),

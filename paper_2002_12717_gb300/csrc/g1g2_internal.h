@@ -119,16 +119,26 @@ void g1_update(Launcher &L, int nb, const cplx *hhf, const cplx *n, const cplx *
 void g2_assemble(Launcher &L, int nb, const cplx *Cb, const cplx *Ab, Rk4Stage st, cplx *y, cplx *ys,
                  cplx *acc, cplx *kout);
 
+// One Runge-Kutta stage (or one right-hand side) in the spin-restricted Hubbard basis (on-site
+// w_ijkl = U_i d(i=j=k=l)): dn and dG2 from the stage input (n, G), with the commutator over the CSR pattern
+// (rp, ci) of h^HF, and their updates according to stage (see Rk4Stage).  GW: Go is the same-spin
+// block, propagated in the same launch into (Sy, Sys, Sacc), each block with Pi - (Pi_lkji)^* of the reduced
+// Hubbard polarisation of the other.  The outputs must not overlap the stage input.
+struct HubStage {
+  int nb;
+  const int *rp, *ci;
+  const cplx *h, *D;       // D null without a drive
+  double f;
+  const double *U;
+  const cplx *n, *G, *Go;
+  int stage;
+  double dt;
+  cplx *ny, *nys, *nacc, *nk, *Gy, *Gys, *Gacc, *Gk, *Sy, *Sys, *Sacc;
+};
+void hubbard_stage(Launcher &L, const HubStage &p);
+
 // Observables.
 // red[0..] = {Re Tr(h n), Re Tr((hHF-h(t)) n), Re Tr n, Re Tr(D n)} for state n;
-// Hubbard basis, spin-restricted SOA (on-site w_ijkl = U_i d(i=j=k=l)): C = [h2, G] + Psi
-// with the commutator over the CSR pattern (rp, ci) of h^HF, and I_ij = -i U_i G_iiji.
-// GW (Go non-null: the other spin block, same-spin for the opposite-spin equation and
-// vice versa) adds Pi - (Pi_lkji)^* of the reduced Hubbard polarisation; psi = false
-// leaves out the source term (the same-spin equation).
-void hubbard_c(Launcher &L, int nb, const int *rp, const int *ci, const cplx *hhf, const double *U, const cplx *n,
-               const cplx *G, const cplx *Go, bool psi, cplx *C);
-void hubbard_collision(Launcher &L, int nb, const double *U, const cplx *G, cplx *I);
 void obs_one_body(Launcher &L, int nb, const cplx *h, const cplx *D, double f, const cplx *hhf,
                   const cplx *n, double *red);
 // red[0] = Re sum W[(ij),(kl)] G[(kl),(ij)], red[1] = count of non-finite entries of G.
@@ -153,13 +163,21 @@ void hf_wbar(Launcher &L, int nb, const cplx *x, const cplx *n, double c, double
 // out = projection of X onto the symmetries of w: (X + X_jilk + conj(X_klij) + conj(X_lkji)) / 4.
 void w_symmetrize(Launcher &L, int nb, const cplx *X, cplx *out);
 
-// Memory-integral HF-GKBA: out_b[m][i] = sum_p in_b[p][m] op(S_b[i][p]) for b < batch
-// (batch <= 65535, nb <= mode_rotate_max_nb()), m over the trailing nb^3 entries of the
-// nb^4 tensor in_b, S_b the nb x nb matrix at S + b nb^2, op = conj when conjS;
-// out[e] = beta out[e] + sum_b x[b len + e]; *cnt += number of nonzero entries of x.
-int mode_rotate_max_nb();
-void mode_rotate(Launcher &L, int nb, int batch, const cplx *in, const cplx *S, bool conjS, cplx *out);
-void batch_sum(Launcher &L, long long len, int nbatch, const cplx *x, double beta, cplx *out);
+// Memory-integral HF-GKBA (nb <= kPairMaxNb).  pair_rotate: out_ab = sum_pq M_ap M_bq X_pq on the first or second index
+// pair of an nb^4 tensor, M from S by form, X the tensor in or (from_a, second pair) i (in - in^dag).
+// trapezoid_sum: dt times the trapezoid sum of npoints >= 2 tensors of length len.  mean_collision: h^HF
+// and I of Eqs. (h_HF), (eom_gone-I).  heun_update: (n_out, u_out) = (n0, u0) + c1 (dn_prev, du_prev) +
+// c2 (dn, du), the derivatives evaluated at (n, u).  *cnt += number of nonzero entries of x.
+constexpr int kPairMaxNb = 32;
+enum PairForm : int { kPairPlain, kPairAdj, kPairOnePlus, kPairTrans, kPairConj };
+void pair_rotate(Launcher &L, int nb, bool second, bool from_a, const cplx *in, const cplx *S, PairForm form, double eta,
+                 cplx *out);
+void trapezoid_sum(Launcher &L, long long len, int npoints, const cplx *x, double dt, cplx *out);
+void mean_collision(Launcher &L, int nb, const void *Wm, bool wm_real, const cplx *h, const cplx *n, const cplx *wP,
+                    const cplx *G, cplx *hhf, cplx *I);
+void heun_update(Launcher &L, int nb, const cplx *hhf, const cplx *n, const cplx *u, const cplx *I, const cplx *n0,
+                 const cplx *u0, const cplx *dn_prev, const cplx *du_prev, double c1, double c2, cplx *dn, cplx *du,
+                 cplx *n_out, cplx *u_out);
 void count_nonzero(Launcher &L, const cplx *x, long long len, double *cnt);
 
 // Measured FP64 FMA rate of the current device in TFLOP/s (eight independent DFMA chains
