@@ -67,6 +67,7 @@ __device__ __forceinline__ void tile_fma(const cplx (*As)[GBM + 1], const cplx (
 template <int TI, int TJ>
 __global__ void __launch_bounds__(GNT) zgemm_kernel(ZGemmDev g, int reduce, int per_split, cplx *partial, int kparts,
                                                      int klen) {
+  dependent_begin();
   __shared__ cplx As[GBK][GBM + 1];
   __shared__ cplx Bs[GBK][GBN + 1];
   const int tid = threadIdx.x;
@@ -146,6 +147,7 @@ __global__ void __launch_bounds__(GNT) zgemm_kernel(ZGemmDev g, int reduce, int 
 
 // Block (32, 32): x = one of 32 consecutive outputs, y = a strided subset of the splits.
 __global__ void __launch_bounds__(1024) zgemm_reduce_kernel(ZGemmDev g, int splits, const cplx *partial) {
+  dependent_begin();
   __shared__ cplx part[32][33];
   const long long mn = (long long)g.M * g.N;
   const long long idx = (long long)blockIdx.x * 32 + threadIdx.x;
@@ -182,6 +184,7 @@ constexpr int PT = 32;
 
 __global__ void permute4_kernel(int nb, const cplx *__restrict__ in, cplx *__restrict__ out, int p0, int p1,
                                 int p2, int p3, cplx alpha, double beta, int conj) {
+  dependent_begin();
   // out axis 3 is innermost in memory; input innermost axis is out-axis p3.
   __shared__ cplx tile[PT][PT + 1];
   const int ntile = (nb + PT - 1) / PT;
@@ -252,6 +255,7 @@ template <bool REAL>
 __global__ void hf_build_kernel(int nb, const void *__restrict__ Wm_, const cplx *__restrict__ h,
                                 const cplx *__restrict__ D, double f, const cplx *__restrict__ n,
                                 cplx *__restrict__ hhf) {
+  dependent_begin();
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const int nb2 = nb * nb;
@@ -425,6 +429,7 @@ __global__ void __launch_bounds__(256) hf_build_ds_kernel(int nb, const float2 *
 }
 
 __global__ void one_pm_kernel(int nb, const cplx *n, double eta, cplx *nbar) {
+  dependent_begin();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= nb * nb) return;
   const int i = idx / nb, j = idx % nb;
@@ -465,6 +470,7 @@ __global__ void __launch_bounds__(256) g1_update_kernel(int nb, const cplx *__re
                                                         const cplx *__restrict__ n, const cplx *__restrict__ I,
                                                         int stage, double dt, cplx *y, cplx *ys, cplx *acc,
                                                         cplx *kout) {
+  dependent_begin();
   const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (idx >= nb * nb) return;
@@ -492,6 +498,7 @@ __global__ void __launch_bounds__(256) g1_update_kernel(int nb, const cplx *__re
 // dG = -i (Cb - Ab + conj(Ab^T)): 32x32 tiles of the (ij),(kl) matrix view.
 __global__ void g2_assemble_kernel(int nb, const cplx *__restrict__ Cb, const cplx *__restrict__ Ab, int stage,
                                    double dt, cplx *y, cplx *ys, cplx *acc, cplx *kout) {
+  dependent_begin();
   __shared__ cplx tile[PT][PT + 1];
   const long long M = (long long)nb * nb;
   const long long r0 = (long long)blockIdx.y * PT, c0 = (long long)blockIdx.x * PT;
@@ -538,7 +545,7 @@ __global__ void g2_assemble_kernel(int nb, const cplx *__restrict__ Cb, const cp
 // between two buffers, as those of n do, because other threads still read the stage input.  At eight sites
 // a stage is bound by launch latency and by one pass through the FP64 pipe (an FP64 instruction takes
 // 64 cycles of it per warp): separate kernels for h^HF, I, G1, C and the update took 42 us per stage,
-// this one NNN us.  The source term is factored into six complex products instead of eight.
+// this one 12 us.  The source term is factored into six complex products instead of eight.
 __device__ __forceinline__ cplx hub_h(const HubStage &p, int i, int j) {
   cplx v = p.h[i * p.nb + j];
   if (p.D) {
@@ -552,7 +559,14 @@ __device__ __forceinline__ cplx hub_diag(const HubStage &p, int i) {
   return {fma(p.U[i], m.x, v.x), fma(p.U[i], m.y, v.y)};
 }
 
+// The pattern with its h^HF entries goes through shared memory: read from global memory per element, the chain
+// row pointer -> column -> (h, G) cost four dependent loads in a row for each of the four indices.
+constexpr int kHubNnz = 512, kHubMaxNb = 128;
+
 __global__ void __launch_bounds__(128) hubbard_stage_kernel(const HubStage p, int g1_blocks, int bx) {
+  __shared__ int srp[kHubMaxNb + 1], sci[kHubNnz];
+  __shared__ cplx srow[kHubNnz], scol[kHubNnz], sdiag[kHubMaxNb];   // h_is, h_si along the pattern; h^HF_ii
+  dependent_begin();
   const int nb = p.nb;
   const long long N = nb, N2 = N * N, N3 = N2 * N;
   if ((int)blockIdx.x < g1_blocks) {
@@ -577,6 +591,26 @@ __global__ void __launch_bounds__(128) hubbard_stage_kernel(const HubStage p, in
     rk4_apply(idx, csub(mul_minus_i(comm), cadd(a, b)), p.stage, p.dt, p.ny, p.nys, p.nacc, p.nk);
     return;
   }
+  const bool cached = p.nnz <= kHubNnz;
+  for (int i = threadIdx.x; i <= nb; i += blockDim.x) {
+    srp[i] = p.rp[i];
+    if (i < nb) sdiag[i] = hub_diag(p, i);
+  }
+  if (cached) {
+    for (int q = threadIdx.x; q < p.nnz; q += blockDim.x) sci[q] = p.ci[q];
+    __syncthreads();
+    for (int q = threadIdx.x; q < p.nnz; q += blockDim.x) {
+      int lo = 0, hi = nb;                                  // the row of entry q
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (srp[mid] <= q) lo = mid;
+        else hi = mid;
+      }
+      srow[q] = hub_h(p, lo, sci[q]);
+      scol[q] = hub_h(p, sci[q], lo);
+    }
+  }
+  __syncthreads();
   const int blk = blockIdx.x - g1_blocks, ij = blk / bx, i = ij / nb, j = ij - i * nb;
   const int kl = (blk - ij * bx) * blockDim.x + threadIdx.x;
   if (kl >= nb * nb) return;
@@ -585,25 +619,20 @@ __global__ void __launch_bounds__(128) hubbard_stage_kernel(const HubStage p, in
   const int k = kl / nb, l = kl - k * nb;
   const long long e = (long long)ij * N2 + kl;
   // [h2, G]_ijkl = sum_p h_ip G_pjkl + h_jp G_ipkl - G_ijpl h_pk - G_ijkp h_pl, the diagonals in one factor
-  const cplx dg = csub(csub(cadd(hub_diag(p, i), hub_diag(p, j)), hub_diag(p, k)), hub_diag(p, l));
-  cplx acc = cmul(dg, G[e]);
-  for (int q = p.rp[i]; q < p.rp[i + 1]; ++q) {
-    const int s = p.ci[q];
-    if (s != i) acc = cfma(hub_h(p, i, s), G[s * N3 + j * N2 + kl], acc);
-  }
-  for (int q = p.rp[j]; q < p.rp[j + 1]; ++q) {
-    const int s = p.ci[q];
-    if (s != j) acc = cfma(hub_h(p, j, s), G[i * N3 + s * N2 + kl], acc);
-  }
-  cplx sub = {0.0, 0.0};
-  for (int q = p.rp[k]; q < p.rp[k + 1]; ++q) {
-    const int s = p.ci[q];
-    if (s != k) sub = cfma(G[(long long)ij * N2 + s * N + l], hub_h(p, s, k), sub);
-  }
-  for (int q = p.rp[l]; q < p.rp[l + 1]; ++q) {
-    const int s = p.ci[q];
-    if (s != l) sub = cfma(G[e - l + s], hub_h(p, s, l), sub);
-  }
+  const cplx dg = csub(csub(cadd(sdiag[i], sdiag[j]), sdiag[k]), sdiag[l]);
+  cplx acc = cmul(dg, G[e]), sub = {0.0, 0.0};
+  auto stencil = [&](int row, const cplx *g, long long step, bool column, cplx &sum) {
+    for (int q = srp[row]; q < srp[row + 1]; ++q) {
+      const int s = cached ? sci[q] : p.ci[q];
+      if (s == row) continue;
+      const cplx hv = cached ? (column ? scol[q] : srow[q]) : column ? hub_h(p, s, row) : hub_h(p, row, s);
+      sum = cfma(hv, g[s * step], sum);
+    }
+  };
+  stencil(i, G + j * N2 + kl, N3, false, acc);
+  stencil(j, G + i * N3 + kl, N2, false, acc);
+  stencil(k, G + (long long)ij * N2 + l, N, true, sub);
+  stencil(l, G + e - l, 1, true, sub);
   if (!other) {
     // Psi = -S: S = n_jk (n_jl x1 + n_ik x4) + n_il (n_ik x2 + n_jl x3)
     const cplx *n = p.n;
@@ -725,6 +754,7 @@ __global__ void sum_pairs_kernel(const double *partials, long long nblk, double 
 // fixed order (deterministic, no atomics)
 __global__ void __launch_bounds__(1024) accumulate_work_kernel(int nb, const cplx *D, const cplx *n, double coeff,
                                                                double *W) {
+  dependent_begin();
   __shared__ double s[32];
   double a = 0;
   for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
@@ -778,10 +808,10 @@ __global__ void count_nonfinite_kernel(const cplx *x, long long len, double *cnt
 void launch_zgemm(dim3 grid, cudaStream_t st, const ZGemm &g, int reduce, int per, cplx *partial, int kparts,
                   int klen) {
   const bool mw = g.M > GBM / GTM, nw = g.N > GBN / GTN;
-  if (mw && nw) zgemm_kernel<GTM, GTN><<<grid, GNT, 0, st>>>(to_dev(g), reduce, per, partial, kparts, klen);
-  else if (mw) zgemm_kernel<GTM, 1><<<grid, GNT, 0, st>>>(to_dev(g), reduce, per, partial, kparts, klen);
-  else if (nw) zgemm_kernel<1, GTN><<<grid, GNT, 0, st>>>(to_dev(g), reduce, per, partial, kparts, klen);
-  else zgemm_kernel<1, 1><<<grid, GNT, 0, st>>>(to_dev(g), reduce, per, partial, kparts, klen);
+  if (mw && nw) launch_dependent(zgemm_kernel<GTM, GTN>, grid, GNT, 0, st, to_dev(g), reduce, per, partial, kparts, klen);
+  else if (mw) launch_dependent(zgemm_kernel<GTM, 1>, grid, GNT, 0, st, to_dev(g), reduce, per, partial, kparts, klen);
+  else if (nw) launch_dependent(zgemm_kernel<1, GTN>, grid, GNT, 0, st, to_dev(g), reduce, per, partial, kparts, klen);
+  else launch_dependent(zgemm_kernel<1, 1>, grid, GNT, 0, st, to_dev(g), reduce, per, partial, kparts, klen);
 }
 
 void zgemm(Launcher &L, const ZGemm &g) {
@@ -810,7 +840,7 @@ void zgemm_reduce(Launcher &L, const ZGemm &g, cplx *partial, int splits) {
   L.after_launch();
   const long long mn = (long long)g.M * g.N;
   L.before("fp64_splitk_reduce");
-  zgemm_reduce_kernel<<<(unsigned)((mn + 31) / 32), dim3(32, 32), 0, L.stream>>>(to_dev(g), splits, partial);
+  launch_dependent(zgemm_reduce_kernel, (unsigned)((mn + 31) / 32), dim3(32, 32), 0, L.stream, to_dev(g), splits, partial);
   L.after_launch();
 }
 
@@ -820,10 +850,10 @@ void permute4(Launcher &L, int nb, const cplx *in, cplx *out, const int p[4], cp
   L.before("permute4");
   if (p[3] == 3) {
     dim3 grid(1, (unsigned)((long long)nb * nb));
-    permute4_kernel<<<grid, block, 0, L.stream>>>(nb, in, out, p[0], p[1], p[2], p[3], alpha, beta, conj);
+    launch_dependent(permute4_kernel, grid, block, 0, L.stream, nb, in, out, p[0], p[1], p[2], p[3], alpha, beta, conj);
   } else {
     dim3 grid(nt * nt, (unsigned)((long long)nb * nb));
-    permute4_kernel<<<grid, block, 0, L.stream>>>(nb, in, out, p[0], p[1], p[2], p[3], alpha, beta, conj);
+    launch_dependent(permute4_kernel, grid, block, 0, L.stream, nb, in, out, p[0], p[1], p[2], p[3], alpha, beta, conj);
   }
   L.after_launch();
 }
@@ -835,9 +865,9 @@ void hf_build(Launcher &L, int nb, const void *Wm, bool wm_real, const cplx *h, 
   const int blocks = (warps * 32 + threads - 1) / threads;
   L.before("hf_build");
   if (wm_real)
-    hf_build_kernel<true><<<blocks, threads, 0, L.stream>>>(nb, Wm, h, D, f, n, hhf);
+    launch_dependent(hf_build_kernel<true>, blocks, threads, 0, L.stream, nb, Wm, h, D, f, n, hhf);
   else
-    hf_build_kernel<false><<<blocks, threads, 0, L.stream>>>(nb, Wm, h, D, f, n, hhf);
+    launch_dependent(hf_build_kernel<false>, blocks, threads, 0, L.stream, nb, Wm, h, D, f, n, hhf);
   L.after_launch();
 }
 
@@ -855,14 +885,14 @@ void hf_build_ds(Launcher &L, int nb, const float2 *Wds, const cplx *h, const cp
 
 void one_pm(Launcher &L, int nb, const cplx *n, double eta, cplx *nbar) {
   L.before("one_minus");
-  one_pm_kernel<<<(nb * nb + 255) / 256, 256, 0, L.stream>>>(nb, n, eta, nbar);
+  launch_dependent(one_pm_kernel, (nb * nb + 255) / 256, 256, 0, L.stream, nb, n, eta, nbar);
   L.after_launch();
 }
 
 void g1_update(Launcher &L, int nb, const cplx *hhf, const cplx *n, const cplx *I, Rk4Stage st, cplx *y, cplx *ys,
                cplx *acc, cplx *kout) {
   L.before("g1_update");
-  g1_update_kernel<<<(nb * nb + 7) / 8, 256, 0, L.stream>>>(nb, hhf, n, I, st.stage, st.dt, y, ys, acc, kout);
+  launch_dependent(g1_update_kernel, (nb * nb + 7) / 8, 256, 0, L.stream, nb, hhf, n, I, st.stage, st.dt, y, ys, acc, kout);
   L.after_launch();
 }
 
@@ -871,7 +901,7 @@ void g2_assemble(Launcher &L, int nb, const cplx *Cb, const cplx *Ab, Rk4Stage s
   const long long M = (long long)nb * nb;
   const unsigned t = (unsigned)((M + PT - 1) / PT);
   L.before("fp64_g2_assemble_rk4");
-  g2_assemble_kernel<<<dim3(t, t), dim3(PT, 8), 0, L.stream>>>(nb, Cb, Ab, st.stage, st.dt, y, ys, acc, kout);
+  launch_dependent(g2_assemble_kernel, dim3(t, t), dim3(PT, 8), 0, L.stream, nb, Cb, Ab, st.stage, st.dt, y, ys, acc, kout);
   L.after_launch();
 }
 
@@ -879,7 +909,7 @@ void hubbard_stage(Launcher &L, const HubStage &p) {
   const int nb2 = p.nb * p.nb, threads = nb2 <= 256 ? 64 : 128;
   const int g1 = (nb2 * 32 + threads - 1) / threads, bx = (nb2 + threads - 1) / threads;
   L.before("hubbard_stage");
-  hubbard_stage_kernel<<<dim3(g1 + bx * nb2, p.Go ? 2 : 1), threads, 0, L.stream>>>(p, g1, bx);
+  launch_dependent(hubbard_stage_kernel, dim3(g1 + bx * nb2, p.Go ? 2 : 1), threads, 0, L.stream, p, g1, bx);
   L.after_launch();
 }
 
@@ -905,7 +935,7 @@ void obs_two_body(Launcher &L, int nb, const cplx *W, const cplx *G, double *par
 
 void accumulate_work(Launcher &L, int nb, const cplx *D, const cplx *n, double coeff, double *W_acc) {
   L.before("drive_work");
-  accumulate_work_kernel<<<1, 1024, 0, L.stream>>>(nb, D, n, coeff, W_acc);
+  launch_dependent(accumulate_work_kernel, 1, 1024, 0, L.stream, nb, D, n, coeff, W_acc);
   L.after_launch();
 }
 
@@ -932,6 +962,7 @@ namespace {
 
 __global__ void zaxpby_kernel(long long n, cplx alpha, const cplx *__restrict__ x, cplx beta,
                               const cplx *__restrict__ y, cplx *out) {
+  dependent_begin();
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     cplx r = cmul(alpha, x[e]);
     if (y) r = cadd(r, cmul(beta, y[e]));
@@ -939,8 +970,31 @@ __global__ void zaxpby_kernel(long long n, cplx alpha, const cplx *__restrict__ 
   }
 }
 
+// out = i (A B - B A): one warp per element, so that the nb^3 FP64 multiply-adds spread over every SM (as products of
+// one 32 x 32 tile each they took 79 us at nb = 32)
+__global__ void __launch_bounds__(256) commutator_kernel(int nb, const cplx *__restrict__ A, const cplx *__restrict__ B,
+                                                         cplx *__restrict__ out) {
+  dependent_begin();
+  const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (idx >= nb * nb) return;
+  const int i = idx / nb, j = idx % nb;
+  cplx comm = {0.0, 0.0};
+  for (int p = lane; p < nb; p += 32) {
+    comm = cfma(A[i * nb + p], B[p * nb + j], comm);
+    comm = csub(comm, cmul(B[i * nb + p], A[p * nb + j]));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    comm.x += __shfl_xor_sync(0xffffffffu, comm.x, o);
+    comm.y += __shfl_xor_sync(0xffffffffu, comm.y, o);
+  }
+  if (lane == 0) out[idx] = {-comm.y, comm.x};
+}
+
 // out = c * (a + a^dag) for an nb x nb matrix
 __global__ void herm_sum_kernel(int nb, cplx c, const cplx *__restrict__ a, cplx *out) {
+  dependent_begin();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nb * nb) return;
   const int i = e / nb, j = e % nb;
@@ -949,6 +1003,7 @@ __global__ void herm_sum_kernel(int nb, cplx c, const cplx *__restrict__ a, cplx
 
 // out = c * (Y + Y^dag), (Y^dag)_ijkl = conj(Y_klij), 32x32 tiles of the (ij),(kl) view
 __global__ void tconj_add_kernel(int nb, cplx c, const cplx *__restrict__ Y, cplx *out) {
+  dependent_begin();
   __shared__ cplx tile[PT][PT + 1];
   const long long M = (long long)nb * nb;
   const long long r0 = (long long)blockIdx.y * PT, c0 = (long long)blockIdx.x * PT;
@@ -968,6 +1023,7 @@ __global__ void tconj_add_kernel(int nb, cplx c, const cplx *__restrict__ Y, cpl
 
 // partial sums of Re sum conj(x) y
 __global__ void real_dot_kernel(long long n, const cplx *__restrict__ x, const cplx *__restrict__ y, double *partials) {
+  dependent_begin();
   __shared__ double s[256];
   double a = 0.0;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
@@ -983,6 +1039,7 @@ __global__ void real_dot_kernel(long long n, const cplx *__restrict__ x, const c
 
 // acc[slot] += coeff * sum(partials)
 __global__ void dot_accumulate_kernel(int nparts, const double *partials, double coeff, double *acc) {
+  dependent_begin();
   __shared__ double s[256];
   double a = 0.0;
   for (int i = threadIdx.x; i < nparts; i += blockDim.x) a += partials[i];
@@ -998,12 +1055,13 @@ __global__ void dot_accumulate_kernel(int nparts, const double *partials, double
 // out_lk (+)= sum_ij Wm[(ij),(lk)] x_ij  (the adjoint of the Hartree-Fock build).  A CTA takes eight columns
 // (64 bytes of every row of a real Wm), its 32 rows of threads the rows of Wm in turn, and reduces them in a
 // fixed order: one thread per column left three quarters of the chip idle and a chain of nb^2 loads
-// (nb = 32: 190 us, now NNN us).
+// (nb = 32: 190 us, now 20 us).
 constexpr int kHtCols = 8, kHtRows = 32;
 template <bool REAL>
 __global__ void __launch_bounds__(kHtCols * kHtRows) hf_build_t_kernel(int nb, const void *__restrict__ Wm_,
                                                                        const cplx *__restrict__ x, cplx *out,
                                                                        int accumulate) {
+  dependent_begin();
   __shared__ cplx part[kHtRows][kHtCols];
   const int nb2 = nb * nb;
   const int tc = threadIdx.x % kHtCols, tr = threadIdx.x / kHtCols;
@@ -1034,7 +1092,7 @@ __global__ void __launch_bounds__(kHtCols * kHtRows) hf_build_t_kernel(int nb, c
 
 void zaxpby(Launcher &L, long long n, cplx alpha, const cplx *x, cplx beta, const cplx *y, cplx *out) {
   L.before("adj_axpby");
-  zaxpby_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 8192), 256, 0, L.stream>>>(n, alpha, x, beta, y, out);
+  launch_dependent(zaxpby_kernel, (unsigned)std::min<long long>((n + 255) / 256, 8192), 256, 0, L.stream, n, alpha, x, beta, y, out);
   L.after_launch();
 }
 
@@ -1084,7 +1142,7 @@ void w_symmetrize(Launcher &L, int nb, const cplx *X, cplx *out) {
 
 void herm_sum(Launcher &L, int nb, cplx c, const cplx *a, cplx *out) {
   L.before("adj_herm_sum");
-  herm_sum_kernel<<<(nb * nb + 127) / 128, 128, 0, L.stream>>>(nb, c, a, out);
+  launch_dependent(herm_sum_kernel, (nb * nb + 127) / 128, 128, 0, L.stream, nb, c, a, out);
   L.after_launch();
 }
 
@@ -1092,17 +1150,23 @@ void tconj_add(Launcher &L, int nb, cplx c, const cplx *Y, cplx *out) {
   const long long M = (long long)nb * nb;
   const unsigned t = (unsigned)((M + PT - 1) / PT);
   L.before("adj_tconj_add");
-  tconj_add_kernel<<<dim3(t, t), dim3(PT, 8), 0, L.stream>>>(nb, c, Y, out);
+  launch_dependent(tconj_add_kernel, dim3(t, t), dim3(PT, 8), 0, L.stream, nb, c, Y, out);
   L.after_launch();
 }
 
 void real_dot_acc(Launcher &L, long long n, const cplx *x, const cplx *y, double coeff, double *partials, double *acc) {
   const int blocks = (int)std::min<long long>((n + 255) / 256, 1024);
   L.before("adj_dot");
-  real_dot_kernel<<<blocks, 256, 0, L.stream>>>(n, x, y, partials);
+  launch_dependent(real_dot_kernel, blocks, 256, 0, L.stream, n, x, y, partials);
   L.after_launch();
   L.before("adj_dot");
-  dot_accumulate_kernel<<<1, 256, 0, L.stream>>>(blocks, partials, coeff, acc);
+  launch_dependent(dot_accumulate_kernel, 1, 256, 0, L.stream, blocks, partials, coeff, acc);
+  L.after_launch();
+}
+
+void commutator_i(Launcher &L, int nb, const cplx *A, const cplx *B, cplx *out) {
+  L.before("adj_commutator");
+  launch_dependent(commutator_kernel, (nb * nb + 7) / 8, 256, 0, L.stream, nb, A, B, out);
   L.after_launch();
 }
 
@@ -1110,9 +1174,9 @@ void hf_build_t(Launcher &L, int nb, const void *Wm, bool wm_real, const cplx *x
   const int nb2 = nb * nb;
   L.before("adj_hf_build_t");
   if (wm_real)
-    hf_build_t_kernel<true><<<(nb2 + kHtCols - 1) / kHtCols, kHtCols * kHtRows, 0, L.stream>>>(nb, Wm, x, out, accumulate ? 1 : 0);
+    launch_dependent(hf_build_t_kernel<true>, (nb2 + kHtCols - 1) / kHtCols, kHtCols * kHtRows, 0, L.stream, nb, Wm, x, out, accumulate ? 1 : 0);
   else
-    hf_build_t_kernel<false><<<(nb2 + kHtCols - 1) / kHtCols, kHtCols * kHtRows, 0, L.stream>>>(nb, Wm, x, out, accumulate ? 1 : 0);
+    launch_dependent(hf_build_t_kernel<false>, (nb2 + kHtCols - 1) / kHtCols, kHtCols * kHtRows, 0, L.stream, nb, Wm, x, out, accumulate ? 1 : 0);
   L.after_launch();
 }
 
@@ -1132,6 +1196,7 @@ namespace {
 __global__ void __launch_bounds__(256) pair_rotate_kernel(int nb, int second, int from_a, const cplx *__restrict__ in,
                                                           const cplx *__restrict__ S, int form, double eta,
                                                           cplx *__restrict__ out) {
+  dependent_begin();
   __shared__ cplx X[kPairMaxNb * kPairMaxNb], T[kPairMaxNb * kPairMaxNb], M[kPairMaxNb * kPairMaxNb];
   const int n2 = nb * nb, c = blockIdx.x;
   for (int e = threadIdx.x; e < n2; e += blockDim.x) {
@@ -1169,6 +1234,7 @@ __global__ void __launch_bounds__(256) pair_rotate_kernel(int nb, int second, in
 // fixed-order reduction over the warps in shared memory (deterministic).
 __global__ void __launch_bounds__(256) trapezoid_sum_kernel(long long len, int nbatch, const cplx *__restrict__ x,
                                                             double dt, cplx *out) {
+  dependent_begin();
   __shared__ cplx part[8][32];
   const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
   const long long e = (long long)blockIdx.x * 32 + lane;
@@ -1198,6 +1264,7 @@ __global__ void __launch_bounds__(128) mean_collision_kernel(int nb, const void 
                                                              const cplx *__restrict__ h, const cplx *__restrict__ n,
                                                              const cplx *__restrict__ wP, const cplx *__restrict__ G,
                                                              cplx *__restrict__ hhf, cplx *__restrict__ I) {
+  dependent_begin();
   __shared__ cplx part[2][4];
   const int i = blockIdx.x / nb, j = blockIdx.x - i * nb, n2 = nb * nb, n3 = n2 * nb;
   cplx a = {0.0, 0.0}, b = {0.0, 0.0};
@@ -1243,6 +1310,7 @@ __global__ void __launch_bounds__(256) heun_update_kernel(int nb, const cplx *__
                                                           const cplx *n0, const cplx *u0, const cplx *dn_prev,
                                                           const cplx *du_prev, double c1, double c2, cplx *dn, cplx *du,
                                                           cplx *n_out, cplx *u_out) {
+  dependent_begin();
   const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (idx >= nb * nb) return;
@@ -1293,20 +1361,20 @@ __global__ void count_nonzero_kernel(const cplx *x, long long len, double *cnt) 
 void pair_rotate(Launcher &L, int nb, bool second, bool from_a, const cplx *in, const cplx *S, PairForm form, double eta,
                  cplx *out) {
   L.before("hfgkba_pair_rotate");
-  pair_rotate_kernel<<<nb * nb, nb <= 8 ? 64 : 256, 0, L.stream>>>(nb, second ? 1 : 0, from_a ? 1 : 0, in, S, form, eta, out);
+  launch_dependent(pair_rotate_kernel, nb * nb, nb <= 8 ? 64 : 256, 0, L.stream, nb, second ? 1 : 0, from_a ? 1 : 0, in, S, form, eta, out);
   L.after_launch();
 }
 
 void trapezoid_sum(Launcher &L, long long len, int npoints, const cplx *x, double dt, cplx *out) {
   L.before("hfgkba_trapezoid");
-  trapezoid_sum_kernel<<<(unsigned)((len + 31) / 32), 256, 0, L.stream>>>(len, npoints, x, dt, out);
+  launch_dependent(trapezoid_sum_kernel, (unsigned)((len + 31) / 32), 256, 0, L.stream, len, npoints, x, dt, out);
   L.after_launch();
 }
 
 void mean_collision(Launcher &L, int nb, const void *Wm, bool wm_real, const cplx *h, const cplx *n, const cplx *wP,
                     const cplx *G, cplx *hhf, cplx *I) {
   L.before("hfgkba_mean_collision");
-  mean_collision_kernel<<<nb * nb, 128, 0, L.stream>>>(nb, Wm, wm_real ? 1 : 0, h, n, wP, G, hhf, I);
+  launch_dependent(mean_collision_kernel, nb * nb, 128, 0, L.stream, nb, Wm, wm_real ? 1 : 0, h, n, wP, G, hhf, I);
   L.after_launch();
 }
 
@@ -1314,7 +1382,7 @@ void heun_update(Launcher &L, int nb, const cplx *hhf, const cplx *n, const cplx
                  const cplx *u0, const cplx *dn_prev, const cplx *du_prev, double c1, double c2, cplx *dn, cplx *du,
                  cplx *n_out, cplx *u_out) {
   L.before("hfgkba_heun");
-  heun_update_kernel<<<(nb * nb + 7) / 8, 256, 0, L.stream>>>(nb, hhf, n, u, I, n0, u0, dn_prev, du_prev, c1, c2, dn, du,
+  launch_dependent(heun_update_kernel, (nb * nb + 7) / 8, 256, 0, L.stream, nb, hhf, n, u, I, n0, u0, dn_prev, du_prev, c1, c2, dn, du,
                                                               n_out, u_out);
   L.after_launch();
 }

@@ -2,11 +2,11 @@
 //
 // GB300 issues about two FP64 multiply-adds per SM and clock (1.2 TFLOP/s for the chip), so a
 // contraction of the FP64 form is bound by the FP64 pipe 50 to 100 times above the time its
-// bytes take.  Here each real operand is cut into seven signed 8-bit digits, the digit
+// bytes take.  Here each real operand is cut into seven (eight) signed 8-bit digits, the digit
 // products run as BF16 MMAs on tcgen05 and are summed as integers (the error-free
 // splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 95 (2012)):
 //
-//   x = 2^(e - 1077) sum_s d_s 256^(6 - s),  |d_s| <= 128,
+//   x = 2^(e - 1077) sum_s d_s 256^(6 - s),  |d_s| <= 128        (long contractions: 2^(e - 1084) .. 256^(7 - s)),
 //
 // with one exponent e per row of A (column of B) and segment of the contraction (at most 256 terms), the one
 // of its largest entry there, so that 56 bits below that entry's leading bit are kept: every entry
@@ -40,21 +40,25 @@ namespace {
 
 using namespace tc;
 
-constexpr int kDig = 7;                    // digits per real operand
+// Digits per real operand: seven of a 56-bit number, in long contractions eight of a 63-bit one.  There one large entry
+// of a sparse cotangent sets the exponent of its segment, and the sums cancel: with seven digits the drive gradient
+// of the 4 x 4 cluster was up to three times further off than from FP64 multiply-adds.
+__host__ __device__ constexpr int digits_of(bool lng) { return lng ? 8 : 7; }
 constexpr int kOrd = 8;                    // orders of digit products
 constexpr int kTM = 128;                   // rows of A per tile (TMEM lanes)
 constexpr int kTNMax = 128;                // real columns per tile, at most
 constexpr int kKB = 16;                    // K elements per block: one MMA step, 32-byte rows
 constexpr int kSeg = 16;                   // K blocks of a segment (256 terms)
 constexpr uint32_t kADig = kTM * 32;       // one digit plane of an A block: 4 KB
-constexpr uint32_t kABlk = kDig * kADig;   // 28 KB
-constexpr uint32_t kStageBytes = 2 * kABlk;   // A and B (at most 128 columns) blocks
 constexpr int kStages = 3;
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = 64 + 32 * kEpiWarps;   // loader warp, MMA warp, epilogue warps
 constexpr int kStgPitch = 5;               // complex per staged row (4 used)
 constexpr uint32_t kStgWarp = 32 * kStgPitch * 16;
-constexpr size_t kSmem = 1024 + kStages * kStageBytes + kEpiWarps * kStgWarp + 256;
+// A and B blocks (at most 128 columns) per stage, and the staging tiles; long contractions have larger blocks but no
+// staging
+constexpr size_t kSmem = 1024 + kStages * 2 * 7 * kADig + kEpiWarps * kStgWarp + 256;
+static_assert(kStages * 2 * 8 * kADig <= kStages * 2 * 7 * kADig + kEpiWarps * kStgWarp, "stages of a long contraction");
 
 constexpr int kNonFinite = 2047;           // row exponent of a row with an Inf or a NaN
 
@@ -78,29 +82,31 @@ __device__ __forceinline__ long long k_offset(const Operand &o, int k) {
   return (long long)b * o.kout + (long long)(k - b * o.kin) * o.sk;
 }
 
-// The digits of x at row exponent emax as one word: byte 6 - s is d_s + 128 for s = 1..6, the
-// bits from 48 up are d_0 (a balanced base-256 expansion is the plain one of X + 128 (256^0 + .. + 256^5)).
+// The ND digits of x at row exponent emax as one word: byte ND - 1 - s is d_s + 128 for s > 0, the bits above the
+// last of these bytes are d_0 (a balanced base-256 expansion is the plain one of X + 128 (256^0 + ..)).
+// X = x 2^(B + 1022 - emax) to nearest, B = 55 bits (ND = 7) or 62 (ND = 8).
+template <int ND>
 __device__ __forceinline__ unsigned long long digits(double x, int emax) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int e = (hi >> 20) & 0x7ff;
   unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo;
-  const int s = emax - max(e, 1) - 2;      // X = m 2^-s, to nearest
+  const int s = emax - max(e, 1) - (ND == 7 ? 2 : 9);      // X = m 2^-s
   if (s <= 0) m <<= -s;
   else m = (s > 60) ? 0ull : (m + (1ull << (s - 1))) >> s;
   const long long X = ((int)hi < 0) ? -(long long)m : (long long)m;
-  return (unsigned long long)(X + 0x0000808080808080ll);
+  return (unsigned long long)(X + (ND == 7 ? 0x0000808080808080ll : 0x0080808080808080ll));
 }
 
 // d_s of two neighbouring elements as a BF16 pair: 2^23 + byte is an FP32 number, the subtraction
 // exact, and an integer of at most 8 bits has nothing in the low half of its FP32 word.
-template <int S>
+template <int ND, int S>
 __device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned long long b) {
   float fa, fb;
   if (S == 0) {
-    fa = (float)((int)(a >> 32) >> 16);
-    fb = (float)((int)(b >> 32) >> 16);
+    fa = (float)((int)(a >> 32) >> (ND == 7 ? 16 : 24));
+    fb = (float)((int)(b >> 32) >> (ND == 7 ? 16 : 24));
   } else {
-    constexpr int byte = 6 - S;
+    constexpr int byte = ND - 1 - S;
     const uint32_t wa = byte < 4 ? (uint32_t)a : (uint32_t)(a >> 32), wb = byte < 4 ? (uint32_t)b : (uint32_t)(b >> 32);
     fa = __uint_as_float(__byte_perm(wa, 0x4B000000u, 0x7440 | (byte & 3))) - 8388736.0f;
     fb = __uint_as_float(__byte_perm(wb, 0x4B000000u, 0x7440 | (byte & 3))) - 8388736.0f;
@@ -108,19 +114,21 @@ __device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned lo
   return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
 }
 
-// Digit planes in global memory, ready for the MMA: block (tile of TR rows, K block) holds kDig planes
+// Digit planes in global memory, ready for the MMA: block (tile of TR rows, K block) holds ND planes
 // of TR rows x 32 bytes in the 32-byte-swizzled K-major layout, so that the GEMM brings the leading planes
 // of a block in with one contiguous bulk copy and no tensor map.
+template <int ND>
 __device__ __forceinline__ void store_digits(uint8_t *out, int TR, int KB, int row, int q, const unsigned long long (&w)[8],
                                              uint32_t flip) {
   const int tile = row / TR, rr = row - tile * TR, kb = q >> 1, c2 = q & 1;
   const uint32_t plane = (uint32_t)TR * 32;
-  uint8_t *o = out + ((size_t)tile * KB + kb) * (kDig * plane) + rr * 32 + ((c2 ^ ((rr >> 2) & 1)) << 4);
+  uint8_t *o = out + ((size_t)tile * KB + kb) * (ND * plane) + rr * 32 + ((c2 ^ ((rr >> 2) & 1)) << 4);
 #define G1G2_PUT(S)                                                                                          \
   *reinterpret_cast<uint4 *>(o + S * plane) =                                                                \
-      make_uint4(digit_pair<S>(w[0], w[1]) ^ flip, digit_pair<S>(w[2], w[3]) ^ flip,                         \
-                 digit_pair<S>(w[4], w[5]) ^ flip, digit_pair<S>(w[6], w[7]) ^ flip)
+      make_uint4(digit_pair<ND, S>(w[0], w[1]) ^ flip, digit_pair<ND, S>(w[2], w[3]) ^ flip,                 \
+                 digit_pair<ND, S>(w[4], w[5]) ^ flip, digit_pair<ND, S>(w[6], w[7]) ^ flip)
   G1G2_PUT(0); G1G2_PUT(1); G1G2_PUT(2); G1G2_PUT(3); G1G2_PUT(4); G1G2_PUT(5); G1G2_PUT(6);
+  if constexpr (ND > 7) G1G2_PUT(7);
 #undef G1G2_PUT
 }
 
@@ -137,17 +145,18 @@ __host__ __device__ constexpr int cut_rows(int form) { return kCutVals / seg_k(f
 
 // Cuts rows x K of an operand into digits, and finds the exponents.  A CTA stages one segment of 32 rows (16 for
 // kPlanes) in shared memory, read along whichever index is contiguous in memory, takes the largest exponent of each
-// row there, and every thread then cuts eight consecutive K values of one row at a time into seven
+// row there, and every thread then cuts eight consecutive K values of one row at a time into seven (eight)
 // 16-byte stores; a warp writes 16 rows x 32 bytes, 512 contiguous bytes, per digit.  Bound by its 16
 // bytes read and 28 written per complex element (56 for kReal).
 template <int FORM>
 __global__ void __launch_bounds__(256) cut_digits_kernel(const Operand A, int r_begin, int k_begin, int Klen, int Kp,
                                                          int TR, int KB, int *__restrict__ rexp,
                                                          uint8_t *__restrict__ out) {
-  constexpr int SK = seg_k(FORM), SR = cut_rows(FORM);
+  constexpr int SK = seg_k(FORM), SR = cut_rows(FORM), ND = digits_of(FORM == kPlanes);
   extern __shared__ double sh[];
   __shared__ long long roff[SR], koff[SK];
   __shared__ int emax[SR];
+  dependent_begin();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r0 = blockIdx.x * SR;                         // within the panel
   const int nr = min(SR, A.rows - r0);                    // A.rows: rows of the panel
@@ -202,15 +211,15 @@ __global__ void __launch_bounds__(256) cut_digits_kernel(const Operand A, int r_
     const int e = emax[r];
     unsigned long long w[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = digits(e == kNonFinite ? 0.0 : src[i], e);
+    for (int i = 0; i < 8; ++i) w[i] = digits<ND>(e == kNonFinite ? 0.0 : src[i], e);
     const int q0 = seg * 2 * kSeg, row = r0 + r;          // 16-byte chunks before this segment
     if (FORM == kRows) {
-      store_digits(out, TR, KB, row, q0 + u * nch + kc, w, 0u);
+      store_digits<ND>(out, TR, KB, row, q0 + u * nch + kc, w, 0u);
     } else if (FORM == kReal) {
-      store_digits(out, TR, KB, 2 * row, q0 + u * nch + kc, w, u ? 0x80008000u : 0u);
-      store_digits(out, TR, KB, 2 * row + 1, q0 + (1 - u) * nch + kc, w, 0u);
+      store_digits<ND>(out, TR, KB, 2 * row, q0 + u * nch + kc, w, u ? 0x80008000u : 0u);
+      store_digits<ND>(out, TR, KB, 2 * row + 1, q0 + (1 - u) * nch + kc, w, 0u);
     } else {
-      store_digits(out, TR, KB, 2 * row + u, q0 + kc, w, 0u);
+      store_digits<ND>(out, TR, KB, 2 * row + u, q0 + kc, w, 0u);
     }
   }
 }
@@ -377,10 +386,12 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
   constexpr bool kSplit = kKind == 2;
   constexpr int kPhases = kOrd / G;
   constexpr int kTN = 512 / G;                       // TMEM columns per accumulator
+  constexpr int kDig = digits_of(kSplit);
+  constexpr uint32_t kABlk = kDig * kADig, kStageBytes = 2 * kABlk;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t *stg_all = smem + kStages * kStageBytes;
-  uint64_t *bars = reinterpret_cast<uint64_t *>(stg_all + kEpiWarps * kStgWarp);
+  uint8_t *stg_all = smem + kStages * kStageBytes;   // not in long contractions
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kSmem - 1024 - 256);
   uint64_t *full = bars, *empty = bars + kStages, *tfull = bars + 2 * kStages, *tempty = tfull + 1, *fin = tempty + 1;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fin + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -399,6 +410,7 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  dependent_begin();
   const int units = p.mtiles * p.ntiles * p.splits;
 
   if (warp == 0) {
@@ -542,7 +554,7 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
           double v[8];
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const int e = ea + __shfl_sync(0xffffffffu, eyl, g - cg + (j >> 1)) - 2114;
+            const int e = ea + __shfl_sync(0xffffffffu, eyl, g - cg + (j >> 1)) - (kSplit ? 2112 : 2114);
             v[j] = fixed_to_double(hi[j], lo[j], e);
           }
           if (any_bad) {
@@ -634,6 +646,7 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
 // Sums the units of a long contraction in a fixed order and combines the four real products:
 // C[i][j] = alpha ((re re - im im) + i (re im + im re)) + beta C.  One warp per output element.
 __global__ void __launch_bounds__(256) fp64_tc_reduce_kernel(const TcGemm p) {
+  dependent_begin();
   const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (idx >= p.rows * p.cols) return;
   const int i = idx / p.cols, j = idx - i * p.cols;
@@ -676,8 +689,8 @@ int tile_columns(int real_cols) {
 template <int kKind>
 void launch_gemm(Launcher &L, const TcGemm &t, int ctas, const char *tag) {
   L.before(tag);
-  if (t.nt <= 64) fp64_tc_gemm_kernel<8, kKind><<<ctas, kThreads, kSmem, L.stream>>>(t);
-  else fp64_tc_gemm_kernel<4, kKind><<<ctas, kThreads, kSmem, L.stream>>>(t);
+  if (t.nt <= 64) launch_dependent(fp64_tc_gemm_kernel<8, kKind>, ctas, kThreads, kSmem, L.stream, t);
+  else launch_dependent(fp64_tc_gemm_kernel<4, kKind>, ctas, kThreads, kSmem, L.stream, t);
   L.after_launch();
 }
 
@@ -690,7 +703,7 @@ void cut(Launcher &L, const Operand &o, int r_begin, int rows, int k_begin, int 
   const size_t sh = (size_t)2 * cut_rows(FORM) * (kt + 1) * sizeof(double);
   dim3 grid((rows + cut_rows(FORM) - 1) / cut_rows(FORM), (Kp + seg_k(FORM) - 1) / seg_k(FORM));
   L.before("fp64_tc_digits");
-  cut_digits_kernel<FORM><<<grid, 256, sh, L.stream>>>(A, r_begin, k_begin, Klen, Kp, TR, KB, rexp, out);
+  launch_dependent(cut_digits_kernel<FORM>, grid, 256, sh, L.stream, A, r_begin, k_begin, Klen, Kp, TR, KB, rexp, out);
   L.after_launch();
 }
 
@@ -710,6 +723,7 @@ struct Fp64Tc {
   double *part = nullptr;               // FP64 sums of a tile per CTA
   int *err = nullptr;
   int sms = 0;
+  int yK = 0, ycols = 0;                // shape of the column operand whose digits B holds whole (0: none)
 };
 
 void fp64_tc_destroy(Fp64Tc *f) {
@@ -725,9 +739,11 @@ Fp64Tc *fp64_tc_create(int nb, bool pair_products) {
   if (!f) return nullptr;
   // digit blocks: all of a big operand up to kPanelBytes, panels of it above
   constexpr size_t kPanelBytes = (size_t)1 << 30;
-  auto blocks = [](long long rows, long long Kp) { return (size_t)((rows + 127) / 128 * 128) * (size_t)Kp * 2 * kDig; };
+  auto blocks = [](long long rows, long long Kp, bool lng = false) {
+    return (size_t)((rows + 127) / 128 * 128) * (size_t)Kp * 2 * digits_of(lng);
+  };
   const size_t big = blocks(N3, 2 * ((N + 7) / 8 * 8)), pair = pair_products ? blocks(2 * N2, 2 * ((N2 + 7) / 8 * 8)) : 0;
-  const size_t lng = blocks(2 * N, (N3 + 255) / 256 * 256);
+  const size_t lng = blocks(2 * N, (N3 + 255) / 256 * 256, true);
   f->a_bytes = std::min(kPanelBytes, std::max({big, pair, lng}));
   f->b_bytes = std::min(kPanelBytes, std::max({blocks(2 * N, 2 * ((N + 7) / 8 * 8)), pair, lng}));
   f->exps = std::max({N3, N2 * ((N2 + 127) / 128), N * ((N3 + 255) / 256)});
@@ -777,6 +793,9 @@ int fp64_tc_error(Fp64Tc *f, cudaStream_t stream) {
 bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
   Fp64Tc *f = L.ftc;
   if (!f) return false;
+  // digits of the last product's column operand, when that product ran here and the caller says that it is the same
+  const int yK = g.same_small ? f->yK : 0, ycols = f->ycols;
+  f->yK = 0;
   const int alpha = unit_of(g.alpha);
   if (alpha < 0 || (g.beta != 0.0 && g.beta != 1.0)) return false;
   if (g.batch > 1 && g.sa_b != 0 && g.sb_b != 0) return false;
@@ -794,13 +813,14 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
   X.rows = (int)rows;
   const int nt = tile_columns(2 * cols);
   // panels of whole tiles
-  const size_t a_tile = (size_t)KB * kABlk, b_tile = (size_t)KB * kDig * nt * 32;
+  constexpr int kDig = digits_of(false);
+  const size_t a_tile = (size_t)KB * kDig * kADig, b_tile = (size_t)KB * kDig * nt * 32;
   const int all_m = (int)((rows + kTM - 1) / kTM), all_n = (2 * cols + nt - 1) / nt;
   const int pm = (int)std::min<size_t>(all_m, f->a_bytes / a_tile), pn = (int)std::min<size_t>(all_n, f->b_bytes / b_tile);
   if (pm < 1 || pn < 1) return false;
   for (int n0 = 0; n0 < all_n; n0 += pn) {
     const int y0 = n0 * nt / 2, ny = std::min(cols - y0, std::min(pn, all_n - n0) * nt / 2);
-    cut<kReal>(L, Y, y0, ny, 0, g.K, Kp, nt, KB, f->ey, f->B);
+    if (!(pn >= all_n && yK == g.K && ycols == cols)) cut<kReal>(L, Y, y0, ny, 0, g.K, Kp, nt, KB, f->ey, f->B);
     for (int m0 = 0; m0 < all_m; m0 += pm) {
       const int r0 = m0 * kTM, nr = (int)std::min<long long>(rows - r0, (long long)std::min(pm, all_m - m0) * kTM);
       if (n0 == 0 || pm < all_m) cut<kRows>(L, X, r0, nr, 0, g.K, Kp, kTM, KB, f->ex, f->A);
@@ -817,6 +837,10 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
       else launch_gemm<1>(L, t, ctas, "fp64_tc_gemm_pair");
     }
   }
+  if (pn >= all_n) {
+    f->yK = g.K;
+    f->ycols = cols;
+  }
   return true;
 }
 
@@ -824,6 +848,7 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
 bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g) {
   Fp64Tc *f = L.ftc;
   if (!f) return false;
+  f->yK = 0;
   const int alpha = unit_of(g.alpha);
   if (alpha < 0 || (g.beta != 0.0 && g.beta != 1.0)) return false;
   const long long Kl = (long long)g.K * g.batch;
@@ -835,7 +860,8 @@ bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g) {
   const int mtiles = (2 * g.M + kTM - 1) / kTM, ntiles = (2 * g.N + nt - 1) / nt;
   const int splits_max = f->sms / (mtiles * ntiles);   // one unit per CTA
   if (splits_max < 1) return false;
-  const size_t a_seg = (size_t)mtiles * kSeg * kABlk, b_seg = (size_t)ntiles * kSeg * kDig * nt * 32;   // bytes per segment
+  constexpr int kDig = digits_of(true);
+  const size_t a_seg = (size_t)mtiles * kSeg * kDig * kADig, b_seg = (size_t)ntiles * kSeg * kDig * nt * 32;   // bytes per segment
   const int all_segs = (K + kSeg * kKB - 1) / (kSeg * kKB);
   int ps = (int)std::min<size_t>(all_segs, std::min(f->a_bytes / a_seg, f->b_bytes / b_seg));
   ps = (int)std::min<long long>(ps, f->exps / std::max(g.M, g.N));
@@ -861,7 +887,7 @@ bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g) {
     launch_gemm<2>(L, t, t.splits * mtiles * ntiles, "fp64_tc_gemm_long");
   }
   L.before("fp64_tc_reduce");
-  fp64_tc_reduce_kernel<<<(g.M * g.N + 7) / 8, 256, 0, L.stream>>>(t);
+  launch_dependent(fp64_tc_reduce_kernel, (g.M * g.N + 7) / 8, 256, 0, L.stream, t);
   L.after_launch();
   return true;
 }

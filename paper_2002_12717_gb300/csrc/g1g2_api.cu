@@ -87,6 +87,7 @@ struct g1g2_ctx {
   bool hub_gw = false;
   cplx *Gss = nullptr, *Gss_s = nullptr, *Gss_acc = nullptr, *Cb2 = nullptr;
   double *hub_U = nullptr;                      // U_i = w_iiii
+  int hub_nnz = 0;
   int *hub_rp = nullptr, *hub_ci = nullptr;     // CSR pattern of h^HF (h, D, diagonal), symmetric
   std::vector<unsigned char> hub_hpat;          // nonzero pattern of h (host)
   int adj_where = G1G2_CKPT_AUTO;               // where the adjoint keeps its checkpoints
@@ -202,9 +203,9 @@ struct StageOut {
   cplx *Gy, *Gys, *Gacc, *Gk;
 };
 
-void mode_left1(g1g2_ctx *c, Launcher &L, const cplx *S, const cplx *X, cplx *out, cplx alpha, double beta);
-void mode_left2(g1g2_ctx *c, Launcher &L, const cplx *S, const cplx *X, cplx *out, cplx alpha, double beta);
-void mode_right4(g1g2_ctx *c, Launcher &L, const cplx *X, const cplx *S, cplx *out, cplx alpha, double beta);
+void mode_left1(g1g2_ctx *c, Launcher &L, const cplx *S, const cplx *X, cplx *out, cplx alpha, double beta, bool same = false);
+void mode_left2(g1g2_ctx *c, Launcher &L, const cplx *S, const cplx *X, cplx *out, cplx alpha, double beta, bool same = false);
+void mode_right4(g1g2_ctx *c, Launcher &L, const cplx *X, const cplx *S, cplx *out, cplx alpha, double beta, bool same = false);
 
 // a2: I_ij = -i sum_(lp) sum_k wP[lp][i][k] G[lp][j][k]   (Eq. eom_gone-I) into c->I
 void collision(g1g2_ctx *c, Launcher &L, const cplx *G_in) {
@@ -244,6 +245,7 @@ void source_A(g1g2_ctx *c, Launcher &L, const cplx *n_in) {
     g.A = n_in; g.sa_m = 1; g.sa_k = N;
     g.B = c->T1; g.sb_b = N2; g.sb_k = N; g.sb_n = 1;
     g.C = c->T2; g.sc_b = N2; g.sc_m = N; g.sc_n = 1;
+    g.same_small = true;
     zgemm(L, g);
   }
   {
@@ -260,6 +262,7 @@ void source_A(g1g2_ctx *c, Launcher &L, const cplx *n_in) {
     g.A = c->nbar; g.sa_m = N; g.sa_k = 1;
     g.B = c->T1; g.sb_k = N3; g.sb_n = 1;
     g.C = c->Ab; g.sc_m = N3; g.sc_n = 1;
+    g.same_small = true;
     zgemm(L, g);
   }
 }
@@ -325,7 +328,7 @@ void rhs_fp64(g1g2_ctx *c, Launcher &L, double t, const cplx *n_in, const cplx *
   const cplx *h = w_only ? c->zero_h : c->h, *D = !w_only && c->hasD ? c->D : nullptr;
   if (c->hub_on && c->se != G1G2_HF) {
     HubStage p{};
-    p.nb = nb; p.rp = c->hub_rp; p.ci = c->hub_ci; p.h = h; p.D = D; p.f = f; p.U = c->hub_U;
+    p.nb = nb; p.nnz = c->hub_nnz; p.rp = c->hub_rp; p.ci = c->hub_ci; p.h = h; p.D = D; p.f = f; p.U = c->hub_U;
     p.n = n_in; p.G = G_in; p.stage = st.stage; p.dt = st.dt;
     p.ny = o.ny; p.nys = o.nys; p.nacc = o.nacc; p.nk = o.nk;
     p.Gy = o.Gy; p.Gys = o.Gys; p.Gacc = o.Gacc; p.Gk = o.Gk;
@@ -362,7 +365,7 @@ void rhs_fp64(g1g2_ctx *c, Launcher &L, double t, const cplx *n_in, const cplx *
     g.A = c->hhf; g.sa_m = N; g.sa_k = 1;
     g.B = G_in; g.sb_b = N3; g.sb_k = N2; g.sb_n = 1;
     g.C = c->Cb; g.sc_b = N3; g.sc_m = N2; g.sc_n = 1;
-    g.beta = 1.0;
+    g.beta = 1.0; g.same_small = true;
     zgemm(L, g);
   }
   {
@@ -380,7 +383,7 @@ void rhs_fp64(g1g2_ctx *c, Launcher &L, double t, const cplx *n_in, const cplx *
     g.A = G_in; g.sa_m = N; g.sa_k = 1;
     g.B = c->hhf; g.sb_k = N; g.sb_n = 1;
     g.C = c->Cb; g.sc_m = N; g.sc_n = 1;
-    g.alpha = {-1.0, 0.0}; g.beta = 1.0;
+    g.alpha = {-1.0, 0.0}; g.beta = 1.0; g.same_small = true;
     zgemm(L, g);
   }
   // a4: Eq. (psi-pm-def) by successive contractions into A; Psi = -A + A^dag in the assembly
@@ -590,48 +593,44 @@ void contract3(g1g2_ctx *c, Launcher &L, int mode, const cplx *X, const cplx *Z,
   zgemm_reduce(L, g, c->partial, c->splits);
 }
 
-// Mode products on nb^4 tensors: right products over index 4 or 3, left products over 1 or 2.
-void mode_right4(g1g2_ctx *c, Launcher &L, const cplx *X, const cplx *S, cplx *out, cplx alpha, double beta) {
+// Mode products on nb^4 tensors: right products over index 4 or 3, left products over 1 or 2.  same: S is the matrix of
+// the previous product, applied from the same side (see ZGemm::same_small).
+void mode_right4(g1g2_ctx *c, Launcher &L, const cplx *X, const cplx *S, cplx *out, cplx alpha, double beta, bool same) {
   const long long N = c->nb;
   ZGemm g;
   g.M = (int)(N * N * N); g.N = c->nb; g.K = c->nb;
   g.A = X; g.sa_m = N; g.sa_k = 1; g.B = S; g.sb_k = N; g.sb_n = 1;
   g.C = out; g.sc_m = N; g.sc_n = 1; g.alpha = alpha; g.beta = beta;
+  g.same_small = same;
   zgemm(L, g);
 }
-void mode_right3(g1g2_ctx *c, Launcher &L, const cplx *X, const cplx *S, cplx *out, cplx alpha, double beta) {
+void mode_right3(g1g2_ctx *c, Launcher &L, const cplx *X, const cplx *S, cplx *out, cplx alpha, double beta, bool same = false) {
   const long long N = c->nb, N2 = N * N;
   ZGemm g;
   g.M = c->nb; g.N = c->nb; g.K = c->nb; g.batch = (int)N2;
   g.A = S; g.sa_m = 1; g.sa_k = N; g.B = X; g.sb_b = N2; g.sb_k = N; g.sb_n = 1;
   g.C = out; g.sc_b = N2; g.sc_m = N; g.sc_n = 1; g.alpha = alpha; g.beta = beta;
+  g.same_small = same;
   zgemm(L, g);
 }
-void mode_left2(g1g2_ctx *c, Launcher &L, const cplx *S, const cplx *X, cplx *out, cplx alpha, double beta) {
+void mode_left2(g1g2_ctx *c, Launcher &L, const cplx *S, const cplx *X, cplx *out, cplx alpha, double beta, bool same) {
   const long long N = c->nb, N2 = N * N, N3 = N2 * N;
   ZGemm g;
   g.M = c->nb; g.N = (int)N2; g.K = c->nb; g.batch = c->nb;
   g.A = S; g.sa_m = N; g.sa_k = 1; g.B = X; g.sb_b = N3; g.sb_k = N2; g.sb_n = 1;
   g.C = out; g.sc_b = N3; g.sc_m = N2; g.sc_n = 1; g.alpha = alpha; g.beta = beta;
+  g.same_small = same;
   zgemm(L, g);
 }
-void mode_left1(g1g2_ctx *c, Launcher &L, const cplx *S, const cplx *X, cplx *out, cplx alpha, double beta) {
+void mode_left1(g1g2_ctx *c, Launcher &L, const cplx *S, const cplx *X, cplx *out, cplx alpha, double beta, bool same) {
   const long long N = c->nb, N3 = N * N * N;
   ZGemm g;
   g.M = c->nb; g.N = (int)N3; g.K = c->nb;
   g.A = S; g.sa_m = N; g.sa_k = 1; g.B = X; g.sb_k = N3; g.sb_n = 1;
   g.C = out; g.sc_m = N3; g.sc_n = 1; g.alpha = alpha; g.beta = beta;
+  g.same_small = same;
   zgemm(L, g);
 }
-void matmul(g1g2_ctx *c, Launcher &L, const cplx *A, const cplx *B, cplx *out, cplx alpha, double beta) {
-  const long long N = c->nb;
-  ZGemm g;
-  g.M = c->nb; g.N = c->nb; g.K = c->nb;
-  g.A = A; g.sa_m = N; g.sa_k = 1; g.B = B; g.sb_k = N; g.sb_n = 1;
-  g.C = out; g.sc_m = N; g.sc_n = 1; g.alpha = alpha; g.beta = beta;
-  zgemm(L, g);
-}
-
 // Vector-Jacobian product of the FP64 right-hand side at (t, n, G): given the
 // cotangents (a, Y) of (dn, dG2), write the cotangents nbar of n, Gbar of G2
 // and hbar of h^HF (which is also the cotangent of the explicit h(t)); with wbar
@@ -646,8 +645,7 @@ void vjp_fp64(g1g2_ctx *c, Launcher &L, double t, const cplx *n, const cplx *G, 
   const double f = drive_f(c, t);
   hf_build(L, nb, c->Wm, c->w_real, c->h, c->hasD ? c->D : nullptr, f, n, c->hhf);
   // dn = -i [hHF, n] - (I + I^dag): cotangent of hHF from the commutator: i [a, n]
-  matmul(c, L, a, n, hbar, I1, 0.0);
-  matmul(c, L, n, a, hbar, mI, 1.0);
+  commutator_i(L, nb, a, n, hbar);
   const bool corr = c->se != G1G2_HF;
   if (corr) {
     // dG2 = -i [h2(hHF), G2] - i Psi: cotangent of hHF from the commutator
@@ -657,8 +655,7 @@ void vjp_fp64(g1g2_ctx *c, Launcher &L, double t, const cplx *n, const cplx *G, 
     contract3(c, L, 4, Y, G, mI, 1.0, hbar);
   }
   // nbar = i [hHF, a] + (adjoint of the Hartree-Fock build)(hbar)
-  matmul(c, L, c->hhf, a, nbar, I1, 0.0);
-  matmul(c, L, a, c->hhf, nbar, mI, 1.0);
+  commutator_i(L, nb, c->hhf, a, nbar);
   hf_build_t(L, nb, c->Wm, c->w_real, hbar, nbar, true);
   const bool restricted = c->basis == G1G2_SPIN_RESTRICTED;
   // wbar from Eq. (h_HF): Wm[(ij),(lk)] = w_ikjl + eta w_iklj (restricted: w_ikjl)
@@ -669,9 +666,9 @@ void vjp_fp64(g1g2_ctx *c, Launcher &L, double t, const cplx *n, const cplx *G, 
   }
   // Gbar = i [h2(hHF), Y]  (the commutator map is anti-Hermitian)
   mode_left1(c, L, c->hhf, Y, Gbar, I1, 0.0);
-  mode_left2(c, L, c->hhf, Y, Gbar, I1, 1.0);
+  mode_left2(c, L, c->hhf, Y, Gbar, I1, 1.0, true);
   mode_right3(c, L, Y, c->hhf, Gbar, mI, 1.0);
-  mode_right4(c, L, Y, c->hhf, Gbar, mI, 1.0);
+  mode_right4(c, L, Y, c->hhf, Gbar, mI, 1.0, true);
   // collision integral I_ij = -i sum w_iklp G2_lpjk, cotangent Ibar = -(a + a^dag):
   // Gbar_lpjk += i sum_i w_iklp Ibar_ij  (batched over (lp) with wP[(lp)][i][k] = w_iklp)
   herm_sum(L, nb, mone, a, c->I);
@@ -698,17 +695,17 @@ void vjp_fp64(g1g2_ctx *c, Launcher &L, double t, const cplx *n, const cplx *G, 
   tconj_add(L, nb, mI, Y, c->AE);
   one_minus(L, nb, n, c->nbar);
   mode_right4(c, L, c->wsrc, n, c->T1, one, 0.0);          // T1_pqrl = sum_s w~_pqrs n_sl
-  mode_right3(c, L, c->T1, n, c->T2, one, 0.0);            // T2_pqkl = sum_r n_rk T1_pqrl
+  mode_right3(c, L, c->T1, n, c->T2, one, 0.0, true);      // T2_pqkl = sum_r n_rk T1_pqrl
   mode_left2(c, L, c->nbar, c->T2, c->AB1, one, 0.0);      // B1 = nbar x_2 T2
   contract3(c, L, 1, c->AE, c->AB1, mone, 1.0, nbar);
   mode_left1(c, L, c->nbar, c->T2, c->AB1, one, 0.0);      // B2 = nbar x_1 T2
   contract3(c, L, 2, c->AE, c->AB1, mone, 1.0, nbar);
   mode_left2(c, L, c->nbar, c->T1, c->AB1, one, 0.0);
-  mode_left1(c, L, c->nbar, c->AB1, c->AB2, one, 0.0);     // B3 = nbar x_1 nbar x_2 T1
+  mode_left1(c, L, c->nbar, c->AB1, c->AB2, one, 0.0, true);   // B3 = nbar x_1 nbar x_2 T1
   contract3(c, L, 3, c->AE, c->AB2, one, 1.0, nbar);
   mode_right3(c, L, c->wsrc, n, c->AB1, one, 0.0);         // T1'_pqks = sum_r w~_pqrs n_rk
   mode_left2(c, L, c->nbar, c->AB1, c->T2, one, 0.0);
-  mode_left1(c, L, c->nbar, c->T2, c->AB2, one, 0.0);      // B4 = nbar x_1 nbar x_2 T1'
+  mode_left1(c, L, c->nbar, c->T2, c->AB2, one, 0.0, true);    // B4 = nbar x_1 nbar x_2 T1'
   contract3(c, L, 4, c->AE, c->AB2, one, 1.0, nbar);
   if (wbar) {
     // A = (nbar (x) nbar) w~ (n (x) n): w~bar_pqrs = sum_ijkl nbar_pi nbar_qj E_ijkl n_kr n_ls
@@ -884,6 +881,7 @@ int hub_upload_pattern(g1g2_ctx *c, const std::vector<cplx> *D) {
     }
     rp[i + 1] = (int)ci.size();
   }
+  c->hub_nnz = (int)ci.size();
   if (cudaMemcpyAsync(c->hub_rp, rp.data(), rp.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream) !=
           cudaSuccess ||
       cudaMemcpyAsync(c->hub_ci, ci.data(), ci.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream) !=

@@ -62,6 +62,30 @@ struct Launcher {
   }
 };
 
+// Launch that may begin while the previous kernel of the stream still runs (programmatic dependent launch): the
+// kernel calls dependent_begin() before it reads or writes global memory, which lets the next one start and
+// waits until the previous kernels have finished.  At nb <= 32 the kernels of a right-hand side last 8 to 30 us
+// each, of which the launch and the set-up hidden this way are about two.
+template <class... KArgs, class... Args>
+inline void launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                             Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+__device__ __forceinline__ void dependent_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Generic strided complex FP64 GEMM, batched:
 //   C_b[m][n] = alpha * sum_k opA(A_b[m][k]) * opB(B_b[k][n]) + beta * C_b[m][n]
 // (reduce = false), or C[m][n] = alpha * sum_b sum_k ... + beta * C (reduce = true).
@@ -73,6 +97,9 @@ struct ZGemm {
   cplx alpha{1.0, 0.0};
   double beta = 0.0;
   bool conjA = false, conjB = false;
+  // the operand with fewer rows (its matrix, strides and contents) is that of the previous product of this stream of
+  // calls: the tensor-core form then keeps its digits
+  bool same_small = false;
 };
 void zgemm(Launcher &L, const ZGemm &g);
 void zgemm_reduce(Launcher &L, const ZGemm &g, cplx *partial, int splits);
@@ -127,6 +154,7 @@ void g2_assemble(Launcher &L, int nb, const cplx *Cb, const cplx *Ab, Rk4Stage s
 struct HubStage {
   int nb;
   const int *rp, *ci;
+  int nnz;                 // rp[nb]
   const cplx *h, *D;       // D null without a drive
   double f;
   const double *U;
@@ -156,6 +184,8 @@ void zaxpby(Launcher &L, long long n, cplx alpha, const cplx *x, cplx beta, cons
 void tconj_add(Launcher &L, int nb, cplx c, const cplx *Y, cplx *out);
 void herm_sum(Launcher &L, int nb, cplx c, const cplx *a, cplx *out);
 void real_dot_acc(Launcher &L, long long n, const cplx *x, const cplx *y, double coeff, double *partials, double *acc);
+// out = i (A B - B A) for nb x nb matrices
+void commutator_i(Launcher &L, int nb, const cplx *A, const cplx *B, cplx *out);
 void hf_build_t(Launcher &L, int nb, const void *Wm, bool wm_real, const cplx *x, cplx *out, bool accumulate);
 // Cotangent of w through the Hartree-Fock matrix Wm[(ij),(lk)] = w_ikjl + eta w_iklj given the
 // cotangent x of h^HF at the state n: wbar_abcd += c (x_ac conj(n_db) + eta x_ad conj(n_cb)).
