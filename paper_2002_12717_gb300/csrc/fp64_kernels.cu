@@ -22,11 +22,7 @@ __device__ __forceinline__ cplx mul_minus_i(cplx z) { return {z.y, -z.x}; }
 
 // ---------------------------------------------------------------------------
 // Strided batched complex GEMM (FP64 CUDA cores).
-// Tile 32x32x16, 64 threads, each thread a 4x4 micro-tile strided by 8.
 // ---------------------------------------------------------------------------
-constexpr int GBM = 32, GBN = 32, GBK = 16, GTM = 4, GTN = 4;
-constexpr int GNT = (GBM / GTM) * (GBN / GTN);  // 64
-
 struct ZGemmDev {
   int M, N, K, batch;
   const cplx *A; long long sa_b, sa_m, sa_k;
@@ -36,112 +32,52 @@ struct ZGemmDev {
   int conjA, conjB;
 };
 
-// Micro-tile product over kcount k-steps of the staged tiles: rows ty + 8 i (i < TI),
-// columns tx + 8 j (j < TJ).  TI, TJ < 4 serve tiles whose valid extent is at most 8
-// rows or columns, and kcount < GBK a ragged K tile, so that padding costs no DFMA
-// (the FP64 pipe is the bound of this kernel).
-template <int TI, int TJ, bool kFullK>
-__device__ __forceinline__ void tile_fma(const cplx (*As)[GBM + 1], const cplx (*Bs)[GBN + 1], int ty, int tx,
-                                         int kcount, cplx (&acc)[GTM][GTN]) {
-  const int kn = kFullK ? GBK : kcount;
-#pragma unroll 4
-  for (int kk = 0; kk < kn; ++kk) {
-    cplx a[TI], bb[TJ];
-#pragma unroll
-    for (int i = 0; i < TI; ++i) a[i] = As[kk][ty + i * (GBM / GTM)];
-#pragma unroll
-    for (int j = 0; j < TJ; ++j) bb[j] = Bs[kk][tx + j * (GBN / GTN)];
-#pragma unroll
-    for (int i = 0; i < TI; ++i)
-#pragma unroll
-      for (int j = 0; j < TJ; ++j) acc[i][j] = cfma(a[i], bb[j], acc[i][j]);
-  }
-}
-
-// reduce != 0: split-K form.  The reduction runs over (batch, K); it is cut
-// into batch * kparts units (unit u: batch u / kparts, K range
-// [(u % kparts) * klen, ...)), and split z sums units [z * per_split, ...)
-// into partial[z].
-// TI, TJ: micro-tile rows and columns computed per thread (GTM, GTN for operands wider
-// than 8 in M and N; 1 where that extent is at most 8, chosen by the host per GEMM).
-template <int TI, int TJ>
-__global__ void __launch_bounds__(GNT) zgemm_kernel(ZGemmDev g, int reduce, int per_split, cplx *partial, int kparts,
-                                                     int klen) {
+// One output element per thread, the operands read through L1.  Bound by the FP64 pipe: a complex multiply-add is
+// four DFMAs, 64 cycles of it per warp, next to which two 16-byte loads per lane (8 to 32 cycles of the load unit,
+// by their strides) are free.  So no tile in shared memory is needed, and none pays for padding: a
+// 32 x 32 x 16 tile with 4 x 4 outputs per thread did ten times the multiply-adds of a batched 12 x 12 x 12 product on 54
+// of the 152 SMs (mode product at nb = 12: 41 us with it, 4.6 us with this kernel).
+// kReduce: split blockIdx.y sums c = (b, k) of [blockIdx.y len, ...) into partial[blockIdx.y].
+constexpr int kZThreads = 64;   // small CTAs: a product at nb = 8 has 4096 outputs for 152 SMs
+template <bool kReduce>
+__global__ void __launch_bounds__(kZThreads) zgemm_kernel(const ZGemmDev g, long long len, cplx *__restrict__ partial) {
   dependent_begin();
-  __shared__ cplx As[GBK][GBM + 1];
-  __shared__ cplx Bs[GBK][GBN + 1];
-  const int tid = threadIdx.x;
-  const int tx = tid % (GBN / GTN), ty = tid / (GBN / GTN);
-  const int m0 = blockIdx.y * GBM, n0 = blockIdx.x * GBN;
-
-  long long b_begin, b_end, b_step;
-  if (reduce) {
-    b_begin = (long long)blockIdx.z * per_split;
-    b_end = min((long long)g.batch * kparts, b_begin + per_split);
-    b_step = 1;
-  } else {
-    b_begin = blockIdx.z;
-    b_end = g.batch;
-    b_step = gridDim.z;
-  }
-  for (long long b0 = b_begin; b0 < b_end; b0 += (reduce ? (b_end - b_begin) : b_step)) {
-    cplx acc[GTM][GTN];
-#pragma unroll
-    for (int i = 0; i < GTM; ++i)
-#pragma unroll
-      for (int j = 0; j < GTN; ++j) acc[i][j] = {0.0, 0.0};
-    const long long bl = reduce ? b_end : b0 + 1;
-    for (long long u = b0; u < bl; ++u) {
-      const long long b = reduce ? u / kparts : u;
-      const int kbeg = reduce ? (int)(u % kparts) * klen : 0;
-      const int kend = reduce ? min(g.K, kbeg + klen) : g.K;
-      const cplx *A = g.A + b * g.sa_b;
-      const cplx *B = g.B + b * g.sb_b;
-      for (int k0 = kbeg; k0 < kend; k0 += GBK) {
-        for (int idx = tid; idx < GBM * GBK; idx += GNT) {
-          int m, k;
-          if (g.sa_k == 1) { m = idx / GBK; k = idx % GBK; } else { k = idx / GBM; m = idx % GBM; }
-          cplx v = {0.0, 0.0};
-          if (m0 + m < g.M && k0 + k < kend) v = A[(long long)(m0 + m) * g.sa_m + (long long)(k0 + k) * g.sa_k];
-          if (g.conjA) v.y = -v.y;
-          As[k][m] = v;
-        }
-        for (int idx = tid; idx < GBN * GBK; idx += GNT) {
-          int n, k;
-          if (g.sb_n == 1) { k = idx / GBN; n = idx % GBN; } else { n = idx / GBK; k = idx % GBK; }
-          cplx v = {0.0, 0.0};
-          if (n0 + n < g.N && k0 + k < kend) v = B[(long long)(k0 + k) * g.sb_k + (long long)(n0 + n) * g.sb_n];
-          if (g.conjB) v.y = -v.y;
-          Bs[k][n] = v;
-        }
-        __syncthreads();
-        // the full micro-tile runs the whole (zero-padded) K tile: a runtime trip count
-        // there costs registers, and wide GEMMs have few ragged K tiles
-        if (TI == GTM && TJ == GTN) tile_fma<TI, TJ, true>(As, Bs, ty, tx, GBK, acc);
-        else tile_fma<TI, TJ, false>(As, Bs, ty, tx, min(GBK, kend - k0), acc);
-        __syncthreads();
+  const long long mn = (long long)g.M * g.N, total = kReduce ? mn : mn * g.batch;
+  const int fa = g.conjA ? (int)0x80000000u : 0, fb = g.conjB ? (int)0x80000000u : 0;   // signs on the integer pipe
+  auto flip = [](double x, int f) { return __hiloint2double(__double2hiint(x) ^ f, __double2loint(x)); };
+  for (long long idx = (long long)blockIdx.x * kZThreads + threadIdx.x; idx < total;
+       idx += (long long)gridDim.x * kZThreads) {
+    const long long b0 = kReduce ? 0 : idx / mn, e = idx - b0 * mn;
+    const int m = (int)(e / g.N), n = (int)(e - (long long)m * g.N);
+    const cplx *A = g.A + b0 * g.sa_b + (long long)m * g.sa_m;
+    const cplx *B = g.B + b0 * g.sb_b + (long long)n * g.sb_n;
+    cplx acc = {0.0, 0.0};
+    auto run = [&](const cplx *pa, const cplx *pb, int kn) {
+#pragma unroll 4
+      for (int k = 0; k < kn; ++k) {
+        cplx x = pa[(long long)k * g.sa_k], y = pb[(long long)k * g.sb_k];
+        x.y = flip(x.y, fa);
+        y.y = flip(y.y, fb);
+        acc = cfma(x, y, acc);
       }
-    }
-    // epilogue
-#pragma unroll
-    for (int i = 0; i < GTM; ++i) {
-      const int m = m0 + ty + i * (GBM / GTM);
-      if (m >= g.M) continue;
-#pragma unroll
-      for (int j = 0; j < GTN; ++j) {
-        const int n = n0 + tx + j * (GBN / GTN);
-        if (n >= g.N) continue;
-        if (reduce) {
-          partial[((long long)blockIdx.z * g.M + m) * g.N + n] = acc[i][j];
-        } else {
-          cplx *c = g.C + b0 * g.sc_b + (long long)m * g.sc_m + (long long)n * g.sc_n;
-          cplx r = cmul(g.alpha, acc[i][j]);
-          if (g.beta != 0.0) r = cadd(r, cscale(*c, g.beta));
-          *c = r;
-        }
+    };
+    if (!kReduce) {
+      run(A, B, g.K);
+      cplx *c = g.C + b0 * g.sc_b + (long long)m * g.sc_m + (long long)n * g.sc_n;
+      cplx r = cmul(g.alpha, acc);
+      if (g.beta != 0.0) r = cadd(r, cscale(*c, g.beta));
+      *c = r;
+    } else {
+      long long c0 = (long long)blockIdx.y * len;
+      const long long c1 = min((long long)g.K * g.batch, c0 + len);
+      while (c0 < c1) {
+        const long long b = c0 / g.K;
+        const int k0 = (int)(c0 - b * g.K), kn = (int)min((long long)(g.K - k0), c1 - c0);
+        run(A + b * g.sa_b + (long long)k0 * g.sa_k, B + b * g.sb_b + (long long)k0 * g.sb_k, kn);
+        c0 += kn;
       }
+      partial[(long long)blockIdx.y * mn + e] = acc;
     }
-    if (reduce) break;
   }
 }
 
@@ -803,40 +739,25 @@ __global__ void count_nonfinite_kernel(const cplx *x, long long len, double *cnt
 // ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
-// Rows (columns) beyond 8 of a tile exist only when M (N) exceeds 8; narrower GEMMs
-// run the 1-row (1-column) micro-tile so that no DFMA is spent on padding.
-void launch_zgemm(dim3 grid, cudaStream_t st, const ZGemm &g, int reduce, int per, cplx *partial, int kparts,
-                  int klen) {
-  const bool mw = g.M > GBM / GTM, nw = g.N > GBN / GTN;
-  if (mw && nw) launch_dependent(zgemm_kernel<GTM, GTN>, grid, GNT, 0, st, to_dev(g), reduce, per, partial, kparts, klen);
-  else if (mw) launch_dependent(zgemm_kernel<GTM, 1>, grid, GNT, 0, st, to_dev(g), reduce, per, partial, kparts, klen);
-  else if (nw) launch_dependent(zgemm_kernel<1, GTN>, grid, GNT, 0, st, to_dev(g), reduce, per, partial, kparts, klen);
-  else launch_dependent(zgemm_kernel<1, 1>, grid, GNT, 0, st, to_dev(g), reduce, per, partial, kparts, klen);
-}
-
 void zgemm(Launcher &L, const ZGemm &g) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
   if (fp64_tc_zgemm(L, g)) return;
-  dim3 grid((g.N + GBN - 1) / GBN, (g.M + GBM - 1) / GBM, std::min(g.batch, 65535));
+  const long long total = (long long)g.M * g.N * g.batch;
+  const unsigned grid = (unsigned)std::min<long long>((total + kZThreads - 1) / kZThreads, 1 << 20);
   L.before("fp64_zgemm");
-  launch_zgemm(grid, L.stream, g, 0, 1, nullptr, 1, g.K);
+  launch_dependent(zgemm_kernel<false>, grid, kZThreads, 0, L.stream, to_dev(g), 0ll, (cplx *)nullptr);
   L.after_launch();
 }
 
 void zgemm_reduce(Launcher &L, const ZGemm &g, cplx *partial, int splits) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
   if (fp64_tc_zgemm_reduce(L, g)) return;
-  // cut K as well when the batch alone gives fewer units than splits
-  const int kblocks = (g.K + GBK - 1) / GBK;
-  const int kparts = std::max(1, std::min(kblocks, (splits + g.batch - 1) / g.batch));
-  const int klen = ((kblocks + kparts - 1) / kparts) * GBK;
-  const long long units = (long long)g.batch * kparts;
-  splits = (int)std::max(1LL, std::min((long long)splits, units));
-  const int per = (int)((units + splits - 1) / splits);
-  splits = (int)((units + per - 1) / per);
-  dim3 grid((g.N + GBN - 1) / GBN, (g.M + GBM - 1) / GBM, splits);
+  // as many splits as fit the buffer, of at least 16 terms each: one of nb = 12 then lasts 2 us
+  const long long Kl = (long long)g.K * g.batch, len = std::max<long long>(16, (Kl + splits - 1) / splits);
+  splits = (int)std::max<long long>(1, (Kl + len - 1) / len);
+  const dim3 grid((unsigned)std::min<long long>(((long long)g.M * g.N + kZThreads - 1) / kZThreads, 1 << 20), splits);
   L.before("fp64_zgemm_splitk");
-  launch_zgemm(grid, L.stream, g, 1, per, partial, kparts, klen);
+  launch_dependent(zgemm_kernel<true>, grid, kZThreads, 0, L.stream, to_dev(g), len, partial);
   L.after_launch();
   const long long mn = (long long)g.M * g.N;
   L.before("fp64_splitk_reduce");

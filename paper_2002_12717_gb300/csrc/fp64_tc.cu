@@ -148,17 +148,24 @@ __host__ __device__ constexpr int cut_rows(int form) { return kCutVals / seg_k(f
 // row there, and every thread then cuts eight consecutive K values of one row at a time into seven (eight)
 // 16-byte stores; a warp writes 16 rows x 32 bytes, 512 contiguous bytes, per digit.  Bound by its 16
 // bytes read and 28 written per complex element (56 for kReal).
+struct CutJob {
+  Operand o;               // o.rows: rows of the panel
+  int r_begin, TR;
+  int *rexp;
+  uint8_t *out;
+};
 template <int FORM>
-__global__ void __launch_bounds__(256) cut_digits_kernel(const Operand A, int r_begin, int k_begin, int Klen, int Kp,
-                                                         int TR, int KB, int *__restrict__ rexp,
-                                                         uint8_t *__restrict__ out) {
+__device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_begin, int Klen, int Kp, int KB) {
   constexpr int SK = seg_k(FORM), SR = cut_rows(FORM), ND = digits_of(FORM == kPlanes);
   extern __shared__ double sh[];
   __shared__ long long roff[SR], koff[SK];
   __shared__ int emax[SR];
-  dependent_begin();
+  const Operand &A = job.o;
+  const int r_begin = job.r_begin, TR = job.TR;
+  int *__restrict__ rexp = job.rexp;
+  uint8_t *__restrict__ out = job.out;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int r0 = blockIdx.x * SR;                         // within the panel
+  const int r0 = block * SR;                              // within the panel
   const int nr = min(SR, A.rows - r0);                    // A.rows: rows of the panel
   const int seg = blockIdx.y, k0 = seg * SK;
   const int kt = min(SK, Kp - k0);                        // padded K values of this segment (multiple of 8)
@@ -222,6 +229,16 @@ __global__ void __launch_bounds__(256) cut_digits_kernel(const Operand A, int r_
       store_digits<ND>(out, TR, KB, 2 * row + u, q0 + kc, w, 0u);
     }
   }
+}
+
+// Both operands of a product in one launch: blocks below xblocks cut x, the others y.  (The column operand is small: as
+// a launch of its own it took 5 us of the 50 us of a mode product at nb = 32.)
+template <int FX, int FY>
+__global__ void __launch_bounds__(256) cut_digits_kernel(const CutJob x, const CutJob y, int xblocks, int k_begin, int Klen,
+                                                         int Kp, int KB) {
+  dependent_begin();
+  if ((int)blockIdx.x < xblocks) cut_digits<FX>(x, blockIdx.x, k_begin, Klen, Kp, KB);
+  else cut_digits<FY>(y, blockIdx.x - xblocks, k_begin, Klen, Kp, KB);
 }
 
 // ---------------------------------------------------------------------------
@@ -681,9 +698,21 @@ int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
 // Real columns per tile: as few tiles of at most 128 as the columns need, evenly filled.  Up to 64 columns
 // run with all orders in TMEM at once (G = 8).
-int tile_columns(int real_cols) {
-  const int tiles = (real_cols + kTNMax - 1) / kTNMax;
-  return round_up((real_cols + tiles - 1) / tiles, 16);
+int even_tiles(int real_cols, int tiles) { return round_up((real_cols + tiles - 1) / tiles, 16); }
+int tile_columns(int real_cols) { return even_tiles(real_cols, (real_cols + kTNMax - 1) / kTNMax); }
+// The same for a product of several segments, which lasts as many rounds of MMAs as the busiest CTA has tiles: the width
+// with the least rounds times cost of an MMA (see the kernel).  128 columns everywhere left nb = 24 (45 tiles) and nb = 27
+// (72) with most SMs idle: 177 and 242 us.
+int tile_columns(int real_cols, int mtiles, int sms) {
+  int best = 0;
+  long long cost = 0;
+  for (int w = kTNMax; w >= 16; w -= 16) {
+    const int nt = even_tiles(real_cols, (real_cols + w - 1) / w);
+    const long long units = (long long)mtiles * ((real_cols + nt - 1) / nt);
+    const long long c = (units + sms - 1) / sms * (4096 + 32 * nt);
+    if (!best || c < cost) { best = nt; cost = c; }
+  }
+  return best;
 }
 
 template <int kKind>
@@ -694,25 +723,35 @@ void launch_gemm(Launcher &L, const TcGemm &t, int ctas, const char *tag) {
   L.after_launch();
 }
 
-template <int FORM>
-void cut(Launcher &L, const Operand &o, int r_begin, int rows, int k_begin, int Klen, int Kp, int TR, int KB, int *rexp,
-         uint8_t *out) {
-  Operand A = o;
-  A.rows = rows;
-  const int kt = std::min(seg_k(FORM), Kp);
-  const size_t sh = (size_t)2 * cut_rows(FORM) * (kt + 1) * sizeof(double);
-  dim3 grid((rows + cut_rows(FORM) - 1) / cut_rows(FORM), (Kp + seg_k(FORM) - 1) / seg_k(FORM));
+CutJob cut_job(const Operand &o, int r_begin, int rows, int TR, int *rexp, uint8_t *out) {
+  CutJob j{o, r_begin, TR, rexp, out};
+  j.o.rows = rows;
+  return j;
+}
+
+// x and y with rows > 0
+template <int FX, int FY>
+void cut(Launcher &L, const CutJob &x, const CutJob &y, int k_begin, int Klen, int Kp, int KB) {
+  static_assert(seg_k(FX) == seg_k(FY), "one grid of segments");
+  constexpr int SR = cut_rows(FX);
+  const size_t sh = (size_t)2 * SR * (std::min(seg_k(FX), Kp) + 1) * sizeof(double);
+  const int xb = (x.o.rows + SR - 1) / SR, yb = (y.o.rows + SR - 1) / SR;
+  if (xb + yb == 0) return;
+  dim3 grid(xb + yb, (Kp + seg_k(FX) - 1) / seg_k(FX));
   L.before("fp64_tc_digits");
-  launch_dependent(cut_digits_kernel<FORM>, grid, 256, sh, L.stream, A, r_begin, k_begin, Klen, Kp, TR, KB, rexp, out);
+  launch_dependent(cut_digits_kernel<FX, FY>, grid, 256, sh, L.stream, x, y, xb, k_begin, Klen, Kp, KB);
   L.after_launch();
 }
 
 }  // namespace
 
 constexpr int kMinK = 8, kMinCols = 8;
-constexpr double kMinWork = 1e6;
+// Complex multiply-adds from which a product is faster here than on zgemm_kernel: a mode product at nb = 16 takes 12 us
+// there and 20 us here (digits and product), at nb = 20 30 and 24 us; a long contraction 17 and 40 us at nb = 16, 60 and 48 us
+// at nb = 24; an nb^2 x nb^2 x nb^2 product at nb = 12 (3e6) 40 and 30 us.
+constexpr double kMinWork = 2.2e6, kMinWorkLong = 4e6;
 
-int fp64_tc_min_nb() { return 16; }
+int fp64_tc_min_nb(bool pair_products) { return pair_products ? 12 : 17; }
 
 struct Fp64Tc {
   uint8_t *A = nullptr, *B = nullptr;   // digit blocks of the two operands
@@ -723,7 +762,7 @@ struct Fp64Tc {
   double *part = nullptr;               // FP64 sums of a tile per CTA
   int *err = nullptr;
   int sms = 0;
-  int yK = 0, ycols = 0;                // shape of the column operand whose digits B holds whole (0: none)
+  int yK = 0, ycols = 0, ynt = 0;       // shape of the column operand whose digits B holds whole (0: none)
 };
 
 void fp64_tc_destroy(Fp64Tc *f) {
@@ -742,7 +781,7 @@ Fp64Tc *fp64_tc_create(int nb, bool pair_products) {
   auto blocks = [](long long rows, long long Kp, bool lng = false) {
     return (size_t)((rows + 127) / 128 * 128) * (size_t)Kp * 2 * digits_of(lng);
   };
-  const size_t big = blocks(N3, 2 * ((N + 7) / 8 * 8)), pair = pair_products ? blocks(2 * N2, 2 * ((N2 + 7) / 8 * 8)) : 0;
+  const size_t big = blocks(N3, 2 * ((N + 7) / 8 * 8)), pair = pair_products ? blocks(2 * N2 + kTNMax, 2 * ((N2 + 7) / 8 * 8)) : 0;
   const size_t lng = blocks(2 * N, (N3 + 255) / 256 * 256, true);
   f->a_bytes = std::min(kPanelBytes, std::max({big, pair, lng}));
   f->b_bytes = std::min(kPanelBytes, std::max({blocks(2 * N, 2 * ((N + 7) / 8 * 8)), pair, lng}));
@@ -764,8 +803,7 @@ Fp64Tc *fp64_tc_create(int nb, bool pair_products) {
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem) != cudaSuccess) goto bad;
   {
     const int sh = 2 * (kCutVals + 32) * (int)sizeof(double);
-    for (const void *k : {(const void *)cut_digits_kernel<kRows>, (const void *)cut_digits_kernel<kReal>,
-                          (const void *)cut_digits_kernel<kPlanes>})
+    for (const void *k : {(const void *)cut_digits_kernel<kRows, kReal>, (const void *)cut_digits_kernel<kPlanes, kPlanes>})
       if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sh) != cudaSuccess) goto bad;
   }
   return f;
@@ -811,7 +849,7 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
   const int Kp = round_up(g.K, 8), KB = 2 * Kp / kKB, segs = (KB + kSeg - 1) / kSeg;
   if (std::max<long long>(rows, cols) * segs > f->exps) return false;
   X.rows = (int)rows;
-  const int nt = tile_columns(2 * cols);
+  const int nt = segs == 1 ? tile_columns(2 * cols) : tile_columns(2 * cols, (int)((rows + kTM - 1) / kTM), f->sms);
   // panels of whole tiles
   constexpr int kDig = digits_of(false);
   const size_t a_tile = (size_t)KB * kDig * kADig, b_tile = (size_t)KB * kDig * nt * 32;
@@ -820,10 +858,11 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
   if (pm < 1 || pn < 1) return false;
   for (int n0 = 0; n0 < all_n; n0 += pn) {
     const int y0 = n0 * nt / 2, ny = std::min(cols - y0, std::min(pn, all_n - n0) * nt / 2);
-    if (!(pn >= all_n && yK == g.K && ycols == cols)) cut<kReal>(L, Y, y0, ny, 0, g.K, Kp, nt, KB, f->ey, f->B);
+    const bool kept = pn >= all_n && yK == g.K && ycols == cols && f->ynt == nt;
     for (int m0 = 0; m0 < all_m; m0 += pm) {
       const int r0 = m0 * kTM, nr = (int)std::min<long long>(rows - r0, (long long)std::min(pm, all_m - m0) * kTM);
-      if (n0 == 0 || pm < all_m) cut<kRows>(L, X, r0, nr, 0, g.K, Kp, kTM, KB, f->ex, f->A);
+      cut<kRows, kReal>(L, cut_job(X, r0, (n0 == 0 || pm < all_m) ? nr : 0, kTM, f->ex, f->A),
+                        cut_job(Y, y0, (m0 == 0 && !kept) ? ny : 0, nt, f->ey, f->B), 0, g.K, Kp, KB);
       TcGemm t{};
       t.A = f->A; t.B = f->B; t.KB = KB; t.segs = segs; t.nt = nt;
       t.mtiles = (nr + kTM - 1) / kTM; t.ntiles = (2 * ny + nt - 1) / nt;
@@ -840,6 +879,7 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
   if (pn >= all_n) {
     f->yK = g.K;
     f->ycols = cols;
+    f->ynt = nt;
   }
   return true;
 }
@@ -852,7 +892,7 @@ bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g) {
   const int alpha = unit_of(g.alpha);
   if (alpha < 0 || (g.beta != 0.0 && g.beta != 1.0)) return false;
   const long long Kl = (long long)g.K * g.batch;
-  if (Kl > (1ll << 30) || std::min(g.M, g.N) < kMinCols || (double)g.M * g.N * Kl < kMinWork) return false;
+  if (Kl > (1ll << 30) || std::min(g.M, g.N) < kMinCols || (double)g.M * g.N * Kl < kMinWorkLong) return false;
   const int K = (int)Kl;
   Operand X{g.A, 0, g.sa_m, g.sa_k, g.sa_b, g.M, g.K, g.M, K, g.conjA ? 1 : 0};
   Operand Y{g.B, 0, g.sb_n, g.sb_k, g.sb_b, g.N, g.K, g.N, K, g.conjB ? 1 : 0};
@@ -870,8 +910,7 @@ bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g) {
   for (int sg0 = 0; sg0 < all_segs; sg0 += ps) {
     const int ns = std::min(ps, all_segs - sg0), k0 = sg0 * kSeg * kKB, Klen = std::min(K - k0, ns * kSeg * kKB);
     const int Kp = round_up(Klen, kKB), KB = Kp / kKB;
-    cut<kPlanes>(L, X, 0, g.M, k0, Klen, Kp, kTM, KB, f->ex, f->A);
-    cut<kPlanes>(L, Y, 0, g.N, k0, Klen, Kp, nt, KB, f->ey, f->B);
+    cut<kPlanes, kPlanes>(L, cut_job(X, 0, g.M, kTM, f->ex, f->A), cut_job(Y, 0, g.N, nt, f->ey, f->B), k0, Klen, Kp, KB);
     t.A = f->A; t.B = f->B; t.KB = KB; t.segs = ns; t.nt = nt; t.mtiles = mtiles; t.ntiles = ntiles;
     // the first panel is the longest: its split count holds for the later ones
     if (sg0 == 0) {

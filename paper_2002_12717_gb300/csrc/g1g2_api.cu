@@ -1204,8 +1204,8 @@ int g1g2_init(g1g2_ctx **out, int nb, const double *h, const double *w, const do
       return bail(rc);
     c->splits = 4 * 152;
     if ((rc = dalloc(c, &c->partial, (size_t)c->splits * N2))) return bail(rc);
-    if (nb >= fp64_tc_min_nb())
-      c->ftc = fp64_tc_create(nb, !restricted_gw && se != G1G2_SOA);
+    const bool pair_products = !restricted_gw && se != G1G2_SOA;
+    if (nb >= fp64_tc_min_nb(pair_products)) c->ftc = fp64_tc_create(nb, pair_products);
     if ((se == G1G2_GW && !restricted_gw) || se == G1G2_TPH || se == G1G2_DSL) {
       if ((rc = dalloc(c, &c->Hb, N4)) || (rc = dalloc(c, &c->Gp, N4)) || (rc = dalloc(c, &c->Hp, N4)) ||
           (rc = dalloc(c, &c->Pp, N4)))

@@ -71,3 +71,13 @@ def test_non_finite_entries_reach_the_same_outputs(bad):
     assert not np.isfinite(got[hit]).any()
     assert np.isfinite(got[~hit]).all()
     assert np.abs(got[~hit] - clean[~hit]).max() <= 1e-15 * np.abs(clean).max()
+
+
+# around the lines between the CUDA-core and the digit products: pair products from nb = 12, mode products from nb = 19
+# (their padded K and ragged tiles on both sides), split tiles of a pair product at nb = 27
+@pytest.mark.parametrize("nb,se,bosons", [(5, "GW", False), (11, "GW", True), (12, "GWX", False), (13, "TPP", False),
+                                          (14, "DSL", False), (15, "GW", False), (18, "SOA", True), (19, "SOA", False),
+                                          (27, "GW", False)])
+def test_rhs_matches_oracle_across_the_dispatch(nb, se, bosons):
+    """As test_rhs_matches_oracle: 1e-12 of the largest entry."""
+    test_rhs_matches_oracle(nb, se, bosons)
