@@ -33,6 +33,7 @@
 
 #include <algorithm>
 #include <new>
+#include <type_traits>
 
 namespace g1g2 {
 
@@ -51,8 +52,12 @@ constexpr int kKB = 16;                    // K elements per block: one MMA step
 constexpr int kSeg = 16;                   // K blocks of a segment (256 terms)
 constexpr uint32_t kADig = kTM * 32;       // one digit plane of an A block: 4 KB
 constexpr int kStages = 3;
-constexpr int kEpiWarps = 16;
+constexpr int kEpiWarps = 12;              // 128 registers per thread (16 warps: 96, spilled in the epilogue's loop, 412 us
+                                           // instead of 346 per mode product at nb = 64; 8 warps: 378 us)
 constexpr int kThreads = 64 + 32 * kEpiWarps;   // loader warp, MMA warp, epilogue warps
+constexpr int kPerQuarter = kEpiWarps / 4;        // epilogue warps per quarter of the TMEM lanes
+constexpr int kMaxGroups = (kTNMax / 8 + kPerQuarter - 1) / kPerQuarter;   // groups of eight columns per epilogue warp
+static_assert(kMaxGroups * 4 <= 32, "one lane per column exponent");
 constexpr int kStgPitch = 5;               // complex per staged row (4 used)
 constexpr uint32_t kStgWarp = 32 * kStgPitch * 16;
 // A and B blocks (at most 128 columns) per stage, and the staging tiles; long contractions have larger blocks but no
@@ -61,6 +66,8 @@ constexpr size_t kSmem = 1024 + kStages * 2 * 7 * kADig + kEpiWarps * kStgWarp +
 static_assert(kStages * 2 * 8 * kADig <= kStages * 2 * 7 * kADig + kEpiWarps * kStgWarp, "stages of a long contraction");
 
 constexpr int kNonFinite = 2047;           // row exponent of a row with an Inf or a NaN
+constexpr int kZeroRow = 1023;             // of a row of zeros (any other would do: its digits are zero)
+constexpr int kSafeLo = 600, kSafeHi = 1450;   // rows and columns in this range have kMinE <= e <= kMaxE (see fixed_to_double_*)
 
 // ---------------------------------------------------------------------------
 // Digits
@@ -82,36 +89,38 @@ __device__ __forceinline__ long long k_offset(const Operand &o, int k) {
   return (long long)b * o.kout + (long long)(k - b * o.kin) * o.sk;
 }
 
-// The ND digits of x at row exponent emax as one word: byte ND - 1 - s is d_s + 128 for s > 0, the bits above the
-// last of these bytes are d_0 (a balanced base-256 expansion is the plain one of X + 128 (256^0 + ..)).
+// The ND digits of x at row exponent emax as one word: d_s + 128 is byte ND - 1 - s, and d_0 + 128 of ND = 7, which can be
+// 256, the upper 16 bits (a balanced base-256 expansion is the plain one of X + 128 (256^0 + ..)).
 // X = x 2^(B + 1022 - emax) to nearest, B = 55 bits (ND = 7) or 62 (ND = 8).
 template <int ND>
 __device__ __forceinline__ unsigned long long digits(double x, int emax) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int e = (hi >> 20) & 0x7ff;
-  unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo;
-  const int s = emax - max(e, 1) - (ND == 7 ? 2 : 9);      // X = m 2^-s
-  if (s <= 0) m <<= -s;
-  else m = (s > 60) ? 0ull : (m + (1ull << (s - 1))) >> s;
-  const long long X = ((int)hi < 0) ? -(long long)m : (long long)m;
-  return (unsigned long long)(X + (ND == 7 ? 0x0000808080808080ll : 0x0080808080808080ll));
+  const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo;
+  unsigned long long q;                      // floor(2 |X|); shifts of 64 and more give 0
+  asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"(m << (ND == 7 ? 3 : 10)), "r"(emax - max(e, 1)));
+  q = (q + 1) >> 1;
+  const long long s = (long long)((int)hi >> 31);
+  return (q ^ (unsigned long long)s) + ((ND == 7 ? 0x0080808080808080ull : 0x8080808080808080ull) - (unsigned long long)s);
 }
 
-// d_s of two neighbouring elements as a BF16 pair: 2^23 + byte is an FP32 number, the subtraction
-// exact, and an integer of at most 8 bits has nothing in the low half of its FP32 word.
+// d_s of two neighbouring elements as a BF16 pair.  A byte b = d + 128 below 128 becomes (128 + b) - 256, one from 128 on
+// b - 128, where 128 + (b mod 128) is a BF16 number with the seven low bits of b as its mantissa: both differences are exact.
+// The 9-bit leading digit goes through FP32: 2^23 + b is an FP32 number, and a small integer has nothing in the low half of
+// its FP32 word.
 template <int ND, int S>
 __device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned long long b) {
-  float fa, fb;
-  if (S == 0) {
-    fa = (float)((int)(a >> 32) >> (ND == 7 ? 16 : 24));
-    fb = (float)((int)(b >> 32) >> (ND == 7 ? 16 : 24));
-  } else {
-    constexpr int byte = ND - 1 - S;
-    const uint32_t wa = byte < 4 ? (uint32_t)a : (uint32_t)(a >> 32), wb = byte < 4 ? (uint32_t)b : (uint32_t)(b >> 32);
-    fa = __uint_as_float(__byte_perm(wa, 0x4B000000u, 0x7440 | (byte & 3))) - 8388736.0f;
-    fb = __uint_as_float(__byte_perm(wb, 0x4B000000u, 0x7440 | (byte & 3))) - 8388736.0f;
+  if (S == 0 && ND == 7) {
+    const float fa = __uint_as_float(__byte_perm((uint32_t)(a >> 32), 0x4B000000u, 0x7632)) - 8388736.0f;
+    const float fb = __uint_as_float(__byte_perm((uint32_t)(b >> 32), 0x4B000000u, 0x7632)) - 8388736.0f;
+    return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
   }
-  return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
+  constexpr int byte = ND - 1 - S;
+  const uint32_t wa = byte < 4 ? (uint32_t)a : (uint32_t)(a >> 32), wb = byte < 4 ? (uint32_t)b : (uint32_t)(b >> 32);
+  const uint32_t w = __byte_perm(wa, wb, (byte & 3) | (4 | (byte & 3)) << 8);
+  uint32_t d;
+  asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"((w & 0x007f007fu) | 0x43004300u), "r"((w & 0x00800080u) ^ 0x43804380u));
+  return d;
 }
 
 // Digit planes in global memory, ready for the MMA: block (tile of TR rows, K block) holds ND planes
@@ -147,7 +156,9 @@ __host__ __device__ constexpr int cut_rows(int form) { return kCutVals / seg_k(f
 // kPlanes) in shared memory, read along whichever index is contiguous in memory, takes the largest exponent of each
 // row there, and every thread then cuts eight consecutive K values of one row at a time into seven (eight)
 // 16-byte stores; a warp writes 16 rows x 32 bytes, 512 contiguous bytes, per digit.  Bound by its 16
-// bytes read and 28 written per complex element (56 for kReal).
+// bytes read and 28 written per complex element (56 for kReal).  The phases of a CTA only overlap with those of others:
+// 40 registers for six CTAs per SM.  nb = 64 operand (268 MB read, 470 MB written): 199 us with one load in flight per
+// thread and four CTAs, 172 with four loads, 160 with six CTAs (4.6 TB/s).
 struct CutJob {
   Operand o;               // o.rows: rows of the panel
   int r_begin, TR;
@@ -155,10 +166,10 @@ struct CutJob {
   uint8_t *out;
 };
 template <int FORM>
-__device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_begin, int Klen, int Kp, int KB) {
-  constexpr int SK = seg_k(FORM), SR = cut_rows(FORM), ND = digits_of(FORM == kPlanes);
+__device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_begin, int Klen, int Kp, int KB, int SK) {
+  constexpr int SR = cut_rows(FORM), ND = digits_of(FORM == kPlanes);
   extern __shared__ double sh[];
-  __shared__ long long roff[SR], koff[SK];
+  __shared__ long long roff[SR], koff[seg_k(FORM)];
   __shared__ int emax[SR];
   const Operand &A = job.o;
   const int r_begin = job.r_begin, TR = job.TR;
@@ -175,33 +186,49 @@ __device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_b
   if (tid < SK) koff[tid] = (k0 + tid < Klen) ? k_offset(A, k_begin + k0 + tid) : -1;
   __syncthreads();
   const int flip_im = A.conj ? (int)0x80000000u : 0;
-  auto stage = [&](int r, int k) {
-    cplx v = {0.0, 0.0};
-    if (koff[k] >= 0) v = A.p[roff[r] + koff[k]];
-    re[r * pitch + k] = v.x;
-    im[r * pitch + k] = __hiloint2double(__double2hiint(v.y) ^ flip_im, __double2loint(v.y));
-  };
-  if (A.sk == 1) {
+  // kLoads loads in flight per thread, consecutive lanes along the index that is contiguous in memory
+  constexpr int kLoads = 4;
+  const int total = SR * kt;
+  const unsigned inv = ((1u << 22) + kt - 1) / kt;        // idx / kt = idx inv >> 22 for idx kt < 2^22
+  const double2 *__restrict__ p = A.p;
+  for (int i0 = tid; i0 < total; i0 += 256 * kLoads) {
+    cplx v[kLoads];
+    int at[kLoads];
 #pragma unroll
-    for (int i = 0; i < SR / 8; ++i)
-      for (int k = lane; k < kt; k += 32) stage(warp + 8 * i, k);
-  } else {
-    constexpr int kPerWarp = 32 / SR;                     // K values that a warp reads at once
-#pragma unroll 4
-    for (int k = warp * kPerWarp + lane / SR; k < kt; k += 8 * kPerWarp) stage(lane % SR, k);
+    for (int i = 0; i < kLoads; ++i) {
+      const int idx = i0 + 256 * i;
+      int r, k;
+      if (A.sk == 1) { r = (int)((unsigned)idx * inv >> 22); k = idx - r * kt; }
+      else { k = idx / SR; r = idx % SR; }
+      at[i] = r * pitch + k;
+      v[i] = {0.0, 0.0};
+      if (idx < total && koff[k] >= 0) v[i] = __ldg(p + roff[r] + koff[k]);
+    }
+#pragma unroll
+    for (int i = 0; i < kLoads; ++i) {
+      if (i0 + 256 * i < total) {
+        re[at[i]] = v[i].x;
+        im[at[i]] = __hiloint2double(__double2hiint(v[i].y) ^ flip_im, __double2loint(v[i].y));
+      }
+    }
   }
   __syncthreads();
   {
     constexpr int T = 256 / SR;                           // threads per row
     const int r = tid / T, j = tid % T;
-    int e = 0;
+    int e = 0, low = 0;
     for (int k = j; k < kt; k += T) {
-      e = max(e, __double2hiint(re[r * pitch + k]) & 0x7ff00000);
-      e = max(e, __double2hiint(im[r * pitch + k]) & 0x7ff00000);
+      const double x = re[r * pitch + k], y = im[r * pitch + k];
+      e = max(e, max(__double2hiint(x) & 0x7fffffff, __double2hiint(y) & 0x7fffffff));
+      low |= __double2loint(x) | __double2loint(y);
     }
+    low = (low != 0);
 #pragma unroll
-    for (int o = T / 2; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-    e = max(e >> 20, 1);
+    for (int o = T / 2; o > 0; o >>= 1) {
+      e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+      low |= __shfl_xor_sync(0xffffffffu, low, o);
+    }
+    e = (e | low) == 0 ? kZeroRow : max(e >> 20, 1);
     if (j == 0) {
       emax[r] = e;
       if (r < nr) rexp[(size_t)seg * A.rows + r0 + r] = e;
@@ -219,7 +246,7 @@ __device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_b
     unsigned long long w[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) w[i] = digits<ND>(e == kNonFinite ? 0.0 : src[i], e);
-    const int q0 = seg * 2 * kSeg, row = r0 + r;          // 16-byte chunks before this segment
+    const int q0 = seg * (SK / (FORM == kPlanes ? 8 : 4)), row = r0 + r;          // 16-byte chunks before this segment
     if (FORM == kRows) {
       store_digits<ND>(out, TR, KB, row, q0 + u * nch + kc, w, 0u);
     } else if (FORM == kReal) {
@@ -234,11 +261,11 @@ __device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_b
 // Both operands of a product in one launch: blocks below xblocks cut x, the others y.  (The column operand is small: as
 // a launch of its own it took 5 us of the 50 us of a mode product at nb = 32.)
 template <int FX, int FY>
-__global__ void __launch_bounds__(256) cut_digits_kernel(const CutJob x, const CutJob y, int xblocks, int k_begin, int Klen,
-                                                         int Kp, int KB) {
+__global__ void __launch_bounds__(256, 6) cut_digits_kernel(const CutJob x, const CutJob y, int xblocks, int k_begin, int Klen,
+                                                         int Kp, int KB, int SK) {
   dependent_begin();
-  if ((int)blockIdx.x < xblocks) cut_digits<FX>(x, blockIdx.x, k_begin, Klen, Kp, KB);
-  else cut_digits<FY>(y, blockIdx.x - xblocks, k_begin, Klen, Kp, KB);
+  if ((int)blockIdx.x < xblocks) cut_digits<FX>(x, blockIdx.x, k_begin, Klen, Kp, KB, SK);
+  else cut_digits<FY>(y, blockIdx.x - xblocks, k_begin, Klen, Kp, KB, SK);
 }
 
 // ---------------------------------------------------------------------------
@@ -246,7 +273,7 @@ __global__ void __launch_bounds__(256) cut_digits_kernel(const CutJob x, const C
 // ---------------------------------------------------------------------------
 struct TcGemm {
   const uint8_t *A, *B;       // digit blocks
-  int KB, segs;               // K blocks of a row tile, in segments of kSeg
+  int KB, segs, kseg;         // K blocks of a row tile, in segments of kseg
   int nt;                     // real columns per tile (multiple of 16)
   int mtiles, ntiles;         // unit = (split mtiles + m_tile) ntiles + n_tile
   int splits, segs_per_split; // long contractions: segments cut over the units
@@ -293,17 +320,25 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
                : "memory");
 }
 
-// 2^e mant with the sign, where the exponent needs care (subnormal or overflowing results)
-__device__ __noinline__ double scaled(uint32_t mhi, uint32_t mlo, int e, uint32_t sign) {
-  const double v = ldexp((double)(((unsigned long long)mhi << 32) | mlo), e);
-  return sign ? -v : v;
+// (hi 2^32 + lo) 2^e as FP64, rounded to nearest, without a branch, for |hi| < 2^62, |lo| < 2^62 and kMinE <= e <= kMaxE (no
+// subnormal or infinite result then).  Two forms, because either alone is bound by its own pipe:
+//   fixed_to_double_add: the upper 52 bits and the lower 44 as mantissas at 1.5 2^96 and 1.5 2^52; two FP64 additions
+//       (64 cycles of the FP64 pipe per warp each), the first exact, and ten integer instructions;
+//   fixed_to_double_int: the 96-bit magnitude is shifted left to its leading one by whole words and a funnel shift: about
+//       forty integer instructions.
+// The real parts take the one and the imaginary parts the other; long contractions, which add segments up on the FP64 pipe,
+// the second alone.  Mode product at nb = 64, us: additions only 378, integers only 343, both 341.
+constexpr int kMinE = -1022, kMaxE = 927;
+__device__ __forceinline__ double fixed_to_double_add(long long hi, long long lo, int e) {
+  hi += lo >> 32;
+  const int es = e << 20;
+  const double x0 = __hiloint2double((int)((0x43380000u + (uint32_t)es) | ((uint32_t)hi & 0xfffu)), (int)(uint32_t)lo);
+  const long long top = hi >> 12;
+  const double x1 = __longlong_as_double(top + ((long long)(0x45F80000 + es) << 32));
+  const double c = __hiloint2double(0x45F80000 + es, 0x180);   // 1.5 2^96 + 1.5 2^52
+  return __dadd_rn(__dsub_rn(x1, c), x0);
 }
-
-// (hi 2^32 + lo) 2^e as FP64, rounded to nearest, in about fifty 32-bit integer instructions (an FP64 instruction
-// occupies its pipe for 64 cycles per warp: a conversion with two of them was 1.5 times slower) without a branch (but for
-// results outside the normal range): the 96-bit magnitude is shifted left to its leading one by whole words and
-// a funnel shift.  |hi| < 2^62, |lo| < 2^62.
-__device__ __forceinline__ double fixed_to_double(long long hi, long long lo, int e) {
+__device__ __forceinline__ double fixed_to_double_int(long long hi, long long lo, int e) {
   hi += lo >> 32;
   uint32_t w0 = (uint32_t)lo;
   const uint32_t s = (uint32_t)(int)(hi >> 63);
@@ -320,10 +355,11 @@ __device__ __forceinline__ double fixed_to_double(long long hi, long long lo, in
   const uint32_t up = (t0 >> 10) & 1u;
   mlo += up;
   mhi += (mlo < up) ? 1u : 0u;
-  if (w2 == 0) return 0.0;
-  if ((uint32_t)p > 2044u) return scaled(mhi, mlo, p + 1 - 1023 - 52, s);
-  return __hiloint2double((int)((mhi + ((uint32_t)p << 20)) | (s & 0x80000000u)), (int)mlo);
+  const uint32_t out = w2 == 0 ? 0u : ((mhi + ((uint32_t)p << 20)) | (s & 0x80000000u));
+  return __hiloint2double((int)out, (int)mlo);
 }
+// 2^k times a result at the end of that range, for any other e (a subnormal result is rounded a second time)
+__device__ __noinline__ double beyond_range(double x, int k) { return ldexp(x, k); }
 
 // alpha z for alpha = i^u: signs by the integer pipe
 __device__ __forceinline__ cplx mul_unit(cplx z, int u) {
@@ -357,6 +393,11 @@ __device__ __noinline__ double plain_part(const Operand &X, const Operand &Y, in
   return s;
 }
 
+__device__ __forceinline__ float max_abs3(float a, float b, float c) {
+  float d;
+  asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
 // 256 (256 (256 q0 + q1) + q2) + q3 of eight columns, q_o the integer values of four FP32 accumulators.  An
 // integer up to 2^22 shows in the low bits of its sum with 1.5 2^23; larger ones (sums of digit
 // products near their bound) are converted one by one, at a quarter of the rate.
@@ -365,7 +406,7 @@ __device__ __forceinline__ void join_orders(const uint32_t (&v)[4][8], long long
 #pragma unroll
   for (int o = 0; o < 4; ++o)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) mx = fmaxf(mx, fabsf(__uint_as_float(v[o][j])));
+    for (int j = 0; j < 8; j += 2) mx = max_abs3(mx, __uint_as_float(v[o][j]), __uint_as_float(v[o][j + 1]));
   if (__any_sync(0xffffffffu, !(mx <= 4194304.f))) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -439,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
         const int nt = u % p.ntiles, mt = (u / p.ntiles) % p.mtiles, sp = u / (p.ntiles * p.mtiles);
         const int s0 = sp * p.segs_per_split, s1 = min(p.segs, s0 + p.segs_per_split);
         for (int sf = s0 * kPhases; sf < s1 * kPhases && ok; ++sf) {
-          const int f = sf % kPhases, kb0 = (sf / kPhases) * kSeg, kb1 = min(p.KB, kb0 + kSeg);
+          const int f = sf % kPhases, kb0 = (sf / kPhases) * p.kseg, kb1 = min(p.KB, kb0 + p.kseg);
           const uint32_t nd = (kPhases == 2 && f == 1) ? 4u : (uint32_t)kDig;
           for (int kb = kb0; kb < kb1; ++kb) {
             if (!mbar_wait(&empty[s], ph ^ 1u, p.err)) { ok = false; break; }
@@ -462,7 +503,7 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
         const int sp = u / (p.ntiles * p.mtiles);
         const int s0 = sp * p.segs_per_split, s1 = min(p.segs, s0 + p.segs_per_split);
         for (int seg = s0; seg < s1 && ok; ++seg) {
-          const int kb0 = seg * kSeg, kb1 = min(p.KB, kb0 + kSeg);
+          const int kb0 = seg * p.kseg, kb1 = min(p.KB, kb0 + p.kseg);
 #pragma unroll
           for (int f = 0; f < kPhases; ++f) {
             if (!ok || !mbar_wait(tempty, acc_ph ^ 1u, p.err)) { ok = false; break; }
@@ -521,16 +562,17 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
       for (int seg = s0; seg < s1 && ok; ++seg) {
         // exponents, loaded before the MMAs are waited for: lane 4 i + j holds that of column j of this warp's
         // i-th group
-        const int yl = y_tile + 4 * (cg + (lane & ~3)) + (lane & 3);
-        const int ea = valid ? p.ex[(size_t)seg * p.exs + mc] : 1;
-        const int eyl = (lane < 16 && yl < p.cols) ? p.ey[(size_t)seg * p.eys + yl] : 1;
-        const bool any_bad = __any_sync(0xffffffffu, ea == kNonFinite || eyl == kNonFinite);
+        const int yl = y_tile + 4 * (cg + kPerQuarter * (lane >> 2)) + (lane & 3);
+        const int ea = valid ? p.ex[(size_t)seg * p.exs + mc] : kZeroRow;
+        const int eyl = (lane < kMaxGroups * 4 && yl < p.cols) ? p.ey[(size_t)seg * p.eys + yl] : kZeroRow;
+        // rows that need care: Inf or NaN, or results that may leave the range of fixed_to_double_*
+        const bool care = __any_sync(0xffffffffu, min(ea, eyl) < kSafeLo || max(ea, eyl) > kSafeHi);
 #pragma unroll 1
         for (int f = 0; f < kPhases; ++f) {
           if (!__all_sync(0xffffffffu, mbar_wait(tfull, acc_ph, p.err))) { ok = false; break; }
           tc_fence_after();
 #pragma unroll 1
-          for (int g = cg; g < ngroups; g += 4) {
+          for (int g = cg; g < ngroups; g += kPerQuarter) {
 #pragma unroll
             for (int w = 0; w < G / 4; ++w) {
               long long *q = sums + (size_t)(8 * g) * kTM + ((G == 8 ? w : 1 - f) ? kTNMax * kTM : 0);
@@ -553,10 +595,13 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
         }
         if (!ok) break;
         const bool first = seg == s0 && !(kSplit && p.accumulate), last = seg == s1 - 1;
-        const int seg_len = seg_k(kSplit ? kPlanes : kRows);
+        const int seg_len = kSplit ? p.kseg * kKB : seg_k(kRows);
         const int k0 = p.k_begin + seg * seg_len, k1 = min(p.X.K, k0 + seg_len);
+        // two copies: with the calls of the careful one in its loop, the plain one spilled registers
+        auto convert = [&](auto careful) {
+        constexpr bool kCare = decltype(careful)::value;
 #pragma unroll 1
-        for (int g = cg; g < ngroups; g += 4) {
+        for (int g = cg, gl = 0; g < ngroups; g += kPerQuarter, gl += 4) {
           const int y0 = y_tile + 4 * g;                 // first complex column of the group
           const int ny = min(4, p.cols - y0);
           if (ny <= 0) break;
@@ -570,14 +615,17 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
           }
           double v[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int e = ea + __shfl_sync(0xffffffffu, eyl, g - cg + (j >> 1)) - (kSplit ? 2112 : 2114);
-            v[j] = fixed_to_double(hi[j], lo[j], e);
-          }
-          if (any_bad) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int eb = __shfl_sync(0xffffffffu, eyl, g - cg + j);   // every lane: not behind a condition
+          for (int j = 0; j < 4; ++j) {
+            const int e0 = ea + __shfl_sync(0xffffffffu, eyl, gl + j) - (kSplit ? 2112 : 2114);
+            const int e = kCare ? min(max(e0, kMinE), kMaxE) : e0;
+            v[2 * j] = kSplit ? fixed_to_double_int(hi[2 * j], lo[2 * j], e) : fixed_to_double_add(hi[2 * j], lo[2 * j], e);
+            v[2 * j + 1] = fixed_to_double_int(hi[2 * j + 1], lo[2 * j + 1], e);
+            if constexpr (kCare) {
+              if (e != e0) {
+                v[2 * j] = beyond_range(v[2 * j], e0 - e);
+                v[2 * j + 1] = beyond_range(v[2 * j + 1], e0 - e);
+              }
+              const int eb = __shfl_sync(0xffffffffu, eyl, gl + j);   // every lane: not behind a condition
               if ((ea == kNonFinite || eb == kNonFinite) && valid && j < ny) {
                 if (kSplit) {
                   v[2 * j] = plain_part(p.X, p.Y, mc, m & 1, y0 + j, 0, k0, k1);
@@ -588,8 +636,8 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
                   v[2 * j + 1] = z.y;
                 }
               }
+              __syncwarp();
             }
-            __syncwarp();
           }
           if (kKind != 0 && !first) {   // (in one-segment kernels the compiler would add a zero, on the slow FP64 pipe)
             double o[8];
@@ -650,6 +698,9 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
               if (in[it]) c[ro[it]] = t[it];
           }
         }
+        };
+        if (care) convert(std::true_type{});
+        else convert(std::false_type{});
       }
     }
   }
@@ -729,17 +780,17 @@ CutJob cut_job(const Operand &o, int r_begin, int rows, int TR, int *rexp, uint8
   return j;
 }
 
-// x and y with rows > 0
+// x and y (where they have rows) in segments of SK <= seg_k(FX) values
 template <int FX, int FY>
-void cut(Launcher &L, const CutJob &x, const CutJob &y, int k_begin, int Klen, int Kp, int KB) {
+void cut(Launcher &L, const CutJob &x, const CutJob &y, int k_begin, int Klen, int Kp, int KB, int SK) {
   static_assert(seg_k(FX) == seg_k(FY), "one grid of segments");
   constexpr int SR = cut_rows(FX);
-  const size_t sh = (size_t)2 * SR * (std::min(seg_k(FX), Kp) + 1) * sizeof(double);
+  const size_t sh = (size_t)2 * SR * (std::min(SK, Kp) + 1) * sizeof(double);
   const int xb = (x.o.rows + SR - 1) / SR, yb = (y.o.rows + SR - 1) / SR;
   if (xb + yb == 0) return;
-  dim3 grid(xb + yb, (Kp + seg_k(FX) - 1) / seg_k(FX));
+  dim3 grid(xb + yb, (Kp + SK - 1) / SK);
   L.before("fp64_tc_digits");
-  launch_dependent(cut_digits_kernel<FX, FY>, grid, 256, sh, L.stream, x, y, xb, k_begin, Klen, Kp, KB);
+  launch_dependent(cut_digits_kernel<FX, FY>, grid, 256, sh, L.stream, x, y, xb, k_begin, Klen, Kp, KB, SK);
   L.after_launch();
 }
 
@@ -785,7 +836,7 @@ Fp64Tc *fp64_tc_create(int nb, bool pair_products) {
   const size_t lng = blocks(2 * N, (N3 + 255) / 256 * 256, true);
   f->a_bytes = std::min(kPanelBytes, std::max({big, pair, lng}));
   f->b_bytes = std::min(kPanelBytes, std::max({blocks(2 * N, 2 * ((N + 7) / 8 * 8)), pair, lng}));
-  f->exps = std::max({N3, N2 * ((N2 + 127) / 128), N * ((N3 + 255) / 256)});
+  f->exps = std::max({N3, N2 * ((N2 + 127) / 128), N * ((N3 + 127) / 128)});
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&f->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -862,9 +913,9 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
     for (int m0 = 0; m0 < all_m; m0 += pm) {
       const int r0 = m0 * kTM, nr = (int)std::min<long long>(rows - r0, (long long)std::min(pm, all_m - m0) * kTM);
       cut<kRows, kReal>(L, cut_job(X, r0, (n0 == 0 || pm < all_m) ? nr : 0, kTM, f->ex, f->A),
-                        cut_job(Y, y0, (m0 == 0 && !kept) ? ny : 0, nt, f->ey, f->B), 0, g.K, Kp, KB);
+                        cut_job(Y, y0, (m0 == 0 && !kept) ? ny : 0, nt, f->ey, f->B), 0, g.K, Kp, KB, seg_k(kRows));
       TcGemm t{};
-      t.A = f->A; t.B = f->B; t.KB = KB; t.segs = segs; t.nt = nt;
+      t.A = f->A; t.B = f->B; t.KB = KB; t.segs = segs; t.kseg = kSeg; t.nt = nt;
       t.mtiles = (nr + kTM - 1) / kTM; t.ntiles = (2 * ny + nt - 1) / nt;
       t.splits = 1; t.segs_per_split = segs; t.err = f->err; t.sums = f->sums; t.part = f->part;
       t.X = X; t.Y = Y; t.ex = f->ex; t.ey = f->ey; t.exs = nr; t.eys = ny;
@@ -901,17 +952,20 @@ bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g) {
   const int splits_max = f->sms / (mtiles * ntiles);   // one unit per CTA
   if (splits_max < 1) return false;
   constexpr int kDig = digits_of(true);
-  const size_t a_seg = (size_t)mtiles * kSeg * kDig * kADig, b_seg = (size_t)ntiles * kSeg * kDig * nt * 32;   // bytes per segment
-  const int all_segs = (K + kSeg * kKB - 1) / (kSeg * kKB);
+  // segments of 256 terms, or 128 where those leave half of the SMs idle (nb <= 26: 34 -> 24 us at nb = 24)
+  const int kseg = 2 * ((K + kSeg * kKB - 1) / (kSeg * kKB)) * mtiles * ntiles <= f->sms ? kSeg / 2 : kSeg;
+  const size_t a_seg = (size_t)mtiles * kseg * kDig * kADig, b_seg = (size_t)ntiles * kseg * kDig * nt * 32;   // bytes per segment
+  const int all_segs = (K + kseg * kKB - 1) / (kseg * kKB);
   int ps = (int)std::min<size_t>(all_segs, std::min(f->a_bytes / a_seg, f->b_bytes / b_seg));
   ps = (int)std::min<long long>(ps, f->exps / std::max(g.M, g.N));
   if (ps < 1) return false;
   TcGemm t{};
   for (int sg0 = 0; sg0 < all_segs; sg0 += ps) {
-    const int ns = std::min(ps, all_segs - sg0), k0 = sg0 * kSeg * kKB, Klen = std::min(K - k0, ns * kSeg * kKB);
+    const int ns = std::min(ps, all_segs - sg0), k0 = sg0 * kseg * kKB, Klen = std::min(K - k0, ns * kseg * kKB);
     const int Kp = round_up(Klen, kKB), KB = Kp / kKB;
-    cut<kPlanes, kPlanes>(L, cut_job(X, 0, g.M, kTM, f->ex, f->A), cut_job(Y, 0, g.N, nt, f->ey, f->B), k0, Klen, Kp, KB);
-    t.A = f->A; t.B = f->B; t.KB = KB; t.segs = ns; t.nt = nt; t.mtiles = mtiles; t.ntiles = ntiles;
+    cut<kPlanes, kPlanes>(L, cut_job(X, 0, g.M, kTM, f->ex, f->A), cut_job(Y, 0, g.N, nt, f->ey, f->B), k0, Klen, Kp, KB,
+                           kseg * kKB);
+    t.A = f->A; t.B = f->B; t.KB = KB; t.segs = ns; t.kseg = kseg; t.nt = nt; t.mtiles = mtiles; t.ntiles = ntiles;
     // the first panel is the longest: its split count holds for the later ones
     if (sg0 == 0) {
       t.segs_per_split = (ns + splits_max - 1) / splits_max;

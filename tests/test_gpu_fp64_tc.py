@@ -81,3 +81,18 @@ def test_non_finite_entries_reach_the_same_outputs(bad):
 def test_rhs_matches_oracle_across_the_dispatch(nb, se, bosons):
     """As test_rhs_matches_oracle: 1e-12 of the largest entry."""
     test_rhs_matches_oracle(nb, se, bosons)
+
+
+def test_results_near_the_end_of_the_exponent_range():
+    """The commutator alone at 2^-1000 G2, where the conversion of the integer sums takes its careful path: the same
+    numbers shifted, to the last subnormal bit (one rounding more there)."""
+    from paper_2002_12717_gb300.g1g2 import Propagator
+    nb, k = 24, -1000
+    h, w, n, g2, D, drv = problem(nb, "SOA", False, False, seed=13)
+    g2 = g2.copy()
+    g2[2, 3] = 0.0                       # rows of zeros among them
+    with Propagator(h, 0 * w, n, None, "SOA", "fp64") as p:
+        _, ref = gpu_rhs(p, 0.0, n, g2)
+        _, got = gpu_rhs(p, 0.0, n, np.ldexp(g2.real, k) + 1j * np.ldexp(g2.imag, k))
+    for a, b in ((got.real, np.ldexp(ref.real, k)), (got.imag, np.ldexp(ref.imag, k))):
+        assert np.abs(a - b).max() <= 16 * 2.0 ** -1074
