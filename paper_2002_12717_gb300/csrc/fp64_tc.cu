@@ -24,8 +24,8 @@
 // at nb = 16, 20, 24 are 2.2e-16, 2.4e-16, 3.7e-16 off (2-norm, extended precision) instead of 3.3e-16, 4.7e-16,
 // 6.4e-16.
 //
-// All conversions run on the integer pipe: FP64 instructions in the prologue or epilogue would
-// cost as much as the MMAs (two per SM and clock).  A row or column that holds an Inf or a NaN has
+// The digits are cut on the integer pipe, and the sums converted on both (fixed_to_double_*): FP64 instructions
+// alone would cost as much as the MMAs (two per SM and clock).  A row or column that holds an Inf or a NaN has
 // no digits; its outputs are recomputed with FP64 multiply-adds in the epilogue, which gives
 // the values the CUDA-core kernel gives.
 #include "g1g2_internal.h"
@@ -427,8 +427,8 @@ __device__ __forceinline__ void join_orders(const uint32_t (&v)[4][8], long long
 }
 
 // Persistent over units of one 128-row tile x nt real columns x a range of segments.  Roles: warp 0 loads
-// digit blocks (bulk copies, three stages of one 16-element K step), warp 1 issues the MMAs, warps 2-17 drain
-// the accumulators at the end of a segment (a warp reads its lane quarter, every fourth group of eight columns) into
+// digit blocks (bulk copies, three stages of one 16-element K step), warp 1 issues the MMAs, warps 2-13 drain
+// the accumulators at the end of a segment (a warp reads its lane quarter, every third group of eight columns) into
 // integer sums in global memory, which stay in L2, and read them back, convert and store (or add up) while the
 // next MMAs run.  (With the sums in registers the loops over columns had to be unrolled into 70 to 140 KB of
 // code, and instruction fetches made the epilogue three times the MMA time.)
@@ -797,9 +797,10 @@ void cut(Launcher &L, const CutJob &x, const CutJob &y, int k_begin, int Klen, i
 }  // namespace
 
 constexpr int kMinK = 8, kMinCols = 8;
-// Complex multiply-adds from which a product is faster here than on zgemm_kernel: a mode product at nb = 16 takes 12 us
-// there and 20 us here (digits and product), at nb = 20 30 and 24 us; a long contraction 17 and 40 us at nb = 16, 60 and 48 us
-// at nb = 24; an nb^2 x nb^2 x nb^2 product at nb = 12 (3e6) 40 and 30 us.
+// Complex multiply-adds from which a product is faster here than on zgemm_kernel, whose time grows with them while digits,
+// product and reduction here cost their launches and one round of MMAs.  Per launch with an event on either side: mode product 13 us
+// there at nb = 15 (34 at nb = 20 by its growth), 25 us here at nb = 16 and 30 at nb = 20; long contraction 25 us there
+// at nb = 15 (45 at nb = 20), 48 us here at nb = 16 and 43 at nb = 24; nb^2 x nb^2 x nb^2 product 43 and 39 us at nb = 12 (3e6).
 constexpr double kMinWork = 2.2e6, kMinWorkLong = 4e6;
 
 int fp64_tc_min_nb(bool pair_products) { return pair_products ? 12 : 17; }
