@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(256) slice_b_kernel(int nb, int nout, int kpad
   const int complex_a = o.complex_a, shift = o.shift, ld = o.ld, transpose = o.transpose, il = o.il;
   __nv_bfloat16 *out = o.out;
   const long long slice_stride = o.slice_stride;
-  __shared__ double red[8];
+  __shared__ int red[8];
   __shared__ double smu;
   const int kt = complex_a ? 2 * kpad : kpad;
   const int total = nout * kt;
@@ -202,20 +202,23 @@ __global__ void __launch_bounds__(256) slice_b_kernel(int nb, int nout, int kpad
   }
   __syncthreads();
   const double mu = smu;
-  double mx = 0.0;
+  // 2^E above the largest magnitude: only its exponent counts, so the maximum is one of high words, on the integer pipe (with
+  // FP64 comparisons every CTA spent 9 k of its cycles on them at nb = 96)
+  int mx = 0;
   for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
     cplx v = S[e];
-    if (e / nb == e % nb) v.x -= mu;
-    mx = fmax(mx, fmax(fabs(v.x), fabs(v.y)));
+    if (shift && e % (nb + 1) == 0) v.x -= mu;
+    const int hx = __double2hiint(v.x) & 0x7fffffff, hy = __double2hiint(v.y) & 0x7fffffff;
+    mx = max(mx, max(hx > 0x7ff00000 ? 0 : hx, hy > 0x7ff00000 ? 0 : hy));   // a NaN has no part in it
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
   __syncthreads();
-  mx = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mx = fmax(mx, red[w]);
+  mx = 0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mx = max(mx, red[w]);
   int E = 0;
-  if (mx > 0.0) frexp(mx, &E);  // mx < 2^E
+  if (mx > 0) frexp(__hiloint2double(mx, 0), &E);  // largest magnitude < 2^E
   double c[4];
   slice_cuts_f64(E, 7, c);
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
