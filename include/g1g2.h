@@ -179,6 +179,8 @@ int g1g2_set_drive(g1g2_ctx *c, const double *D, int kind, const double *params,
  *   n_dev, G2_dev  input state; G2_dev must be Hermitian as an nb^2 x nb^2
  *                  matrix (Eq. Gsymm_b), which the tensor-core form relies on
  *   dn_dev, dG2_dev  outputs dn/dt and dG2/dt (dG2 is zero for HF)
+ * dG2_dev may overlap G2_dev (all of G2 is read before dG2 is written); dn_dev must
+ * not overlap an input.
  * Runs on the context's stream; returns after the launches are queued. */
 int g1g2_rhs(g1g2_ctx *c, double t, const double *n_dev, const double *G2_dev, double *dn_dev,
              double *dG2_dev);

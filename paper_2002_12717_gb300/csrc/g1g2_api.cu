@@ -10,6 +10,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <cmath>
+#include <cstdint>
 #include <complex>
 #include <cstdio>
 #include <cstring>
@@ -318,10 +319,16 @@ void mean_field(g1g2_ctx *c, Launcher &L, const cplx *h, const cplx *D, double f
     hf_build(L, c->nb, c->Wm, c->w_real, h, D, f, n, c->hhf);
 }
 
+// whether [a, a + na) and [b, b + nb) share memory
+bool overlap(const cplx *a, long long na, const cplx *b, long long nb) {
+  const std::uintptr_t x = reinterpret_cast<std::uintptr_t>(a), y = reinterpret_cast<std::uintptr_t>(b);
+  return x < y + nb * sizeof(cplx) && y < x + na * sizeof(cplx);
+}
+
 void rhs_fp64(g1g2_ctx *c, Launcher &L, double t, const cplx *n_in, const cplx *G_in, Rk4Stage st,
               const StageOut &o, bool w_only = false) {
   const int nb = c->nb;
-  const long long N = nb, N2 = N * N, N3 = N2 * N;
+  const long long N = nb, N2 = N * N, N3 = N2 * N, N4 = N2 * N2;
   const double f = drive_f(c, t);
   // with w_only the one-body h(t) is left out (the part of the right-hand side that is linear in w,
   // used for the gradient by the scale of w)
@@ -337,7 +344,12 @@ void rhs_fp64(g1g2_ctx *c, Launcher &L, double t, const cplx *n_in, const cplx *
       p.Go = st.stage <= 0 ? c->Gss : st.stage == 2 ? c->Cb2 : c->Gss_s;
       p.Sy = c->Gss; p.Sys = st.stage == 1 ? c->Cb2 : c->Gss_s; p.Sacc = c->Gss_acc;
     }
+    // A caller may let dG2 overlap G2 (or n): the general basis writes dG2 after its last read of either.  The stage
+    // kernel stores while others still read neighbours, so such a call goes through the commutator buffer, free here
+    const bool through_c = st.stage < 0 && (overlap(o.Gk, N4, G_in, N4) || overlap(o.Gk, N4, n_in, N2));
+    if (through_c) p.Gk = c->Cb;
     hubbard_stage(L, p);
+    if (through_c) cudaMemcpyAsync(o.Gk, c->Cb, N4 * sizeof(cplx), cudaMemcpyDeviceToDevice, c->stream);
     return;
   }
   // a1: Eq. (h_HF)
