@@ -78,7 +78,9 @@ typedef enum {
 /* Arithmetic of the contractions. The RK4 state update, the Hartree-Fock
  * build and the observables are FP64 in every mode. */
 typedef enum {
-  G1G2_FP64 = 0,   /* every contraction in FP64 on the CUDA cores: the reference form */
+  G1G2_FP64 = 0,   /* the reference form.  Every element of a contraction errs by no more than the a-priori bound of
+                      FP64 multiply-adds, n 2^-53 sum |a| |b| over its own n terms (real and imaginary part each), whether
+                      it is formed by them or, in larger products, on the tensor cores from 8-bit digits; typically by less */
   G1G2_TF32X3 = 1, /* split-precision tensor-core contractions: hi/lo TF32 operands, FP32 accumulation */
   G1G2_BF16X4 = 2  /* tensor-core contractions on four BF16 slices per operand with one power-of-two
                       scale per tensor; the leading slice product accumulates exactly in FP32, the

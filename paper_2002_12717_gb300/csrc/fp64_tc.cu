@@ -2,32 +2,39 @@
 //
 // GB300 issues about two FP64 multiply-adds per SM and clock (1.2 TFLOP/s for the chip), so a
 // contraction of the FP64 form is bound by the FP64 pipe 50 to 100 times above the time its
-// bytes take.  Here each real operand is cut into seven (eight) signed 8-bit digits, the digit
+// bytes take.  Here each real operand is cut into eight signed 8-bit digits, the digit
 // products run as BF16 MMAs on tcgen05 and are summed as integers (the error-free
 // splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 95 (2012)):
 //
-//   x = 2^(e - 1077) sum_s d_s 256^(6 - s),  |d_s| <= 128        (long contractions: 2^(e - 1084) .. 256^(7 - s)),
+//   x = 2^(e - 1084) sum_s d_s 256^(7 - s),  |d_s| <= 128, |d_0| <= 64,
 //
 // with one exponent e per row of A (column of B) and segment of the contraction (at most 256 terms), the one
-// of its largest entry there, so that 56 bits below that entry's leading bit are kept: every entry
-// within a factor 4 of the largest is held exactly.  Digits are small integers, exact in BF16.  The products
+// of its largest entry there: an entry is held to 2^-62 of 2^e.  Digits are small integers, exact in BF16.  The products
 // d_s d'_t of one order o = s + t have one common weight 256^-o and a TMEM accumulator of their own; orders
-// 0..7 are formed (34 MMAs per 16-element K step).  The dropped ones weigh 2^-64 of the largest product: with
-// seven orders (28 MMAs) they weighed 2^-56, and rows whose largest entry is ten times the typical one
-// (w and n of a general basis) lost 3e-15 of the result, more than FP64 multiply-adds do.  An FP32
-// accumulator is exact while its sum of integers stays below 2^24: o + 1 products of at most 2^14 over 256
-// terms, so the orders 0..3 never round, and a rounding of the higher ones weighs below 2^-56.  At the end of
+// 0..7 are formed (36 MMAs per 16-element K step).  The dropped ones weigh at most 2^-57 of 2^e 2^e' per term (typically 2^-60).
+// An FP32 accumulator is exact while its sum of integers stays up to 2^24: at most o + 1 products of 2^14 (2^13 with a
+// leading digit) over 256 terms, so the orders 0..4 never round, and 5..7 do so only where the digits of nearly every term are
+// close to 128 and of one sign, by a few units of 2^-50 2^e 2^e'.  At the end of
 // a segment the accumulators go into 64-bit integers (hi: orders 0..3, lo: orders 4..7), whose sum is
 // rounded once to FP64; the segments of a long contraction are added in FP64.  (One exponent for a whole row
-// of 32768 terms lost a factor ten against FP64 multiply-adds in the gradients of sparse cotangents.)  Against FP64
-// multiply-adds, which round after every term, the result is closer to the exact sum: right-hand sides
-// at nb = 16, 20, 24 are 2.2e-16, 2.4e-16, 3.7e-16 off (2-norm, extended precision) instead of 3.3e-16, 4.7e-16,
-// 6.4e-16.
+// of 32768 terms lost a factor ten against FP64 multiply-adds in the gradients of sparse cotangents.)
+//
+// All this is relative to the largest entries, while FP64 multiply-adds err by parts of sum |a| |b|, which is far
+// smaller where entries of very different size meet: far from the diagonal of decaying matrices, beside one huge matrix
+// element, in the imaginary parts of nearly real data.  So one more MMA per K step sums the magnitudes, as BF16
+// numbers (magnitude()), and an element with 0 < sum |a| |b| < 2^e 2^e' max(sqrt(n), 4) / 64, n the smaller of the two rows'
+// numbers of nonzero terms, is taken from FP64 multiply-adds instead (plain_elements(), and the reduction of long
+// contractions).  At that line the digits err by at most n 2^-53 sum |a| |b|, the a-priori bound of n multiply-adds, and
+// typically by half of 2^-53 sum |a| |b|.  Dense seeded bases have 1e-5 or fewer such elements; sparse or decaying
+// operands as many as need them: the 4 x 4 cluster (noise of 1e-17 beside entries of 1) one in seven, for which its
+// gradients take 97 ms instead of 31 with none (160 with all products on the CUDA cores).
+//
+// Against an extended-precision reference the right-hand side of a seeded basis at nb = 24 errs by 2.6e-16 (GW) and 3.8e-16
+// (TPP, complex w) in the 2-norm; FP64 multiply-adds by 6.2e-16 and 9.3e-16, plain FP64 torch by 6.0e-16 and 9.0e-16.
 //
 // The digits are cut on the integer pipe, and the sums converted on both (fixed_to_double_*): FP64 instructions
 // alone would cost as much as the MMAs (two per SM and clock).  A row or column that holds an Inf or a NaN has
-// no digits; its outputs are recomputed with FP64 multiply-adds in the epilogue, which gives
-// the values the CUDA-core kernel gives.
+// no digits; its elements are taken from FP64 multiply-adds too.
 #include "g1g2_internal.h"
 #include "tc_ptx.cuh"
 
@@ -41,11 +48,10 @@ namespace {
 
 using namespace tc;
 
-// Digits per real operand: seven of a 56-bit number, in long contractions eight of a 63-bit one.  There one large entry
-// of a sparse cotangent sets the exponent of its segment, and the sums cancel: with seven digits the drive gradient
-// of the 4 x 4 cluster was up to three times further off than from FP64 multiply-adds.
-__host__ __device__ constexpr int digits_of(bool lng) { return lng ? 8 : 7; }
+constexpr int kDig = 8;                    // digits per real operand
 constexpr int kOrd = 8;                    // orders of digit products
+// A row's exponent comes with the number of its terms that are not zero (of either part's, in long contractions)
+constexpr int kExpBits = 11, kExpMask = (1 << kExpBits) - 1;
 constexpr int kTM = 128;                   // rows of A per tile (TMEM lanes)
 constexpr int kTNMax = 128;                // real columns per tile, at most
 constexpr int kKB = 16;                    // K elements per block: one MMA step, 32-byte rows
@@ -60,10 +66,9 @@ constexpr int kMaxGroups = (kTNMax / 8 + kPerQuarter - 1) / kPerQuarter;   // gr
 static_assert(kMaxGroups * 4 <= 32, "one lane per column exponent");
 constexpr int kStgPitch = 5;               // complex per staged row (4 used)
 constexpr uint32_t kStgWarp = 32 * kStgPitch * 16;
-// A and B blocks (at most 128 columns) per stage, and the staging tiles; long contractions have larger blocks but no
-// staging
-constexpr size_t kSmem = 1024 + kStages * 2 * 7 * kADig + kEpiWarps * kStgWarp + 256;
-static_assert(kStages * 2 * 8 * kADig <= kStages * 2 * 7 * kADig + kEpiWarps * kStgWarp, "stages of a long contraction");
+// A and B blocks (at most 128 columns) per stage, and the staging tiles
+constexpr size_t kSmem = 1024 + kStages * 2 * kDig * kADig + kEpiWarps * kStgWarp + 256;
+static_assert(kSmem <= 227 * 1024, "shared memory of a CTA");
 
 constexpr int kNonFinite = 2047;           // row exponent of a row with an Inf or a NaN
 constexpr int kZeroRow = 1023;             // of a row of zeros (any other would do: its digits are zero)
@@ -89,33 +94,32 @@ __device__ __forceinline__ long long k_offset(const Operand &o, int k) {
   return (long long)b * o.kout + (long long)(k - b * o.kin) * o.sk;
 }
 
-// The ND digits of x at row exponent emax as one word: d_s + 128 is byte ND - 1 - s, and d_0 + 128 of ND = 7, which can be
-// 256, the upper 16 bits (a balanced base-256 expansion is the plain one of X + 128 (256^0 + ..)).
-// X = x 2^(B + 1022 - emax) to nearest, B = 55 bits (ND = 7) or 62 (ND = 8).
-template <int ND>
+// The digits of x at row exponent emax as one word: d_s + 128 is byte 7 - s (a balanced base-256 expansion is the plain
+// one of X + 128 (256^0 + ..)).  X = x 2^(1084 - emax) to nearest, |X| < 2^62, so |d_0| <= 64.
 __device__ __forceinline__ unsigned long long digits(double x, int emax) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int e = (hi >> 20) & 0x7ff;
   const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo;
   unsigned long long q;                      // floor(2 |X|); shifts of 64 and more give 0
-  asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"(m << (ND == 7 ? 3 : 10)), "r"(emax - max(e, 1)));
+  asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"(m << 10), "r"(emax - max(e, 1)));
   q = (q + 1) >> 1;
   const long long s = (long long)((int)hi >> 31);
-  return (q ^ (unsigned long long)s) + ((ND == 7 ? 0x0080808080808080ull : 0x8080808080808080ull) - (unsigned long long)s);
+  return (q ^ (unsigned long long)s) + (0x8080808080808080ull - (unsigned long long)s);
+}
+
+// |x| 2^(1023 - emax) cut to BF16, at least 2^-60 unless x is zero.  A sum of products of these is a lower bound of
+// sum |a| |b| in units of the two rows' exponents (the floor adds less than 2^-50), and zero only if every product is.
+__device__ __forceinline__ uint32_t magnitude(double x, int emax) {
+  const uint32_t hi = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+  const int v = hi >= 0x100000u ? (int)(hi >> 13) - ((emax - 127) << 7) : 0;   // a subnormal x: the floor
+  return (hi | (uint32_t)__double2loint(x)) == 0 ? 0u : (uint32_t)max(v, (127 - 60) << 7);
 }
 
 // d_s of two neighbouring elements as a BF16 pair.  A byte b = d + 128 below 128 becomes (128 + b) - 256, one from 128 on
 // b - 128, where 128 + (b mod 128) is a BF16 number with the seven low bits of b as its mantissa: both differences are exact.
-// The 9-bit leading digit goes through FP32: 2^23 + b is an FP32 number, and a small integer has nothing in the low half of
-// its FP32 word.
-template <int ND, int S>
+template <int S>
 __device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned long long b) {
-  if (S == 0 && ND == 7) {
-    const float fa = __uint_as_float(__byte_perm((uint32_t)(a >> 32), 0x4B000000u, 0x7632)) - 8388736.0f;
-    const float fb = __uint_as_float(__byte_perm((uint32_t)(b >> 32), 0x4B000000u, 0x7632)) - 8388736.0f;
-    return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
-  }
-  constexpr int byte = ND - 1 - S;
+  constexpr int byte = kDig - 1 - S;
   const uint32_t wa = byte < 4 ? (uint32_t)a : (uint32_t)(a >> 32), wb = byte < 4 ? (uint32_t)b : (uint32_t)(b >> 32);
   const uint32_t w = __byte_perm(wa, wb, (byte & 3) | (4 | (byte & 3)) << 8);
   uint32_t d;
@@ -123,22 +127,23 @@ __device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned lo
   return d;
 }
 
-// Digit planes in global memory, ready for the MMA: block (tile of TR rows, K block) holds ND planes
+// Digit planes in global memory, ready for the MMA: block (tile of TR rows, K block) holds kDig planes
 // of TR rows x 32 bytes in the 32-byte-swizzled K-major layout, so that the GEMM brings the leading planes
-// of a block in with one contiguous bulk copy and no tensor map.
-template <int ND>
-__device__ __forceinline__ void store_digits(uint8_t *out, int TR, int KB, int row, int q, const unsigned long long (&w)[8],
-                                             uint32_t flip) {
+// of a block in with one contiguous bulk copy and no tensor map.  The plane of magnitudes is an array of its own: those
+// of eight K blocks come with one copy.
+__device__ __forceinline__ void store_digits(uint8_t *out, uint8_t *mag, int TR, int KB, int row, int q,
+                                             const unsigned long long (&w)[8], uint32_t flip, const uint4 &m) {
   const int tile = row / TR, rr = row - tile * TR, kb = q >> 1, c2 = q & 1;
   const uint32_t plane = (uint32_t)TR * 32;
-  uint8_t *o = out + ((size_t)tile * KB + kb) * (ND * plane) + rr * 32 + ((c2 ^ ((rr >> 2) & 1)) << 4);
-#define G1G2_PUT(S)                                                                                          \
-  *reinterpret_cast<uint4 *>(o + S * plane) =                                                                \
-      make_uint4(digit_pair<ND, S>(w[0], w[1]) ^ flip, digit_pair<ND, S>(w[2], w[3]) ^ flip,                 \
-                 digit_pair<ND, S>(w[4], w[5]) ^ flip, digit_pair<ND, S>(w[6], w[7]) ^ flip)
-  G1G2_PUT(0); G1G2_PUT(1); G1G2_PUT(2); G1G2_PUT(3); G1G2_PUT(4); G1G2_PUT(5); G1G2_PUT(6);
-  if constexpr (ND > 7) G1G2_PUT(7);
+  const size_t block = (size_t)tile * KB + kb, at = rr * 32 + ((c2 ^ ((rr >> 2) & 1)) << 4);
+  uint8_t *o = out + block * (kDig * plane) + at;
+#define G1G2_PUT(S)                                                                              \
+  *reinterpret_cast<uint4 *>(o + S * plane) =                                                    \
+      make_uint4(digit_pair<S>(w[0], w[1]) ^ flip, digit_pair<S>(w[2], w[3]) ^ flip,             \
+                 digit_pair<S>(w[4], w[5]) ^ flip, digit_pair<S>(w[6], w[7]) ^ flip)
+  G1G2_PUT(0); G1G2_PUT(1); G1G2_PUT(2); G1G2_PUT(3); G1G2_PUT(4); G1G2_PUT(5); G1G2_PUT(6); G1G2_PUT(7);
 #undef G1G2_PUT
+  *reinterpret_cast<uint4 *>(mag + block * plane + at) = m;
 }
 
 // How a complex operand becomes real rows:
@@ -152,29 +157,29 @@ constexpr int kCutVals = 4096;   // complex values of an operand per CTA: one se
 __host__ __device__ constexpr int seg_k(int form) { return form == kPlanes ? 256 : 128; }   // operand K values per segment
 __host__ __device__ constexpr int cut_rows(int form) { return kCutVals / seg_k(form); }
 
-// Cuts rows x K of an operand into digits, and finds the exponents.  A CTA stages one segment of 32 rows (16 for
-// kPlanes) in shared memory, read along whichever index is contiguous in memory, takes the largest exponent of each
-// row there, and every thread then cuts eight consecutive K values of one row at a time into seven (eight)
-// 16-byte stores; a warp writes 16 rows x 32 bytes, 512 contiguous bytes, per digit.  Bound by its 16
-// bytes read and 28 written per complex element (56 for kReal).  The phases of a CTA only overlap with those of others:
-// 40 registers for six CTAs per SM.  nb = 64 operand (268 MB read, 470 MB written): 199 us with one load in flight per
-// thread and four CTAs, 172 with four loads, 160 with six CTAs (4.6 TB/s).
+// Cuts rows x K of an operand into digits and magnitudes, and finds the exponents and the numbers of nonzero terms.  A CTA
+// stages one segment of 32 rows (16 for kPlanes) in shared memory, read along whichever index is contiguous in memory, takes
+// the largest exponent of each row there, and every thread then cuts eight consecutive K values of one row at a time into nine
+// 16-byte stores; a warp writes 16 rows x 32 bytes, 512 contiguous bytes, per plane.  Bound by its 16
+// bytes read and 36 written per complex element (72 for kReal).  The phases of a CTA only overlap with those of others:
+// five CTAs per SM.  nb = 64 operand (268 MB read, 604 MB written): 181 us (4.8 TB/s); six CTAs (40 registers) 180,
+// but 203 instead of 199 in GW products and 15.6 instead of 15.2 at nb = 27.
 struct CutJob {
   Operand o;               // o.rows: rows of the panel
   int r_begin, TR;
   int *rexp;
-  uint8_t *out;
+  uint8_t *out, *mag;
 };
 template <int FORM>
 __device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_begin, int Klen, int Kp, int KB, int SK) {
-  constexpr int SR = cut_rows(FORM), ND = digits_of(FORM == kPlanes);
+  constexpr int SR = cut_rows(FORM);
   extern __shared__ double sh[];
   __shared__ long long roff[SR], koff[seg_k(FORM)];
   __shared__ int emax[SR];
   const Operand &A = job.o;
   const int r_begin = job.r_begin, TR = job.TR;
   int *__restrict__ rexp = job.rexp;
-  uint8_t *__restrict__ out = job.out;
+  uint8_t *__restrict__ out = job.out, *__restrict__ mag = job.mag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r0 = block * SR;                              // within the panel
   const int nr = min(SR, A.rows - r0);                    // A.rows: rows of the panel
@@ -216,22 +221,23 @@ __device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_b
   {
     constexpr int T = 256 / SR;                           // threads per row
     const int r = tid / T, j = tid % T;
-    int e = 0, low = 0;
+    int e = 0, terms = 0;
     for (int k = j; k < kt; k += T) {
       const double x = re[r * pitch + k], y = im[r * pitch + k];
-      e = max(e, max(__double2hiint(x) & 0x7fffffff, __double2hiint(y) & 0x7fffffff));
-      low |= __double2loint(x) | __double2loint(y);
+      const int hx = __double2hiint(x) & 0x7fffffff, hy = __double2hiint(y) & 0x7fffffff;
+      const int nx = (hx | __double2loint(x)) != 0, ny = (hy | __double2loint(y)) != 0;
+      e = max(e, max(hx, hy));
+      terms += FORM == kPlanes ? nx | ny : nx + ny;
     }
-    low = (low != 0);
 #pragma unroll
     for (int o = T / 2; o > 0; o >>= 1) {
       e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-      low |= __shfl_xor_sync(0xffffffffu, low, o);
+      terms += __shfl_xor_sync(0xffffffffu, terms, o);
     }
-    e = (e | low) == 0 ? kZeroRow : max(e >> 20, 1);
+    e = terms == 0 ? kZeroRow : max(e >> 20, 1);
     if (j == 0) {
       emax[r] = e;
-      if (r < nr) rexp[(size_t)seg * A.rows + r0 + r] = e;
+      if (r < nr) rexp[(size_t)seg * A.rows + r0 + r] = e | terms << kExpBits;
     }
   }
   __syncthreads();
@@ -244,16 +250,22 @@ __device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_b
     const double *src = (u ? im : re) + r * pitch + kc * 8;
     const int e = emax[r];
     unsigned long long w[8];
+    uint32_t mg[4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = digits<ND>(e == kNonFinite ? 0.0 : src[i], e);
+    for (int i = 0; i < 8; ++i) {
+      const double x = e == kNonFinite ? 0.0 : src[i];
+      w[i] = digits(x, e);
+      mg[i / 2] = i & 1 ? mg[i / 2] | magnitude(x, e) << 16 : magnitude(x, e);
+    }
+    const uint4 m = make_uint4(mg[0], mg[1], mg[2], mg[3]);
     const int q0 = seg * (SK / (FORM == kPlanes ? 8 : 4)), row = r0 + r;          // 16-byte chunks before this segment
     if (FORM == kRows) {
-      store_digits<ND>(out, TR, KB, row, q0 + u * nch + kc, w, 0u);
+      store_digits(out, mag, TR, KB, row, q0 + u * nch + kc, w, 0u, m);
     } else if (FORM == kReal) {
-      store_digits<ND>(out, TR, KB, 2 * row, q0 + u * nch + kc, w, u ? 0x80008000u : 0u);
-      store_digits<ND>(out, TR, KB, 2 * row + 1, q0 + (1 - u) * nch + kc, w, 0u);
+      store_digits(out, mag, TR, KB, 2 * row, q0 + u * nch + kc, w, u ? 0x80008000u : 0u, m);
+      store_digits(out, mag, TR, KB, 2 * row + 1, q0 + (1 - u) * nch + kc, w, 0u, m);
     } else {
-      store_digits<ND>(out, TR, KB, 2 * row + u, q0 + kc, w, 0u);
+      store_digits(out, mag, TR, KB, 2 * row + u, q0 + kc, w, 0u, m);
     }
   }
 }
@@ -261,7 +273,7 @@ __device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_b
 // Both operands of a product in one launch: blocks below xblocks cut x, the others y.  (The column operand is small: as
 // a launch of its own it took 5 us of the 50 us of a mode product at nb = 32.)
 template <int FX, int FY>
-__global__ void __launch_bounds__(256, 6) cut_digits_kernel(const CutJob x, const CutJob y, int xblocks, int k_begin, int Klen,
+__global__ void __launch_bounds__(256, 5) cut_digits_kernel(const CutJob x, const CutJob y, int xblocks, int k_begin, int Klen,
                                                          int Kp, int KB, int SK) {
   dependent_begin();
   if ((int)blockIdx.x < xblocks) cut_digits<FX>(x, blockIdx.x, k_begin, Klen, Kp, KB, SK);
@@ -273,6 +285,7 @@ __global__ void __launch_bounds__(256, 6) cut_digits_kernel(const CutJob x, cons
 // ---------------------------------------------------------------------------
 struct TcGemm {
   const uint8_t *A, *B;       // digit blocks
+  const uint8_t *MA, *MB;     // magnitudes
   int KB, segs, kseg;         // K blocks of a row tile, in segments of kseg
   int nt;                     // real columns per tile (multiple of 16)
   int mtiles, ntiles;         // unit = (split mtiles + m_tile) ntiles + n_tile
@@ -281,6 +294,9 @@ struct TcGemm {
   long long *sums;            // per CTA: [hi, lo][column][row] of a segment
   double *part;               // FP64 sums over segments [unit (long contractions) or CTA][column][row]
   int accumulate;             // long contractions: part holds earlier panels
+  uint32_t *flags, *any;      // long contractions: masks of the elements left to the reduction, [tile][column group][row][segment],
+                              // and their union over the segments of a unit, [unit][column group][row]
+  int all_segs, seg_begin;    // segments of all panels, the first one of this panel
   Operand X, Y;               // rows r_begin + m of X, columns y_begin + y of Y, K from k_begin
   const int *ex, *ey;         // exponents [segment][row of the panel]
   int exs, eys;               // rows of the panel
@@ -320,6 +336,12 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
                : "memory");
 }
 
+// Whether s = sum |a| |b| over at most terms products, in units of the two rows' exponents, is too small for the digits
+// (0 < s < sqrt(terms) / 64, with at least 16 terms)
+__device__ __forceinline__ bool too_small(float s, int terms) {
+  return s > 0.f && s * s < (float)max(terms, 16) * (1.f / 4096.f);
+}
+
 // (hi 2^32 + lo) 2^e as FP64, rounded to nearest, without a branch, for |hi| < 2^62, |lo| < 2^62 and kMinE <= e <= kMaxE (no
 // subnormal or infinite result then).  Two forms, because either alone is bound by its own pipe:
 //   fixed_to_double_add: the upper 52 bits and the lower 44 as mantissas at 1.5 2^96 and 1.5 2^52; two FP64 additions
@@ -327,7 +349,7 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
 //   fixed_to_double_int: the 96-bit magnitude is shifted left to its leading one by whole words and a funnel shift: about
 //       forty integer instructions.
 // The real parts take the one and the imaginary parts the other; long contractions, which add segments up on the FP64 pipe,
-// the second alone.  Mode product at nb = 64, us: additions only 378, integers only 343, both 341.
+// the second alone.  Mode product at nb = 64 (seven digits), us: additions only 378, integers only 343, both 341.
 constexpr int kMinE = -1022, kMaxE = 927;
 __device__ __forceinline__ double fixed_to_double_add(long long hi, long long lo, int e) {
   hi += lo >> 32;
@@ -369,28 +391,128 @@ __device__ __forceinline__ cplx mul_unit(cplx z, int u) {
           __hiloint2double(__double2hiint(y) ^ sy, __double2loint(y))};
 }
 
-// The FP64 multiply-add sum over one segment of an output element whose row or column holds an Inf or a NaN there.
-__device__ __noinline__ cplx plain_sum(const Operand &X, const Operand &Y, int r, int y, int k0, int k1) {
-  const cplx *a = X.p + row_offset(X, r), *b = Y.p + row_offset(Y, y);
-  cplx s = {0.0, 0.0};
-  for (int k = k0; k < k1; ++k) {
-    cplx u = a[k_offset(X, k)], v = b[k_offset(Y, k)];
-    if (X.conj) u.y = -u.y;
-    if (Y.conj) v.y = -v.y;
-    s = {fma(u.x, v.x, fma(-u.y, v.y, s.x)), fma(u.x, v.y, fma(u.y, v.x, s.y))};
-  }
-  return s;
+__device__ __forceinline__ bool is_zero(const cplx &v) {   // on the integer pipe
+  return (((__double2hiint(v.x) | __double2hiint(v.y)) & 0x7fffffff) | __double2loint(v.x) | __double2loint(v.y)) == 0;
 }
-// The same for one of the four real products of a long contraction: part pa of A times part pb of B.
-__device__ __noinline__ double plain_part(const Operand &X, const Operand &Y, int r, int pa, int y, int pb, int k0, int k1) {
-  const cplx *a = X.p + row_offset(X, r), *b = Y.p + row_offset(Y, y);
-  double s = 0.0;
-  for (int k = k0; k < k1; ++k) {
-    const cplx u = a[k_offset(X, k)], v = b[k_offset(Y, k)];
-    const double x = pa ? (X.conj ? -u.y : u.y) : u.x, z = pb ? (Y.conj ? -v.y : v.y) : v.x;
-    s = fma(x, z, s);
+__device__ __forceinline__ double flip(double v, int sign) {
+  return __hiloint2double(__double2hiint(v) ^ sign, __double2loint(v));
+}
+// s += u v, conjugated where fu, fv is the sign bit
+__device__ __forceinline__ void plain_fma(cplx &s, const cplx &u, const cplx &v, int fu, int fv) {
+  const double ui = flip(u.y, fu), vi = flip(v.y, fv);
+  s = {fma(u.x, v.x, fma(-ui, vi, s.x)), fma(u.x, vi, fma(ui, v.x, s.y))};
+}
+// One segment (k0..k1) of the elements that the digits do not give, by FP64 multiply-adds, into the slots of their high
+// sums: bit c = 4 i + j of a lane's mask is complex column y0 + 12 i + j of its row, xt the terms of that row that are not
+// zero, yt those of column c = lane.  Three ways, by the cycles that they keep the FP64 pipe busy (64 per warp and term, 160
+// for sums over the lanes), since such operands are mostly sparse and terms with a zero are left out (unless
+// there is an Inf or a NaN): a row at a time with the columns over the lanes, a column with the rows over the lanes, and
+// single elements with the terms over the lanes.
+__device__ __noinline__ void plain_elements(const TcGemm &p, uint32_t mask, bool finite, int xt, int yt, int row0, int y0, int k0,
+                                            int k1, long long *hi) {
+  const int lane = threadIdx.x & 31, K = k1 - k0;
+  const Operand &X = p.X, &Y = p.Y;
+  const int fx = X.conj ? (int)0x80000000u : 0, fy = Y.conj ? (int)0x80000000u : 0;
+  auto row = [&](int m) { return X.p + row_offset(X, p.r_begin + min(m, p.rows - 1)); };   // lanes beyond the panel: its last
+  auto put = [&](int y, int r, const cplx &s) {
+    __stcg(hi + (size_t)(2 * y) * kTM + r, __double_as_longlong(s.x));
+    __stcg(hi + (size_t)(2 * y + 1) * kTM + r, __double_as_longlong(s.y));
+  };
+  const uint32_t cols = __reduce_or_sync(0xffffffffu, mask);
+  const int by_rows = __reduce_add_sync(0xffffffffu, mask ? min(K, xt) : 0);
+  const int by_cols = __reduce_add_sync(0xffffffffu, cols >> lane & 1u ? min(K, yt) : 0);
+  const int single = (__reduce_add_sync(0xffffffffu, __popc(mask)) * (2 * K + 160)) >> 6;
+  __syncwarp();
+  if (by_rows < min(by_cols, single)) {
+    const int y = 4 * kPerQuarter * (lane >> 2) + (lane & 3);      // this lane's column
+    const cplx *b = Y.p + row_offset(Y, p.y_begin + y0) + y * Y.sx;
+    uint32_t rows = __ballot_sync(0xffffffffu, mask != 0);
+    int r = __ffs((int)rows) - 1, kb = k0;
+    auto load = [&]() { return kb + lane < k1 ? row(row0 + r)[(kb + lane) * X.sk] : cplx{0.0, 0.0}; };
+    cplx next = load(), s = {0.0, 0.0};
+    while (r >= 0) {
+      const cplx u = next;
+      const int r_now = r, kb_now = kb;
+      kb += 32;
+      if (kb >= k1) {                                              // the next row's terms are loaded ahead
+        kb = k0;
+        rows &= rows - 1;
+        r = __ffs((int)rows) - 1;
+      }
+      if (r >= 0) next = load();
+      const bool mine = __shfl_sync(0xffffffffu, mask, r_now) >> lane & 1u;
+      uint32_t nz = __ballot_sync(0xffffffffu, kb_now + lane < k1 && !(finite && is_zero(u)));
+      for (; nz; nz &= nz - 1) {
+        const int q = __ffs((int)nz) - 1;
+        const cplx uq = {__shfl_sync(0xffffffffu, u.x, q), __shfl_sync(0xffffffffu, u.y, q)};
+        if (mine) plain_fma(s, uq, b[(kb_now + q) * Y.sk], fx, fy);
+      }
+      if (kb == k0) {
+        if (mine) put(y, r_now, s);
+        s = {0.0, 0.0};
+      }
+    }
+    __syncwarp();
+    return;
   }
-  return s;
+#pragma unroll 1
+  for (int g = 0; g < kMaxGroups; ++g) {
+    uint32_t col[4];
+    int n = 0, nc = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      col[j] = __ballot_sync(0xffffffffu, mask >> (4 * g + j) & 1u);
+      n += __popc(col[j]);
+      nc += col[j] != 0;
+    }
+    if (n == 0) continue;
+    const int yg = 4 * kPerQuarter * g;
+    const cplx *b = Y.p + row_offset(Y, p.y_begin + y0 + yg);
+    if (n * (2 * K + 160) < 64 * K * nc) {
+#pragma unroll 1
+      for (int j = 0; j < 4; ++j)
+#pragma unroll 1
+        for (uint32_t c = col[j]; c; c &= c - 1) {
+          const int r = __ffs((int)c) - 1;
+          const cplx *a = row(row0 + r), *bj = b + j * Y.sx;
+          cplx s = {0.0, 0.0};
+#pragma unroll 4
+          for (int k = k0 + lane; k < k1; k += 32) plain_fma(s, a[k * X.sk], bj[k * Y.sk], fx, fy);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+            s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+          }
+          if (lane == 0) put(yg + j, r, s);
+        }
+    } else {
+      const bool mine = mask >> (4 * g) & 15u;
+      const cplx *a = row(row0 + lane);
+      cplx s[4] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
+      constexpr int kAhead = 4;                        // rows' terms loaded ahead
+#pragma unroll 1
+      for (int kb = k0; kb < k1; kb += kAhead) {
+        cplx u[kAhead];
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) u[q] = kb + q < k1 ? a[(kb + q) * X.sk] : cplx{0.0, 0.0};
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) {
+          if (kb + q >= k1 || (finite && __all_sync(0xffffffffu, !mine || is_zero(u[q])))) continue;
+          const cplx *bk = b + (kb + q) * Y.sk;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (!col[j]) continue;
+            const cplx v = bk[j * Y.sx];
+            if (!(finite && is_zero(v))) plain_fma(s[j], u[q], v, fx, fy);
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (mask >> (4 * g + j) & 1u) put(yg + j, lane, s[j]);
+    }
+  }
+  __syncwarp();
 }
 
 __device__ __forceinline__ float max_abs3(float a, float b, float c) {
@@ -435,20 +557,22 @@ __device__ __forceinline__ void join_orders(const uint32_t (&v)[4][8], long long
 //
 // An MMA costs the larger of its N / 2 cycles and its operands' shared-memory reads, about (4096 + 32 N) / 88
 // (70 cycles at N = 64, 93 at 128), so wide tiles halve the cost per column.  TMEM holds 512 columns:
-//   G = 8: tiles of up to 64 columns, all eight orders at once (34 MMAs per K step);
-//   G = 4: tiles of up to 128 columns in two phases over a segment, orders 4..7 (24 MMAs), which the conversion of
-//          the last segment overlaps, then orders 0..3 (ten MMAs, four digit planes loaded).
+//   G = 8: tiles of up to 64 columns, all eight orders at once (36 MMAs per K step);
+//   G = 4: tiles of up to 128 columns in two phases over a segment, orders 4..7 (26 MMAs), which the conversion of
+//          the last segment overlaps, then orders 0..3 (ten MMAs, four digit planes loaded);
+// a last phase sums the magnitudes (one MMA per K step, eight steps' planes per stage).  It costs the wait for the tile before and
+// after: with seven digits and without it a mode product at nb = 64 took 341 us, now 370, the pair product of GW 14.3 ms,
+// now 15.0.
 // kKind: 0 one segment per unit, 1 several, 2 a long contraction (several, real products of re and im rows).
 template <int G, int kKind>
-__global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm p) {
+__global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const __grid_constant__ TcGemm p) {
   constexpr bool kSplit = kKind == 2;
-  constexpr int kPhases = kOrd / G;
+  constexpr int kMain = kOrd / G, kPhases = kMain + 1;   // of the digits, and the magnitudes
   constexpr int kTN = 512 / G;                       // TMEM columns per accumulator
-  constexpr int kDig = digits_of(kSplit);
   constexpr uint32_t kABlk = kDig * kADig, kStageBytes = 2 * kABlk;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t *stg_all = smem + kStages * kStageBytes;   // not in long contractions
+  uint8_t *stg_all = smem + kStages * kStageBytes;
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kSmem - 1024 - 256);
   uint64_t *full = bars, *empty = bars + kStages, *tfull = bars + 2 * kStages, *tempty = tfull + 1, *fin = tempty + 1;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fin + 1);
@@ -481,13 +605,16 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
         const int s0 = sp * p.segs_per_split, s1 = min(p.segs, s0 + p.segs_per_split);
         for (int sf = s0 * kPhases; sf < s1 * kPhases && ok; ++sf) {
           const int f = sf % kPhases, kb0 = (sf / kPhases) * p.kseg, kb1 = min(p.KB, kb0 + p.kseg);
-          const uint32_t nd = (kPhases == 2 && f == 1) ? 4u : (uint32_t)kDig;
-          for (int kb = kb0; kb < kb1; ++kb) {
+          // a stage: the digits of one K block (all, or the four leading ones), or the magnitudes of up to kDig
+          const bool mags = f == kMain;
+          for (int kb = kb0; kb < kb1; kb += mags ? kDig : 1) {
             if (!mbar_wait(&empty[s], ph ^ 1u, p.err)) { ok = false; break; }
             uint8_t *st = smem + (size_t)s * kStageBytes;
-            mbar_arrive_expect_tx(&full[s], nd * (kADig + bdig));
-            bulk_load(st, p.A + ((size_t)mt * p.KB + kb) * kABlk, nd * kADig, &full[s]);
-            bulk_load(st + kABlk, p.B + ((size_t)nt * p.KB + kb) * bblk, nd * bdig, &full[s]);
+            const size_t ka = (size_t)mt * p.KB + kb, kc = (size_t)nt * p.KB + kb;
+            const uint32_t np = mags ? (uint32_t)min(kDig, kb1 - kb) : f == 1 ? 4u : (uint32_t)kDig;   // planes
+            mbar_arrive_expect_tx(&full[s], np * (kADig + bdig));
+            bulk_load(st, mags ? p.MA + ka * kADig : p.A + ka * kABlk, np * kADig, &full[s]);
+            bulk_load(st + kABlk, mags ? p.MB + kc * bdig : p.B + kc * bblk, np * bdig, &full[s]);
             if (++s == kStages) { s = 0; ph ^= 1u; }
           }
         }
@@ -508,7 +635,7 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
           for (int f = 0; f < kPhases; ++f) {
             if (!ok || !mbar_wait(tempty, acc_ph ^ 1u, p.err)) { ok = false; break; }
             tc_fence_after();
-            for (int kb = kb0; kb < kb1; ++kb) {
+            for (int kb = kb0; kb < kb1; kb += f == kMain ? kDig : 1) {
               if (!mbar_wait(&full[s], ph, p.err)) { ok = false; break; }
               tc_fence_after();
               const uint32_t sa = smem_u32(smem + (size_t)s * kStageBytes), sb = sa + kABlk;
@@ -518,12 +645,18 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
                 a[q] = smem_desc_sw32(sa + q * kADig);
                 b[q] = smem_desc_sw32(sb + q * bdig);
               }
+              if (f == kMain) {
 #pragma unroll
-              for (int g = 0; g < G; ++g) {
-                const int o = (kPhases - 1 - f) * G + g, q0 = o < kDig ? 0 : o - kDig + 1;
+                for (int q = 0; q < kDig; ++q)
+                  if (kb + q < kb1) mma_bf16(tmem, a[q], b[q], idesc, (kb == kb0 && q == 0) ? 0u : 1u);
+              } else {
 #pragma unroll
-                for (int q = q0; q <= o && q < kDig; ++q)
-                  mma_bf16(tmem + (uint32_t)(g * kTN), a[q], b[o - q], idesc, (q == q0 && kb == kb0) ? 0u : 1u);
+                for (int g = 0; g < G; ++g) {
+                  const int o = (kMain - 1 - f) * G + g, q0 = o < kDig ? 0 : o - kDig + 1;
+#pragma unroll
+                  for (int q = q0; q <= o && q < kDig; ++q)
+                    mma_bf16(tmem + (uint32_t)(g * kTN), a[q], b[o - q], idesc, (q == q0 && kb == kb0) ? 0u : 1u);
+                }
               }
               mma_commit(&empty[s]);
               if (++s == kStages) { s = 0; ph ^= 1u; }
@@ -559,16 +692,16 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
         const int row = p.r_begin + m, b = row / p.X.X;
         off = (long long)b * p.scb + (long long)(row - b * p.X.X) * p.scx;
       }
+      uint32_t any = 0;
       for (int seg = s0; seg < s1 && ok; ++seg) {
         // exponents, loaded before the MMAs are waited for: lane 4 i + j holds that of column j of this warp's
         // i-th group
         const int yl = y_tile + 4 * (cg + kPerQuarter * (lane >> 2)) + (lane & 3);
-        const int ea = valid ? p.ex[(size_t)seg * p.exs + mc] : kZeroRow;
-        const int eyl = (lane < kMaxGroups * 4 && yl < p.cols) ? p.ey[(size_t)seg * p.eys + yl] : kZeroRow;
-        // rows that need care: Inf or NaN, or results that may leave the range of fixed_to_double_*
-        const bool care = __any_sync(0xffffffffu, min(ea, eyl) < kSafeLo || max(ea, eyl) > kSafeHi);
+        const int xr = valid ? p.ex[(size_t)seg * p.exs + mc] : kZeroRow;
+        const int yr = (lane < kMaxGroups * 4 && yl < p.cols) ? p.ey[(size_t)seg * p.eys + yl] : kZeroRow;
+        const int ea = xr & kExpMask, eyl = yr & kExpMask;
 #pragma unroll 1
-        for (int f = 0; f < kPhases; ++f) {
+        for (int f = 0; f < kMain; ++f) {
           if (!__all_sync(0xffffffffu, mbar_wait(tfull, acc_ph, p.err))) { ok = false; break; }
           tc_fence_after();
 #pragma unroll 1
@@ -594,9 +727,42 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
           acc_ph ^= 1u;
         }
         if (!ok) break;
+        // elements whose sum of magnitudes is too small for the digits, or with an Inf or a NaN (bit 4 i + j: column j of
+        // this lane's i-th group)
+        if (!__all_sync(0xffffffffu, mbar_wait(tfull, acc_ph, p.err))) { ok = false; break; }
+        tc_fence_after();
+        uint32_t plain = 0;
+#pragma unroll 1
+        for (int g = cg, gl = 0; g < ngroups; g += kPerQuarter, gl += 4) {
+          uint32_t v[8];
+          tmem_ld8(tmem + lane_base + (uint32_t)(8 * g), v);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          after_wait(v);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int yj = __shfl_sync(0xffffffffu, yr, gl + j);
+            const int terms = min(xr, yj) >> kExpBits;
+            const bool low = too_small(__uint_as_float(v[2 * j]), terms) || too_small(__uint_as_float(v[2 * j + 1]), terms);
+            if ((low || max(ea, yj & kExpMask) == kNonFinite) && y_tile + 4 * g + j < p.cols) plain |= 1u << (gl + j);
+          }
+        }
+        if (!valid) plain = 0;
+        tc_fence_before();
+        mbar_arrive(tempty);
+        acc_ph ^= 1u;
+        const bool some = __any_sync(0xffffffffu, plain != 0);
+        if constexpr (kSplit) {                         // fp64_tc_reduce_kernel adds them: here they may fill a few CTAs' segments
+          p.flags[((size_t)((mt * p.ntiles + ntile) * kPerQuarter + cg) * kTM + r) * p.all_segs + p.seg_begin + seg] = plain;
+          any |= plain;
+        } else if (some) {
+          const bool finite = !__any_sync(0xffffffffu, max(ea, eyl) == kNonFinite);
+          const int k0 = seg * seg_k(kRows);
+          plain_elements(p, plain, finite, xr >> kExpBits, yr >> kExpBits, mt * kTM + 32 * quarter, y_tile + 4 * cg, k0, min(p.X.K, k0 + seg_k(kRows)),
+                         sums - lane + (size_t)(8 * cg) * kTM);
+        }
+        // those, or results that may leave the range of fixed_to_double_*
+        const bool care = some || __any_sync(0xffffffffu, min(ea, eyl) < kSafeLo || max(ea, eyl) > kSafeHi);
         const bool first = seg == s0 && !(kSplit && p.accumulate), last = seg == s1 - 1;
-        const int seg_len = kSplit ? p.kseg * kKB : seg_k(kRows);
-        const int k0 = p.k_begin + seg * seg_len, k1 = min(p.X.K, k0 + seg_len);
         // two copies: with the calls of the careful one in its loop, the plain one spilled registers
         auto convert = [&](auto careful) {
         constexpr bool kCare = decltype(careful)::value;
@@ -616,7 +782,7 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
           double v[8];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const int e0 = ea + __shfl_sync(0xffffffffu, eyl, gl + j) - (kSplit ? 2112 : 2114);
+            const int e0 = ea + __shfl_sync(0xffffffffu, eyl, gl + j) - 2112;
             const int e = kCare ? min(max(e0, kMinE), kMaxE) : e0;
             v[2 * j] = kSplit ? fixed_to_double_int(hi[2 * j], lo[2 * j], e) : fixed_to_double_add(hi[2 * j], lo[2 * j], e);
             v[2 * j + 1] = fixed_to_double_int(hi[2 * j + 1], lo[2 * j + 1], e);
@@ -625,18 +791,10 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
                 v[2 * j] = beyond_range(v[2 * j], e0 - e);
                 v[2 * j + 1] = beyond_range(v[2 * j + 1], e0 - e);
               }
-              const int eb = __shfl_sync(0xffffffffu, eyl, gl + j);   // every lane: not behind a condition
-              if ((ea == kNonFinite || eb == kNonFinite) && valid && j < ny) {
-                if (kSplit) {
-                  v[2 * j] = plain_part(p.X, p.Y, mc, m & 1, y0 + j, 0, k0, k1);
-                  v[2 * j + 1] = plain_part(p.X, p.Y, mc, m & 1, y0 + j, 1, k0, k1);
-                } else {
-                  const cplx z = plain_sum(p.X, p.Y, p.r_begin + m, p.y_begin + y0 + j, k0, k1);
-                  v[2 * j] = z.x;
-                  v[2 * j + 1] = z.y;
-                }
+              if (plain >> (gl + j) & 1u) {
+                v[2 * j] = kSplit ? 0.0 : __longlong_as_double(hi[2 * j]);
+                v[2 * j + 1] = kSplit ? 0.0 : __longlong_as_double(hi[2 * j + 1]);
               }
-              __syncwarp();
             }
           }
           if (kKind != 0 && !first) {   // (in one-segment kernels the compiler would add a zero, on the slow FP64 pipe)
@@ -702,6 +860,10 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
         if (care) convert(std::true_type{});
         else convert(std::false_type{});
       }
+      if constexpr (kSplit) {
+        uint32_t *a = p.any + (size_t)(u * kPerQuarter + cg) * kTM + r;
+        *a = p.accumulate ? *a | any : any;
+      }
     }
   }
   __syncthreads();
@@ -712,25 +874,59 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const TcGemm 
 }
 
 // Sums the units of a long contraction in a fixed order and combines the four real products:
-// C[i][j] = alpha ((re re - im im) + i (re im + im re)) + beta C.  One warp per output element.
-__global__ void __launch_bounds__(256) fp64_tc_reduce_kernel(const TcGemm p) {
-  dependent_begin();
-  const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (idx >= p.rows * p.cols) return;
-  const int i = idx / p.cols, j = idx - i * p.cols;
+// C[i][j] = alpha ((re re - im im) + i (re im + im re)) + beta C.  One CTA per output element, which also adds the
+// segments that the digits do not give, by FP64 multiply-adds (bits of rows 2 i and 2 i + 1 for column j).  Here the whole chip
+// shares them: taken in the GEMM they kept one SM busy for 540 us with the sparse cotangents of the 4 x 4 cluster (202 us
+// with one warp per element).  The next kernel may start once these are done: its CTAs would take the L1 from their loads.
+constexpr int kRedThreads = 128;
+__global__ void __launch_bounds__(kRedThreads) fp64_tc_reduce_kernel(const TcGemm p) {
+  __shared__ double sx[kRedThreads / 32], sy[kRedThreads / 32];
+  dependent_wait();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int i = blockIdx.x / p.cols, j = blockIdx.x - i * p.cols;
   const int mt = 2 * i / kTM, nt = 2 * j / p.nt, rr = 2 * i - mt * kTM, cc = 2 * j - nt * p.nt;
+  const int grp = cc >> 3, cg = grp % kPerQuarter, bit = 4 * (grp / kPerQuarter) + ((cc >> 1) & 3);
   double x = 0.0, y = 0.0;
-  for (int sp = lane; sp < p.splits; sp += 32) {
-    const double *q = p.part + ((size_t)(sp * p.mtiles + mt) * p.ntiles + nt) * kTNMax * kTM + (size_t)cc * kTM + rr;
+  uint32_t any = 0;
+  for (int sp = tid; sp < p.splits; sp += kRedThreads) {
+    const size_t unit = (size_t)(sp * p.mtiles + mt) * p.ntiles + nt;
+    const double *q = p.part + unit * kTNMax * kTM + (size_t)cc * kTM + rr;
     x += q[0] - q[kTM + 1];
     y += q[kTM] + q[1];
+    const uint32_t *a = p.any + (unit * kPerQuarter + cg) * kTM + rr;
+    any |= (a[0] | a[1]) >> bit & 1u;
   }
+  if (__syncthreads_or(any)) {
+    const uint32_t *fl = p.flags + ((size_t)((mt * p.ntiles + nt) * kPerQuarter + cg) * kTM + rr) * p.all_segs;
+    const cplx *a = p.X.p + row_offset(p.X, i), *b = p.Y.p + row_offset(p.Y, j);
+    const int fx = p.X.conj ? (int)0x80000000u : 0, fy = p.Y.conj ? (int)0x80000000u : 0, len = p.kseg * kKB;
+    for (int s0 = 32 * warp; s0 < p.all_segs; s0 += kRedThreads) {
+      const bool in = s0 + lane < p.all_segs;
+      const uint32_t re = __ballot_sync(0xffffffffu, in && (fl[s0 + lane] >> bit & 1u));
+      const uint32_t im = __ballot_sync(0xffffffffu, in && (fl[p.all_segs + s0 + lane] >> bit & 1u));
+      for (uint32_t m = re | im; m; m &= m - 1) {
+        const int s = __ffs((int)m) - 1, k1 = min(p.X.K, (s0 + s + 1) * len);
+        const bool r = re >> s & 1u, t = im >> s & 1u;
+#pragma unroll 8
+        for (int k = (s0 + s) * len + lane; k < k1; k += 32) {
+          const cplx u = a[k_offset(p.X, k)], v = b[k_offset(p.Y, k)];
+          const double ui = flip(u.y, fx), vi = flip(v.y, fy);
+          if (r) { x = fma(u.x, v.x, x); y = fma(u.x, vi, y); }
+          if (t) { x = fma(-ui, vi, x); y = fma(ui, v.x, y); }
+        }
+      }
+    }
+  }
+  dependent_launch();
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     x += __shfl_xor_sync(0xffffffffu, x, o);
     y += __shfl_xor_sync(0xffffffffu, y, o);
   }
-  if (lane != 0) return;
+  if (lane == 0) { sx[warp] = x; sy[warp] = y; }
+  __syncthreads();
+  if (tid != 0) return;
+  for (int w = 1; w < kRedThreads / 32; ++w) { x += sx[w]; y += sy[w]; }
   cplx z = mul_unit({x, y}, p.unit_alpha);
   cplx *c = p.C + (long long)i * p.scx + (long long)j * p.scy;
   if (p.beta) z = {z.x + c->x, z.y + c->y};
@@ -774,8 +970,8 @@ void launch_gemm(Launcher &L, const TcGemm &t, int ctas, const char *tag) {
   L.after_launch();
 }
 
-CutJob cut_job(const Operand &o, int r_begin, int rows, int TR, int *rexp, uint8_t *out) {
-  CutJob j{o, r_begin, TR, rexp, out};
+CutJob cut_job(const Operand &o, int r_begin, int rows, int TR, int *rexp, uint8_t *out, uint8_t *mag) {
+  CutJob j{o, r_begin, TR, rexp, out, mag};
   j.o.rows = rows;
   return j;
 }
@@ -807,11 +1003,14 @@ int fp64_tc_min_nb(bool pair_products) { return pair_products ? 12 : 17; }
 
 struct Fp64Tc {
   uint8_t *A = nullptr, *B = nullptr;   // digit blocks of the two operands
+  uint8_t *MA = nullptr, *MB = nullptr; // their magnitudes, an eighth of the size
   size_t a_bytes = 0, b_bytes = 0;
   int *ex = nullptr, *ey = nullptr;     // exponents
   long long exps = 0;                   // of each
   long long *sums = nullptr;            // hi and lo sums of a tile per CTA
   double *part = nullptr;               // FP64 sums of a tile per CTA
+  uint32_t *flags = nullptr, *any = nullptr;   // elements of long contractions that the digits do not give
+  long long flag_words = 0;
   int *err = nullptr;
   int sms = 0;
   int yK = 0, ycols = 0, ynt = 0;       // shape of the column operand whose digits B holds whole (0: none)
@@ -819,7 +1018,8 @@ struct Fp64Tc {
 
 void fp64_tc_destroy(Fp64Tc *f) {
   if (!f) return;
-  for (void *p : {(void *)f->A, (void *)f->B, (void *)f->ex, (void *)f->ey, (void *)f->sums, (void *)f->part, (void *)f->err})
+  for (void *p : {(void *)f->A, (void *)f->B, (void *)f->MA, (void *)f->MB, (void *)f->ex, (void *)f->ey, (void *)f->sums, (void *)f->part, (void *)f->flags,
+                  (void *)f->any, (void *)f->err})
     if (p) cudaFree(p);
   delete f;
 }
@@ -830,23 +1030,25 @@ Fp64Tc *fp64_tc_create(int nb, bool pair_products) {
   if (!f) return nullptr;
   // digit blocks: all of a big operand up to kPanelBytes, panels of it above
   constexpr size_t kPanelBytes = (size_t)1 << 30;
-  auto blocks = [](long long rows, long long Kp, bool lng = false) {
-    return (size_t)((rows + 127) / 128 * 128) * (size_t)Kp * 2 * digits_of(lng);
-  };
+  auto blocks = [](long long rows, long long Kp) { return (size_t)((rows + 127) / 128 * 128) * (size_t)Kp * 2 * kDig; };
   const size_t big = blocks(N3, 2 * ((N + 7) / 8 * 8)), pair = pair_products ? blocks(2 * N2 + kTNMax, 2 * ((N2 + 7) / 8 * 8)) : 0;
-  const size_t lng = blocks(2 * N, (N3 + 255) / 256 * 256, true);
+  const size_t lng = blocks(2 * N, (N3 + 255) / 256 * 256);
   f->a_bytes = std::min(kPanelBytes, std::max({big, pair, lng}));
   f->b_bytes = std::min(kPanelBytes, std::max({blocks(2 * N, 2 * ((N + 7) / 8 * 8)), pair, lng}));
   f->exps = std::max({N3, N2 * ((N2 + 127) / 128), N * ((N3 + 127) / 128)});
+  f->flag_words = (N3 + 127) / 128 * ((2 * N + kTM - 1) / kTM) * ((2 * N + kTNMax - 1) / kTNMax) * kPerQuarter * kTM;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&f->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     goto bad;
   if (cudaMalloc(&f->A, f->a_bytes) != cudaSuccess || cudaMalloc(&f->B, f->b_bytes) != cudaSuccess ||
+      cudaMalloc(&f->MA, f->a_bytes / kDig) != cudaSuccess || cudaMalloc(&f->MB, f->b_bytes / kDig) != cudaSuccess ||
       cudaMalloc(&f->ex, sizeof(int) * (size_t)f->exps) != cudaSuccess ||
       cudaMalloc(&f->ey, sizeof(int) * (size_t)f->exps) != cudaSuccess ||
       cudaMalloc(&f->sums, (size_t)f->sms * 2 * kTNMax * kTM * sizeof(long long)) != cudaSuccess ||
       cudaMalloc(&f->part, (size_t)f->sms * kTNMax * kTM * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&f->flags, sizeof(uint32_t) * (size_t)f->flag_words) != cudaSuccess ||
+      cudaMalloc(&f->any, sizeof(uint32_t) * (size_t)f->sms * kPerQuarter * kTM) != cudaSuccess ||
       cudaMalloc(&f->err, sizeof(int)) != cudaSuccess || cudaMemset(f->err, 0, sizeof(int)) != cudaSuccess)
     goto bad;
   for (const void *k : {(const void *)fp64_tc_gemm_kernel<8, 0>, (const void *)fp64_tc_gemm_kernel<8, 1>,
@@ -903,7 +1105,6 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
   X.rows = (int)rows;
   const int nt = segs == 1 ? tile_columns(2 * cols) : tile_columns(2 * cols, (int)((rows + kTM - 1) / kTM), f->sms);
   // panels of whole tiles
-  constexpr int kDig = digits_of(false);
   const size_t a_tile = (size_t)KB * kDig * kADig, b_tile = (size_t)KB * kDig * nt * 32;
   const int all_m = (int)((rows + kTM - 1) / kTM), all_n = (2 * cols + nt - 1) / nt;
   const int pm = (int)std::min<size_t>(all_m, f->a_bytes / a_tile), pn = (int)std::min<size_t>(all_n, f->b_bytes / b_tile);
@@ -913,10 +1114,10 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
     const bool kept = pn >= all_n && yK == g.K && ycols == cols && f->ynt == nt;
     for (int m0 = 0; m0 < all_m; m0 += pm) {
       const int r0 = m0 * kTM, nr = (int)std::min<long long>(rows - r0, (long long)std::min(pm, all_m - m0) * kTM);
-      cut<kRows, kReal>(L, cut_job(X, r0, (n0 == 0 || pm < all_m) ? nr : 0, kTM, f->ex, f->A),
-                        cut_job(Y, y0, (m0 == 0 && !kept) ? ny : 0, nt, f->ey, f->B), 0, g.K, Kp, KB, seg_k(kRows));
+      cut<kRows, kReal>(L, cut_job(X, r0, (n0 == 0 || pm < all_m) ? nr : 0, kTM, f->ex, f->A, f->MA),
+                        cut_job(Y, y0, (m0 == 0 && !kept) ? ny : 0, nt, f->ey, f->B, f->MB), 0, g.K, Kp, KB, seg_k(kRows));
       TcGemm t{};
-      t.A = f->A; t.B = f->B; t.KB = KB; t.segs = segs; t.kseg = kSeg; t.nt = nt;
+      t.A = f->A; t.B = f->B; t.MA = f->MA; t.MB = f->MB; t.KB = KB; t.segs = segs; t.kseg = kSeg; t.nt = nt;
       t.mtiles = (nr + kTM - 1) / kTM; t.ntiles = (2 * ny + nt - 1) / nt;
       t.splits = 1; t.segs_per_split = segs; t.err = f->err; t.sums = f->sums; t.part = f->part;
       t.X = X; t.Y = Y; t.ex = f->ex; t.ey = f->ey; t.exs = nr; t.eys = ny;
@@ -952,21 +1153,20 @@ bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g) {
   const int mtiles = (2 * g.M + kTM - 1) / kTM, ntiles = (2 * g.N + nt - 1) / nt;
   const int splits_max = f->sms / (mtiles * ntiles);   // one unit per CTA
   if (splits_max < 1) return false;
-  constexpr int kDig = digits_of(true);
   // segments of 256 terms, or 128 where those leave half of the SMs idle (nb <= 26: 34 -> 24 us at nb = 24)
   const int kseg = 2 * ((K + kSeg * kKB - 1) / (kSeg * kKB)) * mtiles * ntiles <= f->sms ? kSeg / 2 : kSeg;
   const size_t a_seg = (size_t)mtiles * kseg * kDig * kADig, b_seg = (size_t)ntiles * kseg * kDig * nt * 32;   // bytes per segment
   const int all_segs = (K + kseg * kKB - 1) / (kseg * kKB);
   int ps = (int)std::min<size_t>(all_segs, std::min(f->a_bytes / a_seg, f->b_bytes / b_seg));
   ps = (int)std::min<long long>(ps, f->exps / std::max(g.M, g.N));
-  if (ps < 1) return false;
+  if (ps < 1 || (long long)all_segs * mtiles * ntiles * kPerQuarter * kTM > f->flag_words) return false;
   TcGemm t{};
   for (int sg0 = 0; sg0 < all_segs; sg0 += ps) {
     const int ns = std::min(ps, all_segs - sg0), k0 = sg0 * kseg * kKB, Klen = std::min(K - k0, ns * kseg * kKB);
     const int Kp = round_up(Klen, kKB), KB = Kp / kKB;
-    cut<kPlanes, kPlanes>(L, cut_job(X, 0, g.M, kTM, f->ex, f->A), cut_job(Y, 0, g.N, nt, f->ey, f->B), k0, Klen, Kp, KB,
+    cut<kPlanes, kPlanes>(L, cut_job(X, 0, g.M, kTM, f->ex, f->A, f->MA), cut_job(Y, 0, g.N, nt, f->ey, f->B, f->MB), k0, Klen, Kp, KB,
                            kseg * kKB);
-    t.A = f->A; t.B = f->B; t.KB = KB; t.segs = ns; t.kseg = kseg; t.nt = nt; t.mtiles = mtiles; t.ntiles = ntiles;
+    t.A = f->A; t.B = f->B; t.MA = f->MA; t.MB = f->MB; t.KB = KB; t.segs = ns; t.kseg = kseg; t.nt = nt; t.mtiles = mtiles; t.ntiles = ntiles;
     // the first panel is the longest: its split count holds for the later ones
     if (sg0 == 0) {
       t.segs_per_split = (ns + splits_max - 1) / splits_max;
@@ -978,10 +1178,11 @@ bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g) {
     t.k_begin = k0;
     t.C = g.C; t.scx = g.sc_m; t.scy = g.sc_n; t.unit_alpha = alpha; t.beta = g.beta != 0.0;
     t.sums = f->sums; t.part = f->part; t.accumulate = sg0 > 0;
+    t.flags = f->flags; t.any = f->any; t.all_segs = all_segs; t.seg_begin = sg0;
     launch_gemm<2>(L, t, t.splits * mtiles * ntiles, "fp64_tc_gemm_long");
   }
   L.before("fp64_tc_reduce");
-  launch_dependent(fp64_tc_reduce_kernel, (g.M * g.N + 7) / 8, 256, 0, L.stream, t);
+  launch_dependent(fp64_tc_reduce_kernel, g.M * g.N, kRedThreads, 0, L.stream, t);
   L.after_launch();
   return true;
 }
