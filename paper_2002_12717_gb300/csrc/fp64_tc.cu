@@ -619,6 +619,7 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const __grid_
           }
         }
       }
+      wait_loads(full, kStages, s, ph);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -668,7 +669,7 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const __grid_
         }
       }
       mma_commit(fin);
-      mbar_wait(fin, 0, p.err);
+      mbar_wait_own(fin, 0);
     }
   } else {
     const int quarter = warp & 3, cg = (warp - 2) >> 2;

@@ -122,6 +122,7 @@ __global__ void __launch_bounds__(kTsThreads, 1)
           if (++f == nf) { f = 0; ph ^= 1u; }
         }
       }
+      wait_loads(ffull, nf, f, ph);
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------ B producer (slices of w)
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(kTsThreads, 1)
           if (++s == nbs) { s = 0; ph ^= 1u; }
         }
       }
+      wait_loads(bfull, nbs, s, ph);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -198,7 +200,7 @@ __global__ void __launch_bounds__(kTsThreads, 1)
       }
       // every MMA issued by this thread has completed before TMEM is released
       mma_commit(fin);
-      mbar_wait(fin, 0, p.err);
+      mbar_wait_own(fin, 0);
     }
   } else if (warp < kTsEpiWarp0) {
     // ------------------------------------------------------------ converters

@@ -480,6 +480,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           if (++s == (kSliced ? nf : stages)) { s = 0; ph ^= 1u; }
         }
       }
+      wait_loads(kSliced ? ffull : full, kSliced ? nf : stages, s, ph);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -556,7 +557,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       }
       // every MMA issued by this thread has completed before TMEM is released
       mma_commit(fin);
-      mbar_wait(fin, 0, p.err);
+      mbar_wait_own(fin, 0);
     }
   } else if (warp < kEpiWarp0) {
     // ------------------------------------------------------------ converters
@@ -587,7 +588,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             mbar_arrive_expect_tx(&full[s], kSlices * b_bytes);
             tma_load_3d(stg + (size_t)s * stage_bytes + kSlicedBOff, &tmBhi, &full[s], bk, brow, 0);
           }
-          if (!mbar_wait(&ffull[f], fph, p.err)) { ok = false; break; }
+          if (!mbar_wait(&ffull[f], fph, p.err)) {
+            if (ct == 0) mbar_wait_own(&full[s], ph);   // the B load just started
+            ok = false;
+            break;
+          }
           a = reinterpret_cast<float4 *>(fring + (size_t)f * kABytes);
         } else {
           if (!mbar_wait(&full[s], ph, p.err)) { ok = false; break; }
@@ -636,6 +641,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         }
       }
     }
+    if (kSliced && ct == 0) wait_loads(full, stages, s, ph);
   } else {
     // ------------------------------------------------------------ epilogue
     const int r = threadIdx.x - 32 * kEpiWarp0;       // TMEM lane == tile row

@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(kTsThreads, 1)
           if (++f == nf) { f = 0; ph ^= 1u; }
         }
       }
+      wait_loads(ffull, nf, f, ph);
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------ B producer (slices)
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(kTsThreads, 1)
           if (++s == kTsBStages) { s = 0; ph ^= 1u; }
         }
       }
+      wait_loads(bfull, kTsBStages, s, ph);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -199,7 +201,7 @@ __global__ void __launch_bounds__(kTsThreads, 1)
       }
       // every MMA issued by this thread has completed before TMEM is released
       mma_commit(fin);
-      mbar_wait(fin, 0, p.err);
+      mbar_wait_own(fin, 0);
     }
   } else if (warp < kTsEpiWarp0) {
     // ------------------------------------------------------------ converters

@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(kPiThreads, 1)
           if (++s == kPiStages) { s = 0; ph ^= 1u; }
         }
       }
+      wait_loads(full, kPiStages, s, ph);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -142,7 +143,7 @@ __global__ void __launch_bounds__(kPiThreads, 1)
       }
       // every MMA issued by this thread has completed before TMEM is released
       mma_commit(fin);
-      mbar_wait(fin, 0, p.err);
+      mbar_wait_own(fin, 0);
     }
   } else {
     // ------------------------------------------------------------ epilogue (warps 2-5)

@@ -78,6 +78,19 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int *e
   }
 }
 
+// The same wait, bounded alike, that goes on when another role has given up: before a CTA leaves, its own loads have landed in
+// shared memory and its own MMAs are done with TMEM.
+__device__ __forceinline__ void mbar_wait_own(uint64_t *bar, uint32_t parity, unsigned long long limit_ns = kWaitLimitNs) {
+  const unsigned long long t0 = globaltimer();
+  while (!mbar_try_wait(bar, parity))
+    if (globaltimer() - t0 > limit_ns) return;
+}
+// Every load of a ring of stages (one per stage and phase, next: the stage and phase of the load that would come now); a
+// stage that was never loaded has its phase before the first one behind it.
+__device__ __forceinline__ void wait_loads(uint64_t *full, int stages, int next, uint32_t phase) {
+  for (int s = 0; s < stages; ++s) mbar_wait_own(&full[s], s < next ? phase : phase ^ 1u);
+}
+
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y, int z) {
   asm volatile(
