@@ -31,6 +31,15 @@
  * Errors: every int-returning call returns G1G2_OK (0) or a negative code;
  * nothing aborts or throws across the ABI.  g1g2_strerror gives the message,
  * g1g2_last_error_detail the detail of the last failure on this thread.
+ *
+ * Kernels on the tensor cores (both precisions that use them and larger FP64
+ * products) bound their waits and return when one gives up, with incomplete
+ * results.  The calls that synchronise (observables, propagate, propagate_hfgkba,
+ * adjoint, get_state) report it as G1G2_ETIMEOUT, once; results since the last
+ * such call that returned G1G2_OK are then invalid, and set_state starts afresh.
+ * g1g2_rhs, g1g2_rhs_vjp and g1g2_step only queue work: a caller with an
+ * integrator of its own checks with g1g2_get_state(c, NULL, NULL, NULL) before it
+ * uses what they wrote.
  */
 #ifndef G1G2_H
 #define G1G2_H
@@ -311,7 +320,14 @@ int g1g2_hubbard_path(const g1g2_ctx *c);
  * stream of the current device. */
 int g1g2_wait_selftest(int limit_us);
 
-/* Copy the state to / from host memory (G2 may be NULL on get; NULL on set means 0). */
+/* For tests of a caller's error handling: sets the context's error word as a
+ * kernel whose wait gave up does, so that the next synchronising call returns
+ * G1G2_ETIMEOUT.  G1G2_EUNSUPPORTED for a context without tensor-core kernels. */
+int g1g2_wait_inject(g1g2_ctx *c);
+
+/* Copy the state to / from host memory (any pointer may be NULL on get; G2 NULL on set means 0).
+ * g1g2_get_state waits for everything queued and reports a kernel that gave up
+ * (G1G2_ETIMEOUT). */
 int g1g2_get_state(g1g2_ctx *c, double *t, double *G1, double *G2);
 int g1g2_set_state(g1g2_ctx *c, double t, const double *G1, const double *G2);
 

@@ -1068,6 +1068,8 @@ bad:
   return nullptr;
 }
 
+void fp64_tc_inject_error(Fp64Tc *f, cudaStream_t stream) { cudaMemsetAsync(f->err, 1, sizeof(int), stream); }
+
 int fp64_tc_error(Fp64Tc *f, cudaStream_t stream) {
   int e = 0;
   if (cudaMemcpyAsync(&e, f->err, sizeof(int), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||

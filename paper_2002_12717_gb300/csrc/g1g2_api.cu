@@ -1586,7 +1586,8 @@ int g1g2_get_state(g1g2_ctx *c, double *t, double *G1, double *G2) {
     return rc;
   if (G2 && (rc = cuda_check(cudaMemcpyAsync(G2, c->G, N4 * sizeof(cplx), cudaMemcpyDeviceToHost, c->stream), "get")))
     return rc;
-  return cuda_check(cudaStreamSynchronize(c->stream), "get sync");
+  if ((rc = cuda_check(cudaStreamSynchronize(c->stream), "get sync"))) return rc;
+  return wait_error(c);
 }
 
 int g1g2_rhs_vjp(g1g2_ctx *c, double t, const double *n_dev, const double *G2_dev, const double *dn_bar,
@@ -1674,6 +1675,14 @@ int g1g2_fp64_rate(double *tflops) {
 int g1g2_wait_selftest(int limit_us) {
   if (limit_us < 1 || limit_us > 10000000) return fail(G1G2_EINVAL, "limit must be 1 us .. 10 s");
   return tc_wait_selftest(1000ull * (unsigned long long)limit_us, nullptr);
+}
+
+int g1g2_wait_inject(g1g2_ctx *c) {
+  if (!c) return fail(G1G2_EINVAL, "ctx is NULL");
+  if (!c->tc && !c->ftc) return fail(G1G2_EUNSUPPORTED, "this context has no kernels with bounded waits");
+  if (c->tc) tc_inject_error(c->tc, c->stream);
+  if (c->ftc) fp64_tc_inject_error(c->ftc, c->stream);
+  return cuda_check(cudaStreamSynchronize(c->stream), "inject sync");
 }
 
 int g1g2_set_adjoint_checkpoints(g1g2_ctx *c, int where) {

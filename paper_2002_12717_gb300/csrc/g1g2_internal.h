@@ -120,6 +120,8 @@ int fp64_tc_min_nb(bool pair_products);   // smallest basis size with a product 
 void fp64_tc_destroy(Fp64Tc *f);
 // G1G2_ETIMEOUT when one of the kernels gave up on a barrier (synchronises the stream).
 int fp64_tc_error(Fp64Tc *f, cudaStream_t stream);
+// Sets the error word as a kernel that gave up does.
+void fp64_tc_inject_error(Fp64Tc *f, cudaStream_t stream);
 
 // out(a0,a1,a2,a3) = beta*out + alpha*op(in(a_p0, a_p1, a_p2, a_p3)), op = conj if conj.
 void permute4(Launcher &L, int nb, const cplx *in, cplx *out, const int p[4], cplx alpha, double beta,

@@ -1376,11 +1376,14 @@ int tc_error(TcPath *p, cudaStream_t stream) {
   if (cudaMemcpyAsync(&e, p->err, sizeof(int), cudaMemcpyDeviceToHost, stream) != cudaSuccess) return G1G2_ECUDA;
   if (cudaStreamSynchronize(stream) != cudaSuccess) return G1G2_ECUDA;
   if (e) {
+    cudaMemsetAsync(p->err, 0, sizeof(int), stream);   // reported once: later calls run again
     set_error_detail("a tensor-core kernel gave up waiting on a barrier");
     return G1G2_ETIMEOUT;
   }
   return G1G2_OK;
 }
+
+void tc_inject_error(TcPath *p, cudaStream_t stream) { cudaMemsetAsync(p->err, 1, sizeof(int), stream); }
 
 void tc_load_state(TcPath *p, Launcher &L, const cplx *G) {
   int *slot = p->sliced ? p->amax + kAmaxY : nullptr;

@@ -76,6 +76,7 @@ def load():
         "g1g2_adjoint": (ctypes.c_int, [vp, ctypes.c_double, ctypes.c_int, ctypes.c_int, ctypes.c_int, _dp, _dp, _dp,
                                         _dp, _dp]),
         "g1g2_wait_selftest": (ctypes.c_int, [ctypes.c_int]),
+        "g1g2_wait_inject": (ctypes.c_int, [vp]),
         "g1g2_fp64_rate": (ctypes.c_int, [ctypes.POINTER(ctypes.c_double)]),
         "g1g2_g1_rhs_noalloc": (ctypes.c_int, [ctypes.c_int, ctypes.c_int] + [vp] * 6),
         "g1g2_set_hubbard_path": (ctypes.c_int, [vp, ctypes.c_int]),
@@ -237,7 +238,8 @@ class Propagator:
         _check(self._lib.g1g2_set_drive(self._ctx, _cptr(db), int(drive.kind), _cptr(params), len(params)))
 
     def rhs(self, t, n_dev, G2_dev, dn_dev, dG2_dev):
-        """dn/dt and dG2/dt at (t, n, G2) into caller-owned device tensors (complex128, contiguous)."""
+        """dn/dt and dG2/dt at (t, n, G2) into caller-owned device tensors (complex128, contiguous);
+        queued on the context's stream (see synchronize)."""
         for x in (n_dev, G2_dev, dn_dev, dG2_dev):
             if x is not None and not x.is_contiguous():
                 raise ValueError("device tensors must be contiguous")
@@ -284,6 +286,11 @@ class Propagator:
         g = np.zeros((self.nb,) * 4, dtype=np.complex128) if with_g2 else None
         _check(self._lib.g1g2_get_state(self._ctx, ctypes.byref(t), _cptr(n), None if g is None else _cptr(g)))
         return t.value, n, g
+
+    def synchronize(self):
+        """Wait for the queued work; raises G1G2Error (ETIMEOUT) when a kernel of it gave up on a wait and left
+        incomplete results.  rhs, rhs_vjp and step only queue: check before their results are used for good."""
+        _check(self._lib.g1g2_get_state(self._ctx, None, None, None))
 
     def set_state(self, t, n, G2=None):
         nb_ = _c128(n)
