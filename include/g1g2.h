@@ -150,7 +150,10 @@ void g1g2_default_options(g1g2_options *opt);
  * build does not run (see g1g2_selfenergy and g1g2_precision); G1G2_ESYMM
  * when a symmetry is violated beyond sym_tol; G1G2_ENONFINITE when h, w, G1_0 or G2_0 holds a NaN or an Inf
  * (checked on the host before any device work); G1G2_ENOMEM / G1G2_ECUDA on
- * device failure. t starts at 0. */
+ * device failure. t starts at 0.  An FP64 context also takes up to 2.6 GB for
+ * its larger products on the tensor cores, after all else; where they do not
+ * fit, these products run on the CUDA cores (as accurate, up to twenty times
+ * slower; g1g2_profile_report then lists fp64_zgemm in place of fp64_tc_gemm). */
 int g1g2_init(g1g2_ctx **out, int nb, const double *h, const double *w, const double *G1_0,
               const double *G2_0, int se, const g1g2_options *opt);
 

@@ -1000,7 +1000,8 @@ constexpr int kMinK = 8, kMinCols = 8;
 // at nb = 15 (45 at nb = 20), 48 us here at nb = 16 and 43 at nb = 24; nb^2 x nb^2 x nb^2 product 43 and 39 us at nb = 12 (3e6).
 constexpr double kMinWork = 2.2e6, kMinWorkLong = 4e6;
 
-int fp64_tc_min_nb(bool pair_products) { return pair_products ? 12 : 17; }
+// nb^5 products pass kMinWork from nb = 19 on; nb^4 products with the factors of a factorised interaction (nfac <= nb^2) may below
+int fp64_tc_min_nb(bool pair_products, bool factorised) { return pair_products ? 12 : factorised ? 17 : 19; }
 
 struct Fp64Tc {
   uint8_t *A = nullptr, *B = nullptr;   // digit blocks of the two operands

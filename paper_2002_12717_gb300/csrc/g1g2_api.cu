@@ -135,6 +135,15 @@ int wait_error(g1g2_ctx *c) {
   return rc;
 }
 
+// Digit workspace of the FP64 products (up to 2.6 GB; without it they run on the CUDA cores).  Optional, so it is made after
+// everything that a call cannot do without, and not before a call that forms such products: a context on the Hubbard path
+// (or with the spin-restricted Hubbard GW) has none of them until its gradients, its memory integral or the general form.
+void digit_workspace(g1g2_ctx *c) {
+  if (c->ftc || c->prec != G1G2_FP64 || c->se == G1G2_HF || c->hub_gw) return;
+  const bool pair = c->se != G1G2_SOA;
+  if (c->nb >= fp64_tc_min_nb(pair, c->Lf != nullptr)) c->ftc = fp64_tc_create(c->nb, pair);
+}
+
 using zc = std::complex<double>;
 
 // NVTX range for the lifetime of the object: RK4 steps and stages, observables, the
@@ -1216,8 +1225,6 @@ int g1g2_init(g1g2_ctx **out, int nb, const double *h, const double *w, const do
       return bail(rc);
     c->splits = 4 * 152;
     if ((rc = dalloc(c, &c->partial, (size_t)c->splits * N2))) return bail(rc);
-    const bool pair_products = !restricted_gw && se != G1G2_SOA;
-    if (nb >= fp64_tc_min_nb(pair_products)) c->ftc = fp64_tc_create(nb, pair_products);
     if ((se == G1G2_GW && !restricted_gw) || se == G1G2_TPH || se == G1G2_DSL) {
       if ((rc = dalloc(c, &c->Hb, N4)) || (rc = dalloc(c, &c->Gp, N4)) || (rc = dalloc(c, &c->Hp, N4)) ||
           (rc = dalloc(c, &c->Pp, N4)))
@@ -1299,6 +1306,7 @@ int g1g2_init(g1g2_ctx **out, int nb, const double *h, const double *w, const do
     if ((rc = launch_status(L, "tensor-core state"))) return bail(rc);
   }
   if ((rc = cuda_check(cudaStreamSynchronize(c->stream), "init sync"))) return bail(rc);
+  if (!c->hub_on) digit_workspace(c);
   *out = c;
   return G1G2_OK;
 }
@@ -1404,6 +1412,7 @@ int g1g2_init_factorised(g1g2_ctx **out, int nb, const double *h, const double *
       *out = nullptr;
       return rc;
     }
+    if (!c->hub_on) digit_workspace(c);
   }
   release();
   return G1G2_OK;
@@ -1543,6 +1552,8 @@ int g1g2_propagate_hfgkba(g1g2_ctx *c, double dt, int nsteps, double *G1_history
       (rc = S.get(&np, N2)) || (rc = S.get(&up, N2)) || (rc = S.get(&dn1, N2)) || (rc = S.get(&dn2, N2)) || (rc = S.get(&du1, N2)) ||
       (rc = S.get(&du2, N2)))
     return rc;
+  digit_workspace(c);
+  L.ftc = c->ftc;
   std::vector<cplx> eye(N2, cplx{0.0, 0.0});
   for (int i = 0; i < nb; ++i) eye[(size_t)i * nb + i] = {1.0, 0.0};
   if ((rc = cuda_check(cudaMemcpyAsync(uh, eye.data(), N2 * sizeof(cplx), cudaMemcpyHostToDevice, c->stream), "u0")) ||
@@ -1607,6 +1618,7 @@ int g1g2_rhs_vjp(g1g2_ctx *c, double t, const double *n_dev, const double *G2_de
     }
     if (c->se == G1G2_HF) return fail(G1G2_EUNSUPPORTED, "call g1g2_adjoint once before the HF product");
   }
+  digit_workspace(c);
   Launcher L = c->launcher();
   vjp_fp64(c, L, t, reinterpret_cast<const cplx *>(n_dev), reinterpret_cast<const cplx *>(G2_dev),
            reinterpret_cast<const cplx *>(dn_bar), reinterpret_cast<const cplx *>(dG2_bar), reinterpret_cast<cplx *>(n_bar),
@@ -1660,6 +1672,7 @@ int g1g2_set_hubbard_path(g1g2_ctx *c, int enable) {
   if (enable && !c->hub_ok)
     return fail(G1G2_EUNSUPPORTED, "the O(nb^4) path needs spin-restricted SOA, the FP64 form and an on-site w");
   c->hub_on = enable != 0;
+  if (!enable) digit_workspace(c);
   return G1G2_OK;
 }
 
@@ -1788,6 +1801,8 @@ int g1g2_adjoint(g1g2_ctx *c, double dt, int nsteps, int ckpt_every, int objecti
     if ((rc = adj_alloc(c, c->adj_allocs, &p, N4 * sizeof(cplx)))) return done(rc);
     c->adj_wbar = (cplx *)p;
   }
+  digit_workspace(c);
+  L.ftc = c->ftc;
   if (grad_w) cudaMemsetAsync(c->adj_wbar, 0, N4 * sizeof(cplx), c->stream);
   double *dacc = (double *)acc;
   cudaMemsetAsync(dacc, 0, sizeof(double) * (1 + 4 * (size_t)nsteps), c->stream);

@@ -116,7 +116,8 @@ bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g);
 // Workspaces for one context of basis size nb (nullptr when they do not fit: the CUDA-core kernels then take
 // every product); pair_products: nb^2 x nb^2 x nb^2 products are among them.
 Fp64Tc *fp64_tc_create(int nb, bool pair_products);
-int fp64_tc_min_nb(bool pair_products);   // smallest basis size with a product that takes this path
+// smallest basis size with a product that takes this path (factorised: products with nfac factors among them)
+int fp64_tc_min_nb(bool pair_products, bool factorised);
 void fp64_tc_destroy(Fp64Tc *f);
 // G1G2_ETIMEOUT when one of the kernels gave up on a barrier (synchronises the stream).
 int fp64_tc_error(Fp64Tc *f, cudaStream_t stream);
