@@ -323,6 +323,14 @@ int g1g2_hubbard_path(const g1g2_ctx *c);
  * stream of the current device. */
 int g1g2_wait_selftest(int limit_us);
 
+/* Larger FP64 products run on the tensor cores from digits of their operands, of
+ * which at most bytes per operand (and never more than the context allocated, up
+ * to 1 GiB) are held at a time: beyond that a product runs in panels, and one that
+ * holds no tile of it runs on the CUDA cores.  Results agree to rounding.  For the
+ * tests of the panels, which otherwise begin at nb = 65.  G1G2_EUNSUPPORTED for a
+ * context without such products (nb < 12, other precisions, HF). */
+int g1g2_set_digit_panel(g1g2_ctx *c, size_t bytes);
+
 /* For tests of a caller's error handling: sets the context's error word as a
  * kernel whose wait gave up does, so that the next synchronising call returns
  * G1G2_ETIMEOUT.  G1G2_EUNSUPPORTED for a context without tensor-core kernels. */

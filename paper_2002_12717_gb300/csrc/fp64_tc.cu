@@ -1015,7 +1015,9 @@ struct Fp64Tc {
   long long flag_words = 0;
   int *err = nullptr;
   int sms = 0;
-  int yK = 0, ycols = 0, ynt = 0;       // shape of the column operand whose digits B holds whole (0: none)
+  size_t a_panel = 0, b_panel = 0;      // what a product uses of A and B (at most a_bytes and b_bytes)
+  int yK = 0, ycols = 0, ynt = 0;       // shape of the column operand whose digits B holds whole (0: none), and that operand
+  Operand y{};
 };
 
 void fp64_tc_destroy(Fp64Tc *f) {
@@ -1037,6 +1039,8 @@ Fp64Tc *fp64_tc_create(int nb, bool pair_products) {
   const size_t lng = blocks(2 * N, (N3 + 255) / 256 * 256);
   f->a_bytes = std::min(kPanelBytes, std::max({big, pair, lng}));
   f->b_bytes = std::min(kPanelBytes, std::max({blocks(2 * N, 2 * ((N + 7) / 8 * 8)), pair, lng}));
+  f->a_panel = f->a_bytes;
+  f->b_panel = f->b_bytes;
   f->exps = std::max({N3, N2 * ((N2 + 127) / 128), N * ((N3 + 127) / 128)});
   f->flag_words = (N3 + 127) / 128 * ((2 * N + kTM - 1) / kTM) * ((2 * N + kTNMax - 1) / kTNMax) * kPerQuarter * kTM;
   int dev = 0;
@@ -1069,6 +1073,11 @@ bad:
   return nullptr;
 }
 
+void fp64_tc_set_panel(Fp64Tc *f, size_t bytes) {
+  f->a_panel = std::min(f->a_bytes, bytes);
+  f->b_panel = std::min(f->b_bytes, bytes);
+}
+
 void fp64_tc_inject_error(Fp64Tc *f, cudaStream_t stream) { cudaMemsetAsync(f->err, 1, sizeof(int), stream); }
 
 int fp64_tc_error(Fp64Tc *f, cudaStream_t stream) {
@@ -1090,7 +1099,7 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
   Fp64Tc *f = L.ftc;
   if (!f) return false;
   // digits of the last product's column operand, when that product ran here and the caller says that it is the same
-  const int yK = g.same_small ? f->yK : 0, ycols = f->ycols;
+  const int yK = g.same_small ? f->yK : 0;
   f->yK = 0;
   const int alpha = unit_of(g.alpha);
   if (alpha < 0 || (g.beta != 0.0 && g.beta != 1.0)) return false;
@@ -1111,11 +1120,13 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
   // panels of whole tiles
   const size_t a_tile = (size_t)KB * kDig * kADig, b_tile = (size_t)KB * kDig * nt * 32;
   const int all_m = (int)((rows + kTM - 1) / kTM), all_n = (2 * cols + nt - 1) / nt;
-  const int pm = (int)std::min<size_t>(all_m, f->a_bytes / a_tile), pn = (int)std::min<size_t>(all_n, f->b_bytes / b_tile);
+  const int pm = (int)std::min<size_t>(all_m, f->a_panel / a_tile), pn = (int)std::min<size_t>(all_n, f->b_panel / b_tile);
   if (pm < 1 || pn < 1) return false;
   for (int n0 = 0; n0 < all_n; n0 += pn) {
     const int y0 = n0 * nt / 2, ny = std::min(cols - y0, std::min(pn, all_n - n0) * nt / 2);
-    const bool kept = pn >= all_n && yK == g.K && ycols == cols && f->ynt == nt;
+    // (the caller's word covers the contents; where and how they are read is looked at)
+    const bool kept = pn >= all_n && yK == g.K && f->ycols == cols && f->ynt == nt && f->y.p == Y.p && f->y.sx == Y.sx &&
+                      f->y.sk == Y.sk && f->y.conj == Y.conj;
     for (int m0 = 0; m0 < all_m; m0 += pm) {
       const int r0 = m0 * kTM, nr = (int)std::min<long long>(rows - r0, (long long)std::min(pm, all_m - m0) * kTM);
       cut<kRows, kReal>(L, cut_job(X, r0, (n0 == 0 || pm < all_m) ? nr : 0, kTM, f->ex, f->A, f->MA),
@@ -1137,6 +1148,7 @@ bool fp64_tc_zgemm(Launcher &L, const ZGemm &g) {
     f->yK = g.K;
     f->ycols = cols;
     f->ynt = nt;
+    f->y = Y;
   }
   return true;
 }
@@ -1161,7 +1173,7 @@ bool fp64_tc_zgemm_reduce(Launcher &L, const ZGemm &g) {
   const int kseg = 2 * ((K + kSeg * kKB - 1) / (kSeg * kKB)) * mtiles * ntiles <= f->sms ? kSeg / 2 : kSeg;
   const size_t a_seg = (size_t)mtiles * kseg * kDig * kADig, b_seg = (size_t)ntiles * kseg * kDig * nt * 32;   // bytes per segment
   const int all_segs = (K + kseg * kKB - 1) / (kseg * kKB);
-  int ps = (int)std::min<size_t>(all_segs, std::min(f->a_bytes / a_seg, f->b_bytes / b_seg));
+  int ps = (int)std::min<size_t>(all_segs, std::min(f->a_panel / a_seg, f->b_panel / b_seg));
   ps = (int)std::min<long long>(ps, f->exps / std::max(g.M, g.N));
   if (ps < 1 || (long long)all_segs * mtiles * ntiles * kPerQuarter * kTM > f->flag_words) return false;
   TcGemm t{};

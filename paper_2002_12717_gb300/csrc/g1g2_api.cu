@@ -1690,6 +1690,14 @@ int g1g2_wait_selftest(int limit_us) {
   return tc_wait_selftest(1000ull * (unsigned long long)limit_us, nullptr);
 }
 
+int g1g2_set_digit_panel(g1g2_ctx *c, size_t bytes) {
+  if (!c || bytes == 0) return fail(G1G2_EINVAL, "bad argument");
+  digit_workspace(c);
+  if (!c->ftc) return fail(G1G2_EUNSUPPORTED, "this context has no digit workspace");
+  fp64_tc_set_panel(c->ftc, bytes);
+  return G1G2_OK;
+}
+
 int g1g2_wait_inject(g1g2_ctx *c) {
   if (!c) return fail(G1G2_EINVAL, "ctx is NULL");
   if (!c->tc && !c->ftc) return fail(G1G2_EUNSUPPORTED, "this context has no kernels with bounded waits");

@@ -121,6 +121,8 @@ int fp64_tc_min_nb(bool pair_products, bool factorised);
 void fp64_tc_destroy(Fp64Tc *f);
 // G1G2_ETIMEOUT when one of the kernels gave up on a barrier (synchronises the stream).
 int fp64_tc_error(Fp64Tc *f, cudaStream_t stream);
+// Digits of at most bytes per operand at a time: larger products run in panels (one that does not hold a tile, on the CUDA cores).
+void fp64_tc_set_panel(Fp64Tc *f, size_t bytes);
 // Sets the error word as a kernel that gave up does.
 void fp64_tc_inject_error(Fp64Tc *f, cudaStream_t stream);
 

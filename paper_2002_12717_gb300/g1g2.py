@@ -77,6 +77,7 @@ def load():
                                         _dp, _dp]),
         "g1g2_wait_selftest": (ctypes.c_int, [ctypes.c_int]),
         "g1g2_wait_inject": (ctypes.c_int, [vp]),
+        "g1g2_set_digit_panel": (ctypes.c_int, [vp, ctypes.c_size_t]),
         "g1g2_fp64_rate": (ctypes.c_int, [ctypes.POINTER(ctypes.c_double)]),
         "g1g2_g1_rhs_noalloc": (ctypes.c_int, [ctypes.c_int, ctypes.c_int] + [vp] * 6),
         "g1g2_set_hubbard_path": (ctypes.c_int, [vp, ctypes.c_int]),

@@ -161,3 +161,29 @@ def test_coherent_digits(digits, lead):
     s = sum(F(float(p)) * F(float(q)) for p, q in zip(a, b))     # I = -i (i s) = s; dn = -2 s
     size = F(float(np.abs(a) @ np.abs(b)))
     assert np.all(dn == dn[0, 0]) and abs(F(float(dn[0, 0].real)) + 2 * s) <= F(512 * EPS) * 2 * size
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_long_contractions_with_conjugated_operands(kind):
+    """Vector-Jacobian product at n = 0, w = 0 and no cotangent of dn: hbar = i (Y1 + Y2 - Y3 - Y4), the contractions of Y
+    with conj(G2) over all indices but one; fewer than 512 roundings on the way of a term of each, four additions."""
+    from paper_2002_12717_gb300.g1g2 import Propagator
+    nb = 24
+    rng = np.random.default_rng(7)
+    h, y, g = graded(kind, nb, rng)
+    zero = np.zeros((nb, nb))
+    with Propagator(h, np.zeros((nb,) * 4), zero, None, "SOA", "fp64", sym_tol=-1.0) as p:
+        out = [torch.empty_like(dev(x)) for x in (zero, g, zero)]
+        p.rhs_vjp(0.0, dev(zero), dev(g), dev(zero), dev(y), *out)
+        torch.cuda.synchronize()
+    hbar = out[2].cpu().numpy()
+    flat = lambda x, m: np.moveaxis(x, m, 0).reshape(nb, -1)  # noqa: E731
+    for a, b in entries(hbar, hbar.shape, rng, 3):
+        re = im = F(0)
+        sr = si = 0.0
+        for u, v, sign in ((flat(y, 0)[a], flat(g, 0)[b], 1), (flat(y, 1)[a], flat(g, 1)[b], 1),
+                           (flat(y, 2)[b], flat(g, 2)[a], -1), (flat(y, 3)[b], flat(g, 3)[a], -1)):
+            r, m, x, z = exact_dot(u, v.conj())
+            re, im, sr, si = re + sign * r, im + sign * m, sr + x, si + z
+        assert abs(F(float(hbar[a, b].real)) + im) <= F(516 * EPS) * F(si)       # i (re + i im)
+        assert abs(F(float(hbar[a, b].imag)) - re) <= F(516 * EPS) * F(sr)
