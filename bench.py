@@ -323,11 +323,21 @@ def run_ours(args, rank, world, dist):
         roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "peak_source": f"{peak_kind} copy bandwidth, of {peak_kind}"}
     else:
+        # FP64 form: products on the tensor cores issue 36 digit products and one of magnitudes per real multiply-add,
+        # the small ones FP64 multiply-adds
         fl = sum(p["flops_per_step"] * args.steps for p in per.values())
-        zg = sum(v[1] for k, v in prof_all.items() if k.startswith(("fp64_zgemm", "fp64_tc")))
-        achieved = fl / (zg * 1e-3) / 1e12
-        roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": achieved / FP64_PEAK_TFLOPS, "peak_source": FP64_PEAK_NOTE + " (measured DFMA; products on the tensor cores exceed it)"}
+        tc = sum(v[1] for k, v in prof_all.items() if k.startswith("fp64_tc"))
+        zg = sum(v[1] for k, v in prof_all.items() if k.startswith("fp64_zgemm"))
+        achieved = fl / ((tc + zg) * 1e-3) / 1e12
+        if tc > zg:
+            peak = peaks["bf16_tflops_sustained"]
+            roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+                    "work": "algorithmic: 8 flop per complex MAC of every contraction",
+                    "issued_achieved": 37 * achieved, "issued_frac": 37 * achieved / peak, "issued_over_algorithmic": 37.0,
+                    "peak_source": f"{peak_kind} bf16 sustained (cuBLAS loop), of {peak_kind}"}
+        else:
+            roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
+                    "frac": achieved / FP64_PEAK_TFLOPS, "peak_source": FP64_PEAK_NOTE + " (measured DFMA)"}
         dom_tag = "fp64_tc_gemm and fp64_zgemm: every complex contraction"
     roof.update({"traffic": TRAFFIC.get((dom_tag, dom_wl)) if args.precision == "bf16x4" else None,
                  "tensor_pipe_active_pct": TENSOR_PIPE.get((dom_tag, dom_wl)) if args.precision == "bf16x4" else None,
@@ -528,11 +538,10 @@ def nt_scaling(nts, dt=0.02, L=8):
         rows.append(row)
     ntm = max(nts)
     points = ntm * (ntm - 1) + 4 * ntm                    # history points summed over all evaluations
-    rot = prof.get("hfgkba_mode_rotate", (0, 0.0))
-    flops = 4 * 8 * nb ** 5 * points                      # four mode products of nb^5 complex MACs each
+    hist = prof.get("hfgkba_trapezoid", (0, 0.0))          # adds the history up: nb^4 complex doubles per point
     summary = {"workload": f"hubbard-chain-restricted-nb{nb}", "dt": dt,
                "kernels_at_max_N_t": {k: {"launches": v[0], "ms": round(v[1], 3)} for k, v in prof.items()},
-               "mode_rotate_gflops": round(flops / (rot[1] * 1e-3) / 1e9, 1) if rot[1] else None}
+               "history_sum_gbs": round(16 * nb ** 4 * points / (hist[1] * 1e-3) / 1e9, 1) if hist[1] else None}
     if len(rows) >= 2:
         a, b = rows[-2], rows[-1]
         for key in ("hfgkba_s", "g1g2_general_s", "g1g2_hubbard_s"):

@@ -1,6 +1,7 @@
-// Plain FP64 kernels of libg1g2: the reference form of every contraction
-// (CUDA-core DFMA), the Hartree-Fock build, the G1 right-hand side, the G2
-// assembly with the fused RK4 update, and the FP64 observables.
+// Plain FP64 kernels of libg1g2: the contractions that are too small for the digit products of
+// fp64_tc.cu (CUDA-core DFMA), the Hartree-Fock build, the G1 right-hand side, the G2
+// assembly with the fused RK4 update, the Hubbard and memory-integral forms, the kernels of the adjoint, and the FP64
+// observables.
 #include "g1g2_internal.h"
 
 #include <algorithm>

@@ -908,13 +908,16 @@ __global__ void __launch_bounds__(kRedThreads) fp64_tc_reduce_kernel(const TcGem
       for (uint32_t m = re | im; m; m &= m - 1) {
         const int s = __ffs((int)m) - 1, k1 = min(p.X.K, (s0 + s + 1) * len);
         const bool r = re >> s & 1u, t = im >> s & 1u;
+        double xs = 0.0, ys = 0.0;   // by segment: fewer roundings in a row than in one sum over all
 #pragma unroll 8
         for (int k = (s0 + s) * len + lane; k < k1; k += 32) {
           const cplx u = a[k_offset(p.X, k)], v = b[k_offset(p.Y, k)];
           const double ui = flip(u.y, fx), vi = flip(v.y, fy);
-          if (r) { x = fma(u.x, v.x, x); y = fma(u.x, vi, y); }
-          if (t) { x = fma(-ui, vi, x); y = fma(ui, v.x, y); }
+          if (r) { xs = fma(u.x, v.x, xs); ys = fma(u.x, vi, ys); }
+          if (t) { xs = fma(-ui, vi, xs); ys = fma(ui, v.x, ys); }
         }
+        x += xs;
+        y += ys;
       }
     }
   }
