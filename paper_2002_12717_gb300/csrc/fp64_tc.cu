@@ -22,12 +22,14 @@
 // All this is relative to the largest entries, while FP64 multiply-adds err by parts of sum |a| |b|, which is far
 // smaller where entries of very different size meet: far from the diagonal of decaying matrices, beside one huge matrix
 // element, in the imaginary parts of nearly real data.  So one more MMA per K step sums the magnitudes, as BF16
-// numbers (magnitude()), and an element with 0 < sum |a| |b| < 2^e 2^e' max(sqrt(n), 4) / 64, n the smaller of the two rows'
-// numbers of nonzero terms, is taken from FP64 multiply-adds instead (plain_elements(), and the reduction of long
-// contractions).  At that line the digits err by at most n 2^-53 sum |a| |b|, the a-priori bound of n multiply-adds, and
-// typically by half of 2^-53 sum |a| |b|.  Dense seeded bases have 1e-5 or fewer such elements; sparse or decaying
-// operands as many as need them: the 4 x 4 cluster (noise of 1e-17 beside entries of 1) one in seven, for which its
-// gradients take 97 ms instead of 31 with none (160 with all products on the CUDA cores).
+// numbers (magnitude()), and an element with 0 < sum |a| |b| < 2^e 2^e' / 16 is taken from FP64 multiply-adds instead
+// (plain_elements(), and the reduction of long contractions).  From that line on the digits err by at most n 2^-53 sum |a| |b|
+// over the n <= 256 terms of the segment, the a-priori bound of n multiply-adds; at the line typically by 1.5 of 2^-53 sum |a| |b|
+// (multiply-adds: 0.3 for terms of mixed sign, 0.4 sqrt(n / 3) for one sign), above it by less in proportion.
+// Seeded bases have 1e-6 or fewer such elements, up to one in 200 in the source term at times when n is nearly 1/2 (GW, nb = 64:
+// mode products 370 us, 480 on average in such a step).  Sparse or decaying operands have as many as they need: the 4 x 4
+// cluster (noise of 1e-17 beside entries of 1) one in ten, for which its gradients take 95 ms instead of 31 with none (160 with
+// all products on the CUDA cores).
 //
 // Against an extended-precision reference the right-hand side of a seeded basis at nb = 24 errs by 2.6e-16 (GW) and 3.8e-16
 // (TPP, complex w) in the 2-norm; FP64 multiply-adds by 6.2e-16 and 9.3e-16, plain FP64 torch by 6.0e-16 and 9.0e-16.
@@ -50,7 +52,7 @@ using namespace tc;
 
 constexpr int kDig = 8;                    // digits per real operand
 constexpr int kOrd = 8;                    // orders of digit products
-// A row's exponent comes with the number of its terms that are not zero (of either part's, in long contractions)
+// A row's exponent comes with the number of its real terms that are not zero
 constexpr int kExpBits = 11, kExpMask = (1 << kExpBits) - 1;
 constexpr int kTM = 128;                   // rows of A per tile (TMEM lanes)
 constexpr int kTNMax = 128;                // real columns per tile, at most
@@ -336,11 +338,9 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
                : "memory");
 }
 
-// Whether s = sum |a| |b| over at most terms products, in units of the two rows' exponents, is too small for the digits
-// (0 < s < sqrt(terms) / 64, with at least 16 terms)
-__device__ __forceinline__ bool too_small(float s, int terms) {
-  return s > 0.f && s * s < (float)max(terms, 16) * (1.f / 4096.f);
-}
+// Whether s = sum |a| |b|, in units of the two rows' exponents, is too small for the digits: below it their error may pass
+// n 2^-53 s (see the head of the file)
+__device__ __forceinline__ bool too_small(float s) { return s > 0.f && s < 0.0625f; }
 
 // (hi 2^32 + lo) 2^e as FP64, rounded to nearest, without a branch, for |hi| < 2^62, |lo| < 2^62 and kMinE <= e <= kMaxE (no
 // subnormal or infinite result then).  Two forms, because either alone is bound by its own pipe:
@@ -404,12 +404,13 @@ __device__ __forceinline__ void plain_fma(cplx &s, const cplx &u, const cplx &v,
 }
 // One segment (k0..k1) of the elements that the digits do not give, by FP64 multiply-adds, into the slots of their high
 // sums: bit c = 4 i + j of a lane's mask is complex column y0 + 12 i + j of its row, xt the terms of that row that are not
-// zero, yt those of column c = lane.  Three ways, by the cycles that they keep the FP64 pipe busy (64 per warp and term, 160
-// for sums over the lanes), since such operands are mostly sparse and terms with a zero are left out (unless
-// there is an Inf or a NaN): a row at a time with the columns over the lanes, a column with the rows over the lanes, and
-// single elements with the terms over the lanes.
+// zero, yt those of column c = lane.  Three ways, by the cycles that they keep the FP64 pipe busy (64 per warp and term, 32 per
+// sum over two lanes): a row at a time with the columns over the lanes and a column with the rows over the lanes, which
+// leave terms with a zero out (such operands are mostly sparse; not with an Inf or a NaN among them), and a list of
+// elements, each over as many lanes as there are for it.  (One element of the list after another, its terms over the whole
+// warp, waited for memory: one in 400 elements took a product at nb = 64 from 371 to 920 us, now to 650.)
 __device__ __noinline__ void plain_elements(const TcGemm &p, uint32_t mask, bool finite, int xt, int yt, int row0, int y0, int k0,
-                                            int k1, long long *hi) {
+                                            int k1, uint16_t *list, long long *hi) {
   const int lane = threadIdx.x & 31, K = k1 - k0;
   const Operand &X = p.X, &Y = p.Y;
   const int fx = X.conj ? (int)0x80000000u : 0, fy = Y.conj ? (int)0x80000000u : 0;
@@ -419,11 +420,37 @@ __device__ __noinline__ void plain_elements(const TcGemm &p, uint32_t mask, bool
     __stcg(hi + (size_t)(2 * y + 1) * kTM + r, __double_as_longlong(s.y));
   };
   const uint32_t cols = __reduce_or_sync(0xffffffffu, mask);
+  const int total = __reduce_add_sync(0xffffffffu, __popc(mask));
   const int by_rows = __reduce_add_sync(0xffffffffu, mask ? min(K, xt) : 0);
   const int by_cols = __reduce_add_sync(0xffffffffu, cols >> lane & 1u ? min(K, yt) : 0);
-  const int single = (__reduce_add_sync(0xffffffffu, __popc(mask)) * (2 * K + 160)) >> 6;
+  int L = 1;                                                       // lanes per element of the list
+  while (L < 32 && 2 * L * total <= 32) L *= 2;
+  const int listed = (total * L + 31) / 32 * ((K + L - 1) / L + (31 - __clz(L)) / 2);
   __syncwarp();
-  if (by_rows < min(by_cols, single)) {
+  if (listed <= min(by_rows, by_cols)) {
+    int at = __popc(mask);
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2) {
+      const int v = __shfl_up_sync(0xffffffffu, at, o);
+      if (lane >= o) at += v;
+    }
+    at -= __popc(mask);
+    for (uint32_t b = mask; b; b &= b - 1) list[at++] = (uint16_t)(lane | (__ffs((int)b) - 1) << 5);
+    __syncwarp();
+#pragma unroll 1
+    for (int i = 0; i < total; i += 32 / L) {
+      const int e = i + lane / L, c = list[min(e, total - 1)], r = c & 31, y = 4 * kPerQuarter * (c >> 7) + ((c >> 5) & 3);
+      const cplx *a = row(row0 + r), *b = Y.p + row_offset(Y, p.y_begin + y0) + y * Y.sx;
+      cplx s = {0.0, 0.0};
+#pragma unroll 4
+      for (int k = k0 + lane % L; k < k1; k += L) plain_fma(s, a[k * X.sk], b[k * Y.sk], fx, fy);
+      for (int o = L / 2; o > 0; o /= 2) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+      }
+      if (lane % L == 0 && e < total) put(y, r, s);
+    }
+  } else if (by_rows < by_cols) {
     const int y = 4 * kPerQuarter * (lane >> 2) + (lane & 3);      // this lane's column
     const cplx *b = Y.p + row_offset(Y, p.y_begin + y0) + y * Y.sx;
     uint32_t rows = __ballot_sync(0xffffffffu, mask != 0);
@@ -452,44 +479,19 @@ __device__ __noinline__ void plain_elements(const TcGemm &p, uint32_t mask, bool
         s = {0.0, 0.0};
       }
     }
-    __syncwarp();
-    return;
-  }
+  } else {
+    const cplx *a = row(row0 + lane);
 #pragma unroll 1
-  for (int g = 0; g < kMaxGroups; ++g) {
-    uint32_t col[4];
-    int n = 0, nc = 0;
+    for (int g = 0; g < kMaxGroups; ++g) {
+      bool col[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      col[j] = __ballot_sync(0xffffffffu, mask >> (4 * g + j) & 1u);
-      n += __popc(col[j]);
-      nc += col[j] != 0;
-    }
-    if (n == 0) continue;
-    const int yg = 4 * kPerQuarter * g;
-    const cplx *b = Y.p + row_offset(Y, p.y_begin + y0 + yg);
-    if (n * (2 * K + 160) < 64 * K * nc) {
-#pragma unroll 1
-      for (int j = 0; j < 4; ++j)
-#pragma unroll 1
-        for (uint32_t c = col[j]; c; c &= c - 1) {
-          const int r = __ffs((int)c) - 1;
-          const cplx *a = row(row0 + r), *bj = b + j * Y.sx;
-          cplx s = {0.0, 0.0};
-#pragma unroll 4
-          for (int k = k0 + lane; k < k1; k += 32) plain_fma(s, a[k * X.sk], bj[k * Y.sk], fx, fy);
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
-            s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
-          }
-          if (lane == 0) put(yg + j, r, s);
-        }
-    } else {
+      for (int j = 0; j < 4; ++j) col[j] = cols >> (4 * g + j) & 1u;
+      if (!(cols >> (4 * g) & 15u)) continue;
+      const int yg = 4 * kPerQuarter * g;
+      const cplx *b = Y.p + row_offset(Y, p.y_begin + y0 + yg);
       const bool mine = mask >> (4 * g) & 15u;
-      const cplx *a = row(row0 + lane);
       cplx s[4] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
-      constexpr int kAhead = 4;                        // rows' terms loaded ahead
+      constexpr int kAhead = 4;                                    // rows' terms loaded ahead
 #pragma unroll 1
       for (int kb = k0; kb < k1; kb += kAhead) {
         cplx u[kAhead];
@@ -742,8 +744,7 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const __grid_
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const int yj = __shfl_sync(0xffffffffu, yr, gl + j);
-            const int terms = min(xr, yj) >> kExpBits;
-            const bool low = too_small(__uint_as_float(v[2 * j]), terms) || too_small(__uint_as_float(v[2 * j + 1]), terms);
+            const bool low = too_small(__uint_as_float(v[2 * j])) || too_small(__uint_as_float(v[2 * j + 1]));
             if ((low || max(ea, yj & kExpMask) == kNonFinite) && y_tile + 4 * g + j < p.cols) plain |= 1u << (gl + j);
           }
         }
@@ -758,7 +759,8 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const __grid_
         } else if (some) {
           const bool finite = !__any_sync(0xffffffffu, max(ea, eyl) == kNonFinite);
           const int k0 = seg * seg_k(kRows);
-          plain_elements(p, plain, finite, xr >> kExpBits, yr >> kExpBits, mt * kTM + 32 * quarter, y_tile + 4 * cg, k0, min(p.X.K, k0 + seg_k(kRows)),
+          plain_elements(p, plain, finite, xr >> kExpBits, yr >> kExpBits, mt * kTM + 32 * quarter, y_tile + 4 * cg, k0,
+                         min(p.X.K, k0 + seg_k(kRows)), reinterpret_cast<uint16_t *>(stg),
                          sums - lane + (size_t)(8 * cg) * kTM);
         }
         // those, or results that may leave the range of fixed_to_double_*
