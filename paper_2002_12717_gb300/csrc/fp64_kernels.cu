@@ -41,7 +41,7 @@ struct ZGemmDev {
 // kReduce: split blockIdx.y sums c = (b, k) of [blockIdx.y len, ...) into partial[blockIdx.y].
 constexpr int kZThreads = 64;   // small CTAs: a product at nb = 8 has 4096 outputs for 152 SMs
 template <bool kReduce>
-__global__ void __launch_bounds__(kZThreads) zgemm_kernel(const ZGemmDev g, long long len, cplx *__restrict__ partial) {
+__global__ void __launch_bounds__(kZThreads) zgemm_kernel(const ZGemmDev g, long long len, cplx *partial) {
   dependent_begin();
   const long long mn = (long long)g.M * g.N, total = kReduce ? mn : mn * g.batch;
   const int fa = g.conjA ? (int)0x80000000u : 0, fb = g.conjB ? (int)0x80000000u : 0;   // signs on the integer pipe
@@ -119,7 +119,7 @@ ZGemmDev to_dev(const ZGemm &g) {
 // ---------------------------------------------------------------------------
 constexpr int PT = 32;
 
-__global__ void permute4_kernel(int nb, const cplx *__restrict__ in, cplx *__restrict__ out, int p0, int p1,
+__global__ void permute4_kernel(int nb, const cplx *in, cplx *out, int p0, int p1,
                                 int p2, int p3, cplx alpha, double beta, int conj) {
   dependent_begin();
   // out axis 3 is innermost in memory; input innermost axis is out-axis p3.
@@ -189,9 +189,9 @@ __global__ void permute4_kernel(int nb, const cplx *__restrict__ in, cplx *__res
 // Hartree-Fock build: one warp per (i, j).
 // ---------------------------------------------------------------------------
 template <bool REAL>
-__global__ void hf_build_kernel(int nb, const void *__restrict__ Wm_, const cplx *__restrict__ h,
-                                const cplx *__restrict__ D, double f, const cplx *__restrict__ n,
-                                cplx *__restrict__ hhf) {
+__global__ void hf_build_kernel(int nb, const void *Wm_, const cplx *h,
+                                const cplx *D, double f, const cplx *n,
+                                cplx *hhf) {
   dependent_begin();
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -403,8 +403,8 @@ __device__ __forceinline__ void rk4_apply(long long e, cplx k, int stage, double
 // dn/dt = -i [hHF, n] - (I + I^dag) (Eqs. eom_gone-2, eom_gone-I) and its RK4 stage update:
 // one warp per element (i, j), the lanes splitting the sum over p and reducing in a fixed
 // order, so that the nb^3 FP64 multiply-adds spread over every SM.
-__global__ void __launch_bounds__(256) g1_update_kernel(int nb, const cplx *__restrict__ hhf,
-                                                        const cplx *__restrict__ n, const cplx *__restrict__ I,
+__global__ void __launch_bounds__(256) g1_update_kernel(int nb, const cplx *hhf,
+                                                        const cplx *n, const cplx *I,
                                                         int stage, double dt, cplx *y, cplx *ys, cplx *acc,
                                                         cplx *kout) {
   dependent_begin();
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(256) g1_update_kernel(int nb, const cplx *__re
 }
 
 // dG = -i (Cb - Ab + conj(Ab^T)): 32x32 tiles of the (ij),(kl) matrix view.
-__global__ void g2_assemble_kernel(int nb, const cplx *__restrict__ Cb, const cplx *__restrict__ Ab, int stage,
+__global__ void g2_assemble_kernel(int nb, const cplx *Cb, const cplx *Ab, int stage,
                                    double dt, cplx *y, cplx *ys, cplx *acc, cplx *kout) {
   dependent_begin();
   __shared__ cplx tile[PT][PT + 1];
@@ -882,8 +882,8 @@ void count_nonfinite(Launcher &L, const cplx *x, long long len, double *cnt) {
 namespace g1g2 {
 namespace {
 
-__global__ void zaxpby_kernel(long long n, cplx alpha, const cplx *__restrict__ x, cplx beta,
-                              const cplx *__restrict__ y, cplx *out) {
+__global__ void zaxpby_kernel(long long n, cplx alpha, const cplx *x, cplx beta,
+                              const cplx *y, cplx *out) {
   dependent_begin();
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     cplx r = cmul(alpha, x[e]);
@@ -894,8 +894,8 @@ __global__ void zaxpby_kernel(long long n, cplx alpha, const cplx *__restrict__ 
 
 // out = i (A B - B A): one warp per element, so that the nb^3 FP64 multiply-adds spread over every SM (as products of
 // one 32 x 32 tile each they took 79 us at nb = 32)
-__global__ void __launch_bounds__(256) commutator_kernel(int nb, const cplx *__restrict__ A, const cplx *__restrict__ B,
-                                                         cplx *__restrict__ out) {
+__global__ void __launch_bounds__(256) commutator_kernel(int nb, const cplx *A, const cplx *B,
+                                                         cplx *out) {
   dependent_begin();
   const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -915,7 +915,7 @@ __global__ void __launch_bounds__(256) commutator_kernel(int nb, const cplx *__r
 }
 
 // out = c * (a + a^dag) for an nb x nb matrix
-__global__ void herm_sum_kernel(int nb, cplx c, const cplx *__restrict__ a, cplx *out) {
+__global__ void herm_sum_kernel(int nb, cplx c, const cplx *a, cplx *out) {
   dependent_begin();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nb * nb) return;
@@ -924,7 +924,7 @@ __global__ void herm_sum_kernel(int nb, cplx c, const cplx *__restrict__ a, cplx
 }
 
 // out = c * (Y + Y^dag), (Y^dag)_ijkl = conj(Y_klij), 32x32 tiles of the (ij),(kl) view
-__global__ void tconj_add_kernel(int nb, cplx c, const cplx *__restrict__ Y, cplx *out) {
+__global__ void tconj_add_kernel(int nb, cplx c, const cplx *Y, cplx *out) {
   dependent_begin();
   __shared__ cplx tile[PT][PT + 1];
   const long long M = (long long)nb * nb;
@@ -944,7 +944,7 @@ __global__ void tconj_add_kernel(int nb, cplx c, const cplx *__restrict__ Y, cpl
 }
 
 // partial sums of Re sum conj(x) y
-__global__ void real_dot_kernel(long long n, const cplx *__restrict__ x, const cplx *__restrict__ y, double *partials) {
+__global__ void real_dot_kernel(long long n, const cplx *x, const cplx *y, double *partials) {
   dependent_begin();
   __shared__ double s[256];
   double a = 0.0;
@@ -980,8 +980,8 @@ __global__ void dot_accumulate_kernel(int nparts, const double *partials, double
 // (nb = 32: 190 us, now 20 us).
 constexpr int kHtCols = 8, kHtRows = 32;
 template <bool REAL>
-__global__ void __launch_bounds__(kHtCols * kHtRows) hf_build_t_kernel(int nb, const void *__restrict__ Wm_,
-                                                                       const cplx *__restrict__ x, cplx *out,
+__global__ void __launch_bounds__(kHtCols * kHtRows) hf_build_t_kernel(int nb, const void *Wm_,
+                                                                       const cplx *x, cplx *out,
                                                                        int accumulate) {
   dependent_begin();
   __shared__ cplx part[kHtRows][kHtCols];
@@ -1115,9 +1115,9 @@ namespace {
 // four-index transformations of the memory integral are two such launches each.  M is built from S:
 // S itself, S^dag, 1 + eta S, S^T or S^*.  from_a: X = i (A - A^dag) of the tensor A = in (second = 1), the
 // source -i Psi formed on the fly.  At these sizes a launch is latency and one pass through the FP64 pipe.
-__global__ void __launch_bounds__(256) pair_rotate_kernel(int nb, int second, int from_a, const cplx *__restrict__ in,
-                                                          const cplx *__restrict__ S, int form, double eta,
-                                                          cplx *__restrict__ out) {
+__global__ void __launch_bounds__(256) pair_rotate_kernel(int nb, int second, int from_a, const cplx *in,
+                                                          const cplx *S, int form, double eta,
+                                                          cplx *out) {
   dependent_begin();
   __shared__ cplx X[kPairMaxNb * kPairMaxNb], T[kPairMaxNb * kPairMaxNb], M[kPairMaxNb * kPairMaxNb];
   const int n2 = nb * nb, c = blockIdx.x;
@@ -1154,7 +1154,7 @@ __global__ void __launch_bounds__(256) pair_rotate_kernel(int nb, int second, in
 // out[e] = dt (sum_b x[b len + e] - (x[e] + x[(nbatch - 1) len + e]) / 2), the trapezoid rule over a history of
 // nbatch >= 2 points: 32 consecutive entries per block, the points split over the block's eight warps, then a
 // fixed-order reduction over the warps in shared memory (deterministic).
-__global__ void __launch_bounds__(256) trapezoid_sum_kernel(long long len, int nbatch, const cplx *__restrict__ x,
+__global__ void __launch_bounds__(256) trapezoid_sum_kernel(long long len, int nbatch, const cplx *x,
                                                             double dt, cplx *out) {
   dependent_begin();
   __shared__ cplx part[8][32];
@@ -1182,10 +1182,10 @@ __global__ void __launch_bounds__(256) trapezoid_sum_kernel(long long len, int n
 // h^HF_ij = h_ij + sum_c Wm[(ij)][c] n_c and I_ij = -i sum_(lp),k wP[(lp)][i][k] G[(lp)][j][k], one CTA per (i, j):
 // for small nb, where one launch with nb^3 terms per CTA costs less than the split-K product, its
 // reduction and the Hartree-Fock build.
-__global__ void __launch_bounds__(128) mean_collision_kernel(int nb, const void *__restrict__ Wm, int wm_real,
-                                                             const cplx *__restrict__ h, const cplx *__restrict__ n,
-                                                             const cplx *__restrict__ wP, const cplx *__restrict__ G,
-                                                             cplx *__restrict__ hhf, cplx *__restrict__ I) {
+__global__ void __launch_bounds__(128) mean_collision_kernel(int nb, const void *Wm, int wm_real,
+                                                             const cplx *h, const cplx *n,
+                                                             const cplx *wP, const cplx *G,
+                                                             cplx *hhf, cplx *I) {
   dependent_begin();
   __shared__ cplx part[2][4];
   const int i = blockIdx.x / nb, j = blockIdx.x - i * nb, n2 = nb * nb, n3 = n2 * nb;
@@ -1227,8 +1227,8 @@ __global__ void __launch_bounds__(128) mean_collision_kernel(int nb, const void 
 
 // One half of a Heun step for n and u, one warp per element: dn = -i [h^HF, n] - (I + I^dag), du = -i h^HF u at
 // (n, u), then out = base + c1 prev + c2 derivative (prev null in the predictor), the derivative kept in (dn, du).
-__global__ void __launch_bounds__(256) heun_update_kernel(int nb, const cplx *__restrict__ hhf, const cplx *__restrict__ n,
-                                                          const cplx *__restrict__ u, const cplx *__restrict__ I,
+__global__ void __launch_bounds__(256) heun_update_kernel(int nb, const cplx *hhf, const cplx *n,
+                                                          const cplx *u, const cplx *I,
                                                           const cplx *n0, const cplx *u0, const cplx *dn_prev,
                                                           const cplx *du_prev, double c1, double c2, cplx *dn, cplx *du,
                                                           cplx *n_out, cplx *u_out) {

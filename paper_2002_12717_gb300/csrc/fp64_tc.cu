@@ -197,7 +197,7 @@ __device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_b
   constexpr int kLoads = 4;
   const int total = SR * kt;
   const unsigned inv = ((1u << 22) + kt - 1) / kt;        // idx / kt = idx inv >> 22 for idx kt < 2^22
-  const double2 *__restrict__ p = A.p;
+  const cplx *p = A.p;
   for (int i0 = tid; i0 < total; i0 += 256 * kLoads) {
     cplx v[kLoads];
     int at[kLoads];
@@ -209,7 +209,7 @@ __device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_b
       else { k = idx / SR; r = idx % SR; }
       at[i] = r * pitch + k;
       v[i] = {0.0, 0.0};
-      if (idx < total && koff[k] >= 0) v[i] = __ldg(p + roff[r] + koff[k]);
+      if (idx < total && koff[k] >= 0) v[i] = p[roff[r] + koff[k]];
     }
 #pragma unroll
     for (int i = 0; i < kLoads; ++i) {
@@ -229,7 +229,7 @@ __device__ __forceinline__ void cut_digits(const CutJob &job, int block, int k_b
       const int hx = __double2hiint(x) & 0x7fffffff, hy = __double2hiint(y) & 0x7fffffff;
       const int nx = (hx | __double2loint(x)) != 0, ny = (hy | __double2loint(y)) != 0;
       e = max(e, max(hx, hy));
-      terms += FORM == kPlanes ? nx | ny : nx + ny;
+      terms += nx + ny;
     }
 #pragma unroll
     for (int o = T / 2; o > 0; o >>= 1) {

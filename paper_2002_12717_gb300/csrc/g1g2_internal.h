@@ -67,7 +67,8 @@ struct Launcher {
 // finished and then lets the next one start, so that at most two are on the chip.  At nb <= 32 the kernels of a right-hand
 // side last 8 to 30 us each, of which the launch and the set-up hidden this way are about two.  (With the next one let in
 // before the wait, three were in flight and took room from the first: gradients at nb = 24 1203 us instead of 1139, memory
-// integral at nb = 8 8.70 ms instead of 8.35.)
+// integral at nb = 8 8.70 ms instead of 8.35.)  The previous kernel may still write what this one reads when this one starts,
+// so its inputs are not read-only for its lifetime: no __ldg and no const __restrict__ on them (the read-only path).
 template <class... KArgs, class... Args>
 inline void launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                              Args... args) {
