@@ -27,8 +27,8 @@
 // over the n <= 256 terms of the segment, the a-priori bound of n multiply-adds; at the line typically by 1.5 of 2^-53 sum |a| |b|
 // (multiply-adds: 0.3 for terms of mixed sign, 0.4 sqrt(n / 3) for one sign), above it by less in proportion.
 // Seeded bases have 1e-6 or fewer such elements, up to one in 200 in the source term at times when n is nearly 1/2 (GW, nb = 64:
-// mode products 370 us, 480 on average in such a step).  Sparse or decaying operands have as many as they need: the 4 x 4
-// cluster (noise of 1e-17 beside entries of 1) one in ten, for which its gradients take 95 ms instead of 31 with none (160 with
+// mode products 370 us, 470 on average in such a step).  Sparse or decaying operands have as many as they need: the 4 x 4
+// cluster (noise of 1e-17 beside entries of 1) one in ten, for which its gradients take 68 ms instead of 31 with none (160 with
 // all products on the CUDA cores).
 //
 // Against an extended-precision reference the right-hand side of a seeded basis at nb = 24 errs by 2.6e-16 (GW) and 3.8e-16
@@ -394,6 +394,9 @@ __device__ __forceinline__ cplx mul_unit(cplx z, int u) {
 __device__ __forceinline__ bool is_zero(const cplx &v) {   // on the integer pipe
   return (((__double2hiint(v.x) | __double2hiint(v.y)) & 0x7fffffff) | __double2loint(v.x) | __double2loint(v.y)) == 0;
 }
+__device__ __forceinline__ bool is_finite(const cplx &v) {
+  return max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff) < 0x7ff00000;
+}
 __device__ __forceinline__ double flip(double v, int sign) {
   return __hiloint2double(__double2hiint(v) ^ sign, __double2loint(v));
 }
@@ -408,7 +411,8 @@ __device__ __forceinline__ void plain_fma(cplx &s, const cplx &u, const cplx &v,
 // sum over two lanes): a row at a time with the columns over the lanes and a column with the rows over the lanes, which
 // leave terms with a zero out (such operands are mostly sparse; not with an Inf or a NaN among them), and a list of
 // elements, each over as many lanes as there are for it.  (One element of the list after another, its terms over the whole
-// warp, waited for memory: one in 400 elements took a product at nb = 64 from 371 to 920 us, now to 650.)
+// warp, waited for memory: one in 400 elements took a product at nb = 64 from 371 to 920 us, now to 620.  Columns four at a time,
+// all their terms looked at, took 137 us per mode product of the 4 x 4 cluster, now 79.)
 __device__ __noinline__ void plain_elements(const TcGemm &p, uint32_t mask, bool finite, int xt, int yt, int row0, int y0, int k0,
                                             int k1, uint16_t *list, long long *hi) {
   const int lane = threadIdx.x & 31, K = k1 - k0;
@@ -480,38 +484,45 @@ __device__ __noinline__ void plain_elements(const TcGemm &p, uint32_t mask, bool
       }
     }
   } else {
-    const cplx *a = row(row0 + lane);
-#pragma unroll 1
-    for (int g = 0; g < kMaxGroups; ++g) {
-      bool col[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) col[j] = cols >> (4 * g + j) & 1u;
-      if (!(cols >> (4 * g) & 15u)) continue;
-      const int yg = 4 * kPerQuarter * g;
-      const cplx *b = Y.p + row_offset(Y, p.y_begin + y0 + yg);
-      const bool mine = mask >> (4 * g) & 15u;
-      cplx s[4] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
-      constexpr int kAhead = 4;                                    // rows' terms loaded ahead
-#pragma unroll 1
-      for (int kb = k0; kb < k1; kb += kAhead) {
+    const cplx *a = row(row0 + lane), *b = Y.p + row_offset(Y, p.y_begin + y0);
+    uint32_t rest = cols;
+    int c = __ffs((int)rest) - 1, kb = k0;
+    auto column = [&](int i) { return 4 * kPerQuarter * (i >> 2) + (i & 3); };
+    auto load = [&]() { return kb + lane < k1 ? b[column(c) * Y.sx + (kb + lane) * Y.sk] : cplx{0.0, 0.0}; };
+    cplx next = load(), s = {0.0, 0.0};
+    while (c >= 0) {
+      const cplx v = next;
+      const int c_now = c, kb_now = kb;
+      kb += 32;
+      if (kb >= k1) {                                              // the next column's terms are loaded ahead
+        kb = k0;
+        rest &= rest - 1;
+        c = __ffs((int)rest) - 1;
+      }
+      if (c >= 0) next = load();
+      const bool mine = mask >> c_now & 1u;
+      uint32_t nz = __ballot_sync(0xffffffffu, kb_now + lane < k1 && !(finite && is_zero(v)));
+      while (nz) {
+        constexpr int kAhead = 4;                                  // rows' terms on their way
+        int q[kAhead];
         cplx u[kAhead];
 #pragma unroll
-        for (int q = 0; q < kAhead; ++q) u[q] = kb + q < k1 ? a[(kb + q) * X.sk] : cplx{0.0, 0.0};
+        for (int t = 0; t < kAhead; ++t) {
+          q[t] = __ffs((int)nz) - 1;
+          nz &= nz - 1;
+          u[t] = (mine && q[t] >= 0) ? a[(kb_now + q[t]) * X.sk] : cplx{0.0, 0.0};
+        }
 #pragma unroll
-        for (int q = 0; q < kAhead; ++q) {
-          if (kb + q >= k1 || (finite && __all_sync(0xffffffffu, !mine || is_zero(u[q])))) continue;
-          const cplx *bk = b + (kb + q) * Y.sk;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if (!col[j]) continue;
-            const cplx v = bk[j * Y.sx];
-            if (!(finite && is_zero(v))) plain_fma(s[j], u[q], v, fx, fy);
-          }
+        for (int t = 0; t < kAhead; ++t) {
+          if (q[t] < 0) continue;
+          const cplx vq = {__shfl_sync(0xffffffffu, v.x, q[t]), __shfl_sync(0xffffffffu, v.y, q[t])};
+          if (mine && !(finite && is_zero(u[t]))) plain_fma(s, u[t], vq, fx, fy);
         }
       }
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (mask >> (4 * g + j) & 1u) put(yg + j, lane, s[j]);
+      if (kb == k0) {
+        if (mine) put(column(c_now), lane, s);
+        s = {0.0, 0.0};
+      }
     }
   }
   __syncwarp();
@@ -879,8 +890,9 @@ __global__ void __launch_bounds__(kThreads, 1) fp64_tc_gemm_kernel(const __grid_
 // Sums the units of a long contraction in a fixed order and combines the four real products:
 // C[i][j] = alpha ((re re - im im) + i (re im + im re)) + beta C.  One CTA per output element, which also adds the
 // segments that the digits do not give, by FP64 multiply-adds (bits of rows 2 i and 2 i + 1 for column j).  Here the whole chip
-// shares them: taken in the GEMM they kept one SM busy for 540 us with the sparse cotangents of the 4 x 4 cluster (202 us
-// with one warp per element).  The next kernel may start once these are done: its CTAs would take the L1 from their loads.
+// shares them: taken in the GEMM they kept one SM busy for 540 us with the sparse cotangents of the 4 x 4 cluster; 202 us here
+// with one warp per element, 141 with a CTA, 106 with terms of zeros left out.  The next kernel may start once these are done: its
+// CTAs would take the L1 from their loads.
 constexpr int kRedThreads = 128;
 __global__ void __launch_bounds__(kRedThreads) fp64_tc_reduce_kernel(const TcGemm p) {
   __shared__ double sx[kRedThreads / 32], sy[kRedThreads / 32];
@@ -914,6 +926,7 @@ __global__ void __launch_bounds__(kRedThreads) fp64_tc_reduce_kernel(const TcGem
 #pragma unroll 8
         for (int k = (s0 + s) * len + lane; k < k1; k += 32) {
           const cplx u = a[k_offset(p.X, k)], v = b[k_offset(p.Y, k)];
+          if ((is_zero(u) && is_finite(v)) || (is_zero(v) && is_finite(u))) continue;
           const double ui = flip(u.y, fx), vi = flip(v.y, fy);
           if (r) { xs = fma(u.x, v.x, xs); ys = fma(u.x, vi, ys); }
           if (t) { xs = fma(-ui, vi, xs); ys = fma(ui, v.x, ys); }
